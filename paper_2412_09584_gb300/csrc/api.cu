@@ -450,9 +450,10 @@ BoundArgs make_bound_args(bab_ctx *c, const float *x0, const float *goal, int H,
     return a;
 }
 
-// IBP into the scratch (or the caller's arrays); fills the interval fields of `a`.
+// IBP into the scratch (or the caller's arrays); fills the interval fields of `a`.  with_S: the margin helpers are
+// wanted too (a bound follows).
 int run_ibp(bab_ctx *c, BoundArgs &a, Carver &cv, float *pre_lo, float *pre_hi, float *x_lo, float *x_hi,
-            float *lb_ibp, cudaStream_t st)
+            float *lb_ibp, cudaStream_t st, bool with_S = true)
 {
     const NetDesc &N = c->net;
     size_t nh = (size_t)a.n * a.H * N.sumh, nx = (size_t)a.n * (a.H + 1) * N.s;
@@ -464,6 +465,7 @@ int run_ibp(bab_ctx *c, BoundArgs &a, Carver &cv, float *pre_lo, float *pre_hi, 
     a.lb_ibp = lb_ibp;
     const bool tc = c->interval_precision != BAB_PREC_FP32 && a.batch.P <= 1 && a.cost.kind == 0;
     const bool tf = c->interval_precision == BAB_PREC_TF32X3;
+    if (!tc && !with_S) a.S = nullptr;
     a.ibp_img = tf ? c->d_ibp_tf : c->d_ibp;
     cudaError_t e = !tc ? launch_ibp(a, c->num_sms, st)
                         : (tf ? launch_ibp_tc_tf32(a, c->num_sms, st) : launch_ibp_tc(a, c->num_sms, st));
@@ -1126,7 +1128,7 @@ int bab_bound_ibp(bab_ctx *c, const float *x0, const float *goal, int H, float r
     if (rc) return rc;
     BoundArgs a = make_bound_args(c, x0, goal, H, rho, lo, hi, n, d_n);
     Carver cv{reinterpret_cast<char *>(c->scratch)};
-    return run_ibp(c, a, cv, pre_lo, pre_hi, x_lo, x_hi, lb_ibp, (cudaStream_t)stream);
+    return run_ibp(c, a, cv, pre_lo, pre_hi, x_lo, x_hi, lb_ibp, (cudaStream_t)stream, false);
 }
 
 // The CROWN launch of a bound precision (the tensor-core ones need a.mu set by the caller).
@@ -1226,7 +1228,7 @@ int bab_alpha_init(bab_ctx *c, const float *x0, const float *goal, int H, float 
     cudaStream_t st = (cudaStream_t)stream;
     BoundArgs a = make_bound_args(c, x0, goal, H, rho, lo, hi, n, d_n);
     Carver cv{reinterpret_cast<char *>(c->scratch)};
-    rc = run_ibp(c, a, cv, nullptr, nullptr, nullptr, nullptr, nullptr, st);
+    rc = run_ibp(c, a, cv, nullptr, nullptr, nullptr, nullptr, nullptr, st, false);
     if (rc) return rc;
     a.alpha = alpha;
     cudaError_t e = launch_alpha_init(a, st);

@@ -17,10 +17,10 @@
 //                concretizing point u*, giving dLB/dalpha = A_j z~_j.
 //   k_adam       projected Adam ascent on alpha.
 //
-// A CTA owns RB boxes (rows); the network image lives in shared memory when
-// it fits (otherwise it is read through L2); the rows move through the layers
-// as register-blocked FP32 products (dense_rows), and each per-row reduction
-// is one warp with shuffles.
+// In k_crown and k_alpha_fwd a CTA owns RB boxes (rows); the network image lives
+// in shared memory when it fits (otherwise it is read through L2); the rows move
+// through the layers as register-blocked FP32 products (dense_rows), and each
+// per-row reduction is one warp with shuffles.  k_ibp has its own tiles.
 #include <cmath>
 
 #include "bab_internal.cuh"
@@ -58,152 +58,447 @@ __device__ __forceinline__ float half2f(unsigned long long v, int e)
     return __uint_as_float((uint32_t)(e ? v >> 32 : v));
 }
 
+constexpr int kIbpNT = 512;  // threads of k_ibp
+constexpr int kIbpGroups = 4; // independent row groups of a CTA (weights in shared memory)
+
 // Where a layer's outputs go: the interval bounds and S of step t to global memory (rows < nlive, columns < dl;
-// no pre-activation bounds for the output layer), and the next layer's input (ReLU of the bounds, or the bounds
-// of the output layer themselves) to the tile's shared-memory buffers.
+// no pre-activation bounds for the output layer, no S where the caller takes none), and the next layer's input
+// (ReLU of the bounds, or the bounds of the output layer themselves) to the tile's shared-memory buffers.
 struct IbpSink {
-    float *pre_lo, *pre_hi, *S;  // at (box0 * H + t) of the [n][H][...] arrays
+    float *pre_lo, *pre_hi, *S;  // at (box0 * H + t) of the [n][H][...] arrays, the layer's first column
     size_t rstride_h, rstride_s; // per row: H * sumh, H * (sumh + s)
-    int hoff, soff, dl, nrows;
-    bool hidden;
+    uint32_t *mask;              // [rows][2][4], zero before: bit (c / 4) % 32 of word [c / 128][c % 4] set where column
+                                 // c's lower end is not 0 (the next layer's input)
+    int dl, nrows;
+    bool full;                   // every warp that stores has all 32 lanes storing
+    bool hidden, vec_h, vec_s;   // vec: four columns from a multiple of 4 on are 16-byte aligned
 };
 
-// One layer of interval bounds for RB rows, TR rows x TN columns per thread: per output the three directed-
-// rounding sums (lower, upper, and S = sum_k |W_jk| max|a_k|) over the inputs in order from the bias, the
-// endpoint of each input picked by the sign of the weight; two adjacent columns run as one paired FMA.
+// A layer's outputs of one thread: TR rows x TN columns, lower and upper sums and S, written to the sink and to the
+// next layer's input.  Returns whether a value is not finite.
 template <int TR, int TN>
-__device__ __forceinline__ void ibp_dense(const float *__restrict__ alo, const float *__restrict__ ahi, int ld,
-                                          const float *__restrict__ Wt, const float *__restrict__ bias, int Kp, int Np,
-                                          float *__restrict__ zlo, float *__restrict__ zhi, const IbpSink &o)
+__device__ __forceinline__ bool ibp_store(const float (&l)[TR][TN], const float (&h)[TR][TN], const float (&S)[TR][TN],
+                                          int r0, int c0, int Np, int ld, float *__restrict__ zlo,
+                                          float *__restrict__ zhi, const IbpSink &o)
 {
-    static_assert(TN % 2 == 0, "column pairs");
+    bool bad = false;
+    // the lanes of a warp hold whole rows' segments of 4 seg columns (seg = 32, 16, .. 1): masks by ballot
+    const int seg = Np / 4;
+    const bool by_ballot = TN == 4 && (seg % 32 == 0 || (seg <= 16 && (seg & (seg - 1)) == 0 && o.full));
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+        const int r = r0 + i;
+        const bool live = r < o.nrows;
+        const bool whole = TN == 4 && c0 + 4 <= o.dl;
+        if (live && o.S) {
+            float *p = o.S + r * o.rstride_s + c0;
+            if (whole && o.vec_s)
+                *reinterpret_cast<float4 *>(p) = make_float4(S[i][0], S[i][1 % TN], S[i][2 % TN], S[i][3 % TN]);
+            else
+#pragma unroll
+                for (int j = 0; j < TN; ++j)
+                    if (c0 + j < o.dl) p[j] = S[i][j];
+        }
+        if (live && o.hidden) {
+            float *pl = o.pre_lo + r * o.rstride_h + c0, *ph = o.pre_hi + r * o.rstride_h + c0;
+            if (whole && o.vec_h) {
+                *reinterpret_cast<float4 *>(pl) = make_float4(l[i][0], l[i][1 % TN], l[i][2 % TN], l[i][3 % TN]);
+                *reinterpret_cast<float4 *>(ph) = make_float4(h[i][0], h[i][1 % TN], h[i][2 % TN], h[i][3 % TN]);
+            } else
+#pragma unroll
+                for (int j = 0; j < TN; ++j)
+                    if (c0 + j < o.dl) {
+                        pl[j] = l[i][j];
+                        ph[j] = h[i][j];
+                    }
+        }
+        float vl[TN], vh[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const bool relu = o.hidden && c0 + j < o.dl;
+            vl[j] = relu ? fmaxf(l[i][j], 0.f) : l[i][j];
+            vh[j] = relu ? fmaxf(h[i][j], 0.f) : h[i][j];
+            bad |= !(fabsf(l[i][j]) < INFINITY) || !(fabsf(h[i][j]) < INFINITY);
+        }
+        if (o.hidden) {
+            uint32_t *mk = o.mask + 8 * r + 4 * (c0 >> 7);
+            if (by_ballot) {
+                uint32_t m[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) m[j] = __ballot_sync(0xFFFFFFFFu, vl[j % TN] != 0.f);
+                if (seg < 32) {
+                    const int first = (threadIdx.x & 31) & ~(seg - 1);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) m[j] = (m[j] >> first) & ((1u << seg) - 1u);
+                }
+                if ((threadIdx.x & 31 & (seg - 1)) == 0) *reinterpret_cast<uint4 *>(mk) = make_uint4(m[0], m[1], m[2], m[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < TN; ++j)
+                    if (vl[j] != 0.f && c0 + j < Np) atomicOr(mk + ((c0 + j) & 3), 1u << ((c0 >> 2) & 31));
+            }
+        }
+        if (TN == 4) {
+            // (Np is a multiple of 4)
+            *reinterpret_cast<float4 *>(zlo + r * ld + c0) = make_float4(vl[0], vl[1 % TN], vl[2 % TN], vl[3 % TN]);
+            *reinterpret_cast<float4 *>(zhi + r * ld + c0) = make_float4(vh[0], vh[1 % TN], vh[2 % TN], vh[3 % TN]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (c0 + j < Np) {
+                    zlo[r * ld + c0 + j] = vl[j];
+                    zhi[r * ld + c0 + j] = vh[j];
+                }
+        }
+    }
+    return bad;
+}
+
+// One input of a thread's TR x TN outputs, two columns per FMA pair:
+//   lower += w+ a_lo + w- a_hi (rounded down),  upper += w+ a_hi + w- a_lo (rounded up),
+//   V     += |w| max|a| for the first layer, |w| a_lo for the later ones (rounded up),
+// w+ = max(w, 0), w- = min(w, 0).  One of the two products of a weight is an exact zero, so each sum has the bits of
+// the one that takes the endpoint by the sign of the weight.  LOWER: some row's a_lo is not 0; without it only the
+// products of the upper end are left.
+template <int TR, int TN, bool FIRST, bool LOWER>
+__device__ __forceinline__ void ibp_input(const float *__restrict__ wr, const float4 (&l4)[TR], const float4 (&h4)[TR], int kk, unsigned long long (&l2)[TR][TN / 2],
+                                          unsigned long long (&h2)[TR][TN / 2], unsigned long long (&v2)[TR][TN / 2])
+{
     constexpr int TP = TN / 2;
-    const int ngc = (Np + TN - 1) / TN;
-    const int items = (RB / TR) * ngc;
-    for (int it = threadIdx.x; it < items; it += NT) {
-        const int cg = it % ngc, rg = it / ngc;
-        const int c0 = cg * TN, r0 = rg * TR;
-        unsigned long long accl[TR][TP], acch[TR][TP], accs[TR][TP];
+    float w[TN];
+    if (TN == 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(wr);
+        w[0] = q.x;
+        w[1] = q.y;
+        w[2 % TN] = q.z;
+        w[3 % TN] = q.w;
+    } else {
+        const float2 q = *reinterpret_cast<const float2 *>(wr);
+        w[0] = q.x;
+        w[1] = q.y;
+    }
+    unsigned long long wp[TP], wn[TP], wa[TP];
 #pragma unroll
-        for (int jp = 0; jp < TP; ++jp) {
-            const int j = c0 + 2 * jp;
-            const unsigned long long b2 = pack2f(j < Np ? bias[j] : 0.f, j + 1 < Np ? bias[j + 1] : 0.f);
+    for (int j = 0; j < TP; ++j) {
+        wp[j] = pack2f(fmaxf(w[2 * j], 0.f), fmaxf(w[2 * j + 1], 0.f));
+        wn[j] = pack2f(fminf(w[2 * j], 0.f), fminf(w[2 * j + 1], 0.f));
+        wa[j] = pack2f(fabsf(w[2 * j]), fabsf(w[2 * j + 1]));
+    }
 #pragma unroll
-            for (int i = 0; i < TR; ++i) {
-                accl[i][jp] = acch[i][jp] = b2;
-                accs[i][jp] = 0ull;
+    for (int i = 0; i < TR; ++i) {
+        const float ah = kk == 0 ? h4[i].x : kk == 1 ? h4[i].y : kk == 2 ? h4[i].z : h4[i].w;
+        const unsigned long long ah2 = pack2f(ah, ah);
+        if (!LOWER) {
+#pragma unroll
+            for (int j = 0; j < TP; ++j) {
+                l2[i][j] = ffma2_rd(wn[j], ah2, l2[i][j]);
+                h2[i][j] = ffma2_ru(wp[j], ah2, h2[i][j]);
             }
-        }
-        const bool full = (c0 + TN <= Np);
-        for (int k = 0; k < Kp; k += 4) {
-            float4 l4[TR], h4[TR];
+        } else {
+            const float al = kk == 0 ? l4[i].x : kk == 1 ? l4[i].y : kk == 2 ? l4[i].z : l4[i].w;
+            const float am = FIRST ? fmaxf(fabsf(al), fabsf(ah)) : al;
+            const unsigned long long al2 = pack2f(al, al), am2 = pack2f(am, am);
 #pragma unroll
-            for (int i = 0; i < TR; ++i) {
-                l4[i] = *reinterpret_cast<const float4 *>(alo + (r0 + i) * ld + k);
-                h4[i] = *reinterpret_cast<const float4 *>(ahi + (r0 + i) * ld + k);
+            for (int j = 0; j < TP; ++j) {
+                l2[i][j] = ffma2_rd(wn[j], ah2, ffma2_rd(wp[j], al2, l2[i][j]));
+                h2[i][j] = ffma2_ru(wn[j], al2, ffma2_ru(wp[j], ah2, h2[i][j]));
+                v2[i][j] = ffma2_ru(wa[j], am2, v2[i][j]);
             }
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                float w[TN];
-                const float *wr = Wt + (size_t)(k + kk) * Np + c0;
-                if (full && TN % 4 == 0) {
-                    // whole 16-byte groups (Np and c0 are multiples of 4)
-#pragma unroll
-                    for (int j = 0; j < TN; j += 4) {
-                        const float4 q = *reinterpret_cast<const float4 *>(wr + j);
-                        w[j] = q.x;
-                        w[j + 1] = q.y;
-                        w[j + 2] = q.z;
-                        w[j + 3] = q.w;
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < TN; ++j) w[j] = (c0 + j < Np) ? wr[j] : 0.f;
-                }
-                bool pos[TN];
-                unsigned long long w2[TP], a2[TP];
-#pragma unroll
-                for (int jp = 0; jp < TP; ++jp) {
-                    pos[2 * jp] = w[2 * jp] >= 0.f;
-                    pos[2 * jp + 1] = w[2 * jp + 1] >= 0.f;
-                    w2[jp] = pack2f(w[2 * jp], w[2 * jp + 1]);
-                    a2[jp] = pack2f(fabsf(w[2 * jp]), fabsf(w[2 * jp + 1]));
-                }
-#pragma unroll
-                for (int i = 0; i < TR; ++i) {
-                    const float al = kk == 0 ? l4[i].x : kk == 1 ? l4[i].y : kk == 2 ? l4[i].z : l4[i].w;
-                    const float ah = kk == 0 ? h4[i].x : kk == 1 ? h4[i].y : kk == 2 ? h4[i].z : h4[i].w;
-                    const float am = fmaxf(fabsf(al), fabsf(ah));
-                    const unsigned long long m2 = pack2f(am, am);
-#pragma unroll
-                    for (int jp = 0; jp < TP; ++jp) {
-                        const bool p0 = pos[2 * jp], p1 = pos[2 * jp + 1];
-                        accl[i][jp] = ffma2_rd(w2[jp], pack2f(p0 ? al : ah, p1 ? al : ah), accl[i][jp]);
-                        acch[i][jp] = ffma2_ru(w2[jp], pack2f(p0 ? ah : al, p1 ? ah : al), acch[i][jp]);
-                        accs[i][jp] = ffma2_ru(a2[jp], m2, accs[i][jp]);
-                    }
-                }
-            }
-        }
-        // write the rows' bounds and S, and the next layer's input
-#pragma unroll
-        for (int i = 0; i < TR; ++i) {
-            const int r = r0 + i;
-            const bool live = r < o.nrows;
-#pragma unroll
-            for (int jp = 0; jp < TP; ++jp)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int j = c0 + 2 * jp + e;
-                    if (j >= Np) continue;
-                    const float zl = half2f(accl[i][jp], e), zh = half2f(acch[i][jp], e);
-                    if (live && j < o.dl) {
-                        o.S[r * o.rstride_s + o.soff + j] = half2f(accs[i][jp], e);
-                        if (o.hidden) {
-                            o.pre_lo[r * o.rstride_h + o.hoff + j] = zl;
-                            o.pre_hi[r * o.rstride_h + o.hoff + j] = zh;
-                        }
-                    }
-                    const bool relu = o.hidden && j < o.dl;
-                    zlo[r * ld + j] = relu ? fmaxf(zl, 0.f) : zl;
-                    zhi[r * ld + j] = relu ? fmaxf(zh, 0.f) : zh;
-                }
         }
     }
 }
 
-template <bool WSMEM>
-__global__ void __launch_bounds__(NT) k_ibp(BoundArgs a)
+// The sums of one thread's TR x TN outputs over the inputs k0 <= k < k1 (multiples of 4, within one group of 128),
+// in input order.  mask: bit (k / 4) % 32 of word k % 4 says whether some row's lower end of input k is not 0.  After
+// a ReLU nearly all are 0 (90-100% on the pushing and object-manipulation networks), so most of a layer is two FMAs a
+// weight and row: 3.2 cycles per scheduler (pairs; 4.0 with scalar FMAs) against 6.9 with all five, and 7.2-8 with
+// the endpoints selected instead (the selects run on the half-wide ALU pipe).
+template <int TR, int TN, bool FIRST, bool FINE>
+__device__ __forceinline__ void ibp_span(const float *__restrict__ alo, const float *__restrict__ ahi, int ld,
+                                         const float *__restrict__ W, int ldw, int k0, int k1, int r0,
+                                         const uint32_t (&mask)[4], unsigned long long (&l2)[TR][TN / 2],
+                                         unsigned long long (&h2)[TR][TN / 2], unsigned long long (&v2)[TR][TN / 2])
 {
+    const uint32_t some = mask[0] | mask[1] | mask[2] | mask[3];
+#pragma unroll 1
+    for (int k = k0; k < k1; k += 4) {
+        float4 l4[TR], h4[TR];
+        const int b = (k >> 2) & 31;
+#pragma unroll
+        for (int i = 0; i < TR; ++i) h4[i] = *reinterpret_cast<const float4 *>(ahi + (r0 + i) * ld + k);
+        const float *wq = W + (size_t)(k - k0) * ldw;
+        if (!FIRST && !((some >> b) & 1u)) {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) ibp_input<TR, TN, FIRST, false>(wq + kk * ldw, l4, h4, kk, l2, h2, v2);
+        } else {
+#pragma unroll
+            for (int i = 0; i < TR; ++i) l4[i] = *reinterpret_cast<const float4 *>(alo + (r0 + i) * ld + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+                if (FIRST || !FINE || ((mask[kk] >> b) & 1u))
+                    ibp_input<TR, TN, FIRST, true>(wq + kk * ldw, l4, h4, kk, l2, h2, v2);
+                else
+                    ibp_input<TR, TN, FIRST, false>(wq + kk * ldw, l4, h4, kk, l2, h2, v2);
+        }
+    }
+}
+
+// The masks of inputs k .. k + 127 (k a multiple of 128) over rows r0 .. r0 + TR - 1.
+template <int TR>
+__device__ __forceinline__ void ibp_mask(const uint32_t *__restrict__ mask, int r0, int k, uint32_t (&m)[4])
+{
+    m[0] = m[1] = m[2] = m[3] = 0u;
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(mask + 8 * (r0 + i) + 4 * (k >> 7));
+        m[0] |= q.x;
+        m[1] |= q.y;
+        m[2] |= q.z;
+        m[3] |= q.w;
+    }
+}
+
+// The sums turned into a thread's bounds and S.
+template <int TR, int TN, bool FIRST>
+__device__ __forceinline__ void ibp_unpack(const float *__restrict__ bias, unsigned long long (&l2)[TR][TN / 2],
+                                           unsigned long long (&h2)[TR][TN / 2], unsigned long long (&v2)[TR][TN / 2],
+                                           float (&l)[TR][TN], float (&h)[TR][TN], float (&S)[TR][TN])
+{
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            l[i][j] = half2f(l2[i][j / 2], j & 1);
+            h[i][j] = half2f(h2[i][j / 2], j & 1);
+            const float v = half2f(v2[i][j / 2], j & 1);
+            S[i][j] = FIRST ? v : ibp_s(l[i][j], h[i][j], bias[j], v);
+        }
+}
+
+// One layer with the weights in shared memory, TR rows x TN columns per thread and pass.
+template <int TR, int TN, bool FIRST>
+__device__ __forceinline__ bool ibp_dense(int tid, const float *__restrict__ alo, const float *__restrict__ ahi,
+                                          const uint32_t *__restrict__ mask, int ld, int rb,
+                                          const float *__restrict__ Wt, const float *__restrict__ bias, int Kp, int Np,
+                                          float *__restrict__ zlo, float *__restrict__ zhi, const IbpSink &o)
+{
+    const int ngc = Np / TN;  // (Np is a multiple of 4)
+    const int items = (rb / TR) * ngc;
+    bool bad = false;
+    for (int it = tid; it < items; it += kIbpNT / kIbpGroups) {
+        const int rg = it / ngc, c0 = (it - rg * ngc) * TN, r0 = rg * TR;
+        constexpr int TP = TN / 2;
+        unsigned long long l2[TR][TP], h2[TR][TP], v2[TR][TP];
+#pragma unroll
+        for (int j = 0; j < TP; ++j)
+#pragma unroll
+            for (int i = 0; i < TR; ++i) {
+                l2[i][j] = h2[i][j] = pack2f(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]);
+                v2[i][j] = 0ull;
+            }
+        for (int k = 0; k < Kp; k += 128) {
+            uint32_t m[4];
+            ibp_mask<TR>(mask, r0, k, m);
+            ibp_span<TR, TN, FIRST, true>(alo, ahi, ld, Wt + (size_t)k * Np + c0, Np, k, min(Kp, k + 128), r0, m, l2, h2, v2);
+        }
+        float l[TR][TN], h[TR][TN], S[TR][TN];
+        ibp_unpack<TR, TN, FIRST>(bias + c0, l2, h2, v2, l, h, S);
+        bad |= ibp_store<TR, TN>(l, h, S, r0, c0, Np, ld, zlo, zhi, o);
+    }
+    return bad;
+}
+
+// A later layer with few outputs (the network's last): one output per thread and pass, two chains of Kp FMAs whose
+// latency is what the layer takes, so each input's endpoint is selected by the sign of the weight off the chain.
+__device__ __forceinline__ bool ibp_dense_narrow(int tid, int nt, const float *__restrict__ alo,
+                                                 const float *__restrict__ ahi, int ld, int rb,
+                                                 const float *__restrict__ Wt, const float *__restrict__ bias, int Kp,
+                                                 int Np, float *__restrict__ zlo, float *__restrict__ zhi, const IbpSink &o)
+{
+    bool bad = false;
+    for (int it = tid; it < rb * Np; it += nt) {
+        const int r = it / Np, c = it - r * Np;
+        const float *al = alo + r * ld, *ah = ahi + r * ld, *w = Wt + c;
+        float l[1][1], h[1][1], S[1][1];
+        l[0][0] = h[0][0] = bias[c];
+        S[0][0] = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < Kp; k += 4) {
+            const float4 h4 = *reinterpret_cast<const float4 *>(ah + k), l4 = *reinterpret_cast<const float4 *>(al + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const float wk = w[(size_t)(k + kk) * Np];
+                const float hi = kk == 0 ? h4.x : kk == 1 ? h4.y : kk == 2 ? h4.z : h4.w;
+                const float lo = kk == 0 ? l4.x : kk == 1 ? l4.y : kk == 2 ? l4.z : l4.w;
+                const bool pos = wk >= 0.f;
+                l[0][0] = __fmaf_rd(wk, pos ? lo : hi, l[0][0]);
+                h[0][0] = __fmaf_ru(wk, pos ? hi : lo, h[0][0]);
+                S[0][0] = __fmaf_ru(fabsf(wk), lo, S[0][0]);
+            }
+        }
+        S[0][0] = ibp_s(l[0][0], h[0][0], bias[c], S[0][0]);
+        bad |= ibp_store<1, 1>(l, h, S, r, c, Np, ld, zlo, zhi, o);
+    }
+    return bad;
+}
+
+// The same layer where an input (or a weight) is not finite: 0 x inf must not reach the sums, so each input's
+// endpoint is picked by the sign of the weight (the same bits for the rows that are finite).  One output per thread
+// and pass.
+__device__ __noinline__ bool ibp_dense_any(int tid, int nt, bool first, const float *__restrict__ alo,
+                                           const float *__restrict__ ahi, int ld, int rb,
+                                           const float *__restrict__ Wt, const float *__restrict__ bias, int Kp,
+                                           int Np, float *__restrict__ zlo, float *__restrict__ zhi, const IbpSink &o)
+{
+    bool bad = false;
+    for (int it = tid; it < rb * Np; it += nt) {
+        const int r = it / Np, c = it - r * Np;
+        float l[1][1], h[1][1], S[1][1];
+        l[0][0] = h[0][0] = bias[c];
+        S[0][0] = 0.f;
+        for (int k = 0; k < Kp; ++k) {
+            const float w = Wt[(size_t)k * Np + c], al = alo[r * ld + k], ah = ahi[r * ld + k];
+            const bool pos = w >= 0.f;
+            l[0][0] = __fmaf_rd(w, pos ? al : ah, l[0][0]);
+            h[0][0] = __fmaf_ru(w, pos ? ah : al, h[0][0]);
+            S[0][0] = __fmaf_ru(fabsf(w), first ? fmaxf(fabsf(al), fabsf(ah)) : al, S[0][0]);
+        }
+        if (!first) S[0][0] = ibp_s(l[0][0], h[0][0], bias[c], S[0][0]);
+        bad |= ibp_store<1, 1>(l, h, S, r, c, Np, ld, zlo, zhi, o);
+    }
+    return bad;
+}
+
+// Weights beyond shared memory: the layer's forward image goes through a ring of kIbpStages stages of kIbpSpan
+// inputs each, copied asynchronously while the stage before is multiplied; every thread owns the same TR x TN
+// outputs throughout (kIbpStreamRows / TR x Np / TN of them, at most kIbpNT).
+constexpr int kIbpSpan = 32, kIbpStages = 2, kIbpStreamRows = 32;
+
+template <int TR, int TN, bool FIRST>
+__device__ __forceinline__ bool ibp_dense_stream(const float *__restrict__ alo, const float *__restrict__ ahi,
+                                                 const uint32_t *__restrict__ mask, int ld,
+                                                 float *__restrict__ ring, const float *__restrict__ Wt,
+                                                 const float *__restrict__ bias, int Kp, int Np,
+                                                 float *__restrict__ zlo, float *__restrict__ zhi, const IbpSink &o)
+{
+    const int ngc = Np / TN;
+    const int rg = threadIdx.x / ngc, c0 = (threadIdx.x - rg * ngc) * TN, r0 = rg * TR;
+    const bool mine = rg < kIbpStreamRows / TR;
+    const int nspan = (Kp + kIbpSpan - 1) / kIbpSpan;
+    auto fetch = [&](int q) {
+        if (q < nspan) {
+            const int k0 = q * kIbpSpan, n4 = min(kIbpSpan, Kp - k0) * Np / 4;
+            const float4 *src = reinterpret_cast<const float4 *>(Wt + (size_t)k0 * Np);
+            const uint32_t dst =
+                (uint32_t)__cvta_generic_to_shared(ring + (size_t)(q % kIbpStages) * kIbpSpan * kMaxWidth);
+            for (int i = threadIdx.x; i < n4; i += kIbpNT)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + i) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    constexpr int TP = TN / 2;
+    unsigned long long l2[TR][TP], h2[TR][TP], v2[TR][TP];
+#pragma unroll
+    for (int j = 0; j < TP; ++j) {
+        const unsigned long long b2 = mine ? pack2f(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]) : 0ull;
+#pragma unroll
+        for (int i = 0; i < TR; ++i) {
+            l2[i][j] = h2[i][j] = b2;
+            v2[i][j] = 0ull;
+        }
+    }
+    uint32_t m[4] = {0u, 0u, 0u, 0u};
+    fetch(0);
+    for (int q = 0; q < nspan; ++q) {
+        fetch(q + 1);  // its stage was last read before the barrier that closed the span before
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        if (mine) {
+            const int k0 = q * kIbpSpan;
+            if (k0 % 128 == 0) ibp_mask<TR>(mask, r0, k0, m);
+            ibp_span<TR, TN, FIRST, false>(alo, ahi, ld, ring + (size_t)(q % kIbpStages) * kIbpSpan * kMaxWidth + c0, Np, k0,
+                                    min(Kp, k0 + kIbpSpan), r0, m, l2, h2, v2);
+        }
+        __syncthreads();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (!mine) return false;
+    float l[TR][TN], h[TR][TN], S[TR][TN];
+    ibp_unpack<TR, TN, FIRST>(bias + c0, l2, h2, v2, l, h, S);
+    return ibp_store<TR, TN>(l, h, S, r0, c0, Np, ld, zlo, zhi, o);
+}
+
+// Leading dimension of the tile's activation rows: 4 mod 8 floats, so that the 16-byte loads of different rows by
+// one warp fall on different banks.
+__host__ __device__ constexpr int ibp_ld(int maxw_p) { return ((maxw_p + 7) & ~7) + 4; }
+
+// Shared-memory floats of one group of rb rows (a multiple of 4).
+__host__ __device__ inline size_t ibp_rest_floats(const NetDesc &N, int rb)
+{
+    return (4 * (size_t)rb * ibp_ld(N.maxw_p) + 28 * (size_t)rb + 2 * (size_t)rb * pad4(N.s) + rb + 3) & ~size_t(3);
+}
+
+// Barrier of one row group (threads nt, barrier id g + 1), and whether any of its threads passed a nonzero v.
+__device__ __forceinline__ int group_or(int g, int nt, int v)
+{
+    int r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, %3, p;\n\t"
+                 "selp.s32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r)
+                 : "r"(v), "r"(g + 1), "r"(nt)
+                 : "memory");
+    return r;
+}
+
+// Interval bounds of a tile of boxes.  The weights sit in shared memory and the CTA's warps form kIbpGroups groups of
+// rb boxes each that share them and run on their own (buffers, barriers): while one group waits at a layer's end or
+// walks the narrow output layer, the others multiply.  STREAM: the image does not fit; one group of rb =
+// kIbpStreamRows boxes.  tiles: two bits per layer, the tile of ibp_tile.  safe: some weight may not be finite.
+// What bounds it: issue slots and the latencies of a layer's ends (a step of the pushing network is four layers); the
+// FMAs of the upper ends alone take 3.2 (4 x 4 outputs a thread) to 4.2 cycles (2 x 4) per weight and row.  Measured,
+// all arrays written: pushing 3001 boxes 1079 -> 586 us; object manipulation, 16384 boxes, 51.4 -> 20.6 ms.
+template <bool STREAM>
+__global__ void __launch_bounds__(kIbpNT, 1) k_ibp(BoundArgs a, int rb, int tiles, int vec_h, int vec_s, int safe)
+{
+    constexpr int G = STREAM ? 1 : kIbpGroups, TG = kIbpNT / G;
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
     const NetDesc &N = a.net;
     const int s = N.s, k = N.k, L = N.L, d = a.d, H = a.H, sumh = N.sumh;
-    const int ld = N.maxw_p, s4 = pad4(s);
+    const int ld = ibp_ld(N.maxw_p), s4 = pad4(s);
+    const int nlive = live_count(a.n, a.d_n, a.row0);
+    if ((int)blockIdx.x * G * rb >= nlive) return;
+    // a group's first warps do its narrow layers: spread the groups' over the schedulers (warp id modulo 4)
+    const int grp = threadIdx.x / TG, tid = (threadIdx.x + 32 * grp) % TG;
+    const int box0 = ((int)blockIdx.x * G + grp) * rb;
     const float *img = a.fwd;
-    float *p = sm;
-    if (WSMEM) {
-        for (int i = threadIdx.x; i < N.img_floats / 4; i += NT) smem4[i] = reinterpret_cast<const float4 *>(a.fwd)[i];
+    float *p = sm, *ring = nullptr;
+    if (STREAM) {
+        ring = p;
+        p += (size_t)kIbpStages * kIbpSpan * kMaxWidth;
+    } else {
+        for (int i = threadIdx.x; i < N.img_floats / 4; i += kIbpNT)
+            smem4[i] = reinterpret_cast<const float4 *>(a.fwd)[i];
         img = sm;
         p += N.img_floats;
+        __syncthreads();
     }
-    float *blo[2], *bhi[2];
-    blo[0] = p; p += RB * ld;
-    bhi[0] = p; p += RB * ld;
-    blo[1] = p; p += RB * ld;
-    bhi[1] = p; p += RB * ld;
-    float *xl = p; p += RB * s4;
-    float *xu = p; p += RB * s4;
-    float *lbacc = p; p += RB;
-    float *pbx = p; p += 4 * RB;  // pusher position box per row (obstacle cost): lo x, lo y, hi x, hi y
-
-    const int nlive = live_count(a.n, a.d_n, a.row0);
-    const int box0 = blockIdx.x * RB;
     if (box0 >= nlive) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    p += (size_t)grp * ibp_rest_floats(N, rb);
+    // activation buffers (lower and upper ends of buffer i), masks [3][rb][2][4] (IbpSink::mask), and per row: the
+    // pusher position box of the obstacle cost (lo x, lo y, hi x, hi y), the state box, the bound so far
+    float *act = p;
+    auto buf_lo = [&](int i) { return act + 2 * i * rb * ld; };
+    auto buf_hi = [&](int i) { return act + (2 * i + 1) * rb * ld; };
+    uint32_t *masks = reinterpret_cast<uint32_t *>(act + 4 * rb * ld);
+    float *pbx = act + 4 * rb * ld + 24 * rb, *xl = pbx + 4 * rb, *xu = xl + rb * s4, *lbacc = xu + rb * s4;
+    int mcur = 0;
+
+    const int lane = tid & 31, warp = tid >> 5;
     const int Kp1 = pad4(s + k);
 
-    for (int i = threadIdx.x; i < RB * s; i += NT) {
+    for (int i = tid; i < 24 * rb; i += TG) masks[i] = 0u;
+    for (int i = tid; i < rb * s; i += TG) {
         const int r = i / s, c = i % s;
         xl[r * s4 + c] = a.x0[c];
         xu[r * s4 + c] = a.x0[c];
@@ -212,123 +507,177 @@ __global__ void __launch_bounds__(NT) k_ibp(BoundArgs a)
             a.x_hi[(size_t)(box0 + r) * (H + 1) * s + c] = a.x0[c];
         }
     }
-    for (int r = threadIdx.x; r < RB; r += NT) {
+    for (int r = tid; r < rb; r += TG) {
         lbacc[r] = 0.f;
         pbx[4 * r] = pbx[4 * r + 2] = a.cost.p0x;
         pbx[4 * r + 1] = pbx[4 * r + 3] = a.cost.p0y;
     }
-    __syncthreads();
+    group_or(grp, TG, 0);
 
-    for (int t = 0; t < H; ++t) {
-        for (int i = threadIdx.x; i < RB * Kp1; i += NT) {
-            const int r = i / Kp1, c = i % Kp1;
-            const int box = box0 + r;
-            float vl = 0.f, vh = 0.f;
-            if (c < s) {
-                vl = xl[r * s4 + c];
-                vh = xu[r * s4 + c];
-            } else if (c < s + k && box < nlive) {
-                vl = a.lo[(size_t)box * d + t * k + (c - s)];
-                vh = a.hi[(size_t)box * d + t * k + (c - s)];
+    // a warp's rows are warp and warp + TG / 32 (rb is at most twice that); where a row's inputs fit the lanes, each
+    // step's action bounds are loaded one step ahead
+    const bool ahead = !STREAM && Kp1 <= 32;
+    float ul[2] = {0.f, 0.f}, uh[2] = {0.f, 0.f};
+    auto load_u = [&](int t) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = warp + i * (TG / 32);
+            if (r < rb && box0 + r < nlive && t < H && lane >= s && lane < s + k) {
+                ul[i] = a.lo[(size_t)(box0 + r) * d + t * k + (lane - s)];
+                uh[i] = a.hi[(size_t)(box0 + r) * d + t * k + (lane - s)];
             }
-            blo[0][r * ld + c] = vl;
-            bhi[0][r * ld + c] = vh;
         }
-        if (a.cost.kind == 1)
-            for (int r = threadIdx.x; r < RB; r += NT)
-                if (box0 + r < nlive) {
-                    const float *ul = a.lo + (size_t)(box0 + r) * d + t * k, *uh = a.hi + (size_t)(box0 + r) * d + t * k;
+    };
+    if (ahead) load_u(0);
+    int cur = 0;
+    for (int t = 0; t <= H; ++t) {
+        // per row, one warp: x_t in [x_{t-1}] + [z_L] and the interval bound of its cost, then the next input row
+        // [x_t | u_t | 0] and the bound of rho ||u_t||^2
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = warp + i * (TG / 32);
+            if (r >= rb) break;
+            const int box = box0 + r;
+            const bool live = box < nlive;
+            float v = 0.f, vu = 0.f;
+            for (int c = lane; c < Kp1; c += 32) {
+                float nl = 0.f, nh = 0.f;
+                if (c < s) {
+                    nl = xl[r * s4 + c];
+                    nh = xu[r * s4 + c];
+                    if (t > 0) {
+                        nl = __fadd_rd(nl, buf_lo(cur)[r * ld + c]);
+                        nh = __fadd_ru(nh, buf_hi(cur)[r * ld + c]);
+                        xl[r * s4 + c] = nl;
+                        xu[r * s4 + c] = nh;
+                        if (live && a.x_lo) {
+                            a.x_lo[((size_t)box * (H + 1) + t) * s + c] = nl;
+                            a.x_hi[((size_t)box * (H + 1) + t) * s + c] = nh;
+                        }
+                        const float g = a.goal[c];
+                        if (a.cost.kind == 0) {
+                            v = __fadd_rd(v, sq_min_rd(__fsub_rd(nl, g), __fsub_ru(nh, g)));
+                        } else {
+                            // distance from g to the interval, rounded down, squared rounded down
+                            const float e = fmaxf(fmaxf(__fsub_rd(nl, g), __fsub_rd(g, nh)), 0.f);
+                            v = __fmaf_rd(e, e, v);
+                        }
+                    }
+                } else if (c < s + k && live && t < H) {
+                    nl = ahead ? ul[i] : a.lo[(size_t)box * d + t * k + (c - s)];
+                    nh = ahead ? uh[i] : a.hi[(size_t)box * d + t * k + (c - s)];
+                }
+                bad |= !(fabsf(nl) < INFINITY) || !(fabsf(nh) < INFINITY);
+                buf_lo(0)[r * ld + c] = nl;
+                buf_hi(0)[r * ld + c] = nh;
+            }
+            if (t > 0) {
+                v = warp_sum_rd(v);
+                if (a.cost.kind == 1) {
+                    // w_t times the distance from g to the box, then the penalties at their minima (rounded down)
+                    __syncwarp();
+                    float pen = 0.f;
+                    const int nq = s / 2 + 1;
+                    for (int q = lane; q < a.cost.n_obs * nq; q += 32) {
+                        const int o = q / nq, kp = q % nq - 1;
+                        pen = __fadd_rd(pen, kp < 0 ? penalty_min_rd(a.cost, o, pbx[4 * r], pbx[4 * r + 2],
+                                                                     pbx[4 * r + 1], pbx[4 * r + 3])
+                                                    : penalty_min_rd(a.cost, o, xl[r * s4 + 2 * kp], xu[r * s4 + 2 * kp],
+                                                                     xl[r * s4 + 2 * kp + 1], xu[r * s4 + 2 * kp + 1]));
+                    }
+                    pen = warp_sum_rd(pen);
+                    v = __fadd_rd(__fmul_rd(a.cost.w[t - 1], __fsqrt_rd(v)), pen);
+                }
+            }
+            if (a.rho > 0.f && t < H) {
+                if (ahead) {
+                    const float q = live && lane >= s && lane < s + k ? sq_min_rd(ul[i], uh[i]) : 0.f;
+                    vu = __shfl_sync(0xFFFFFFFFu, q, lane + s);
+                    vu = lane < k ? __fadd_rd(0.f, vu) : 0.f;
+                } else if (live)
+                    for (int j = lane; j < k; j += 32)
+                        vu = __fadd_rd(vu, sq_min_rd(a.lo[(size_t)box * d + t * k + j], a.hi[(size_t)box * d + t * k + j]));
+                vu = warp_sum_rd(vu);
+            }
+            if (lane == 0) {
+                float lb = lbacc[r];
+                if (t > 0) lb = __fadd_rd(lb, v);
+                if (a.rho > 0.f && t < H) lb = __fadd_rd(lb, __fmul_rd(a.rho, vu));
+                lbacc[r] = lb;
+                if (a.cost.kind == 1 && live && t < H) {
+                    // the pusher after u_t (read at x_{t+1}'s cost)
+                    const float *ul = a.lo + (size_t)box * d + t * k, *uh = a.hi + (size_t)box * d + t * k;
                     pbx[4 * r] = __fadd_rd(pbx[4 * r], ul[0]);
                     pbx[4 * r + 1] = __fadd_rd(pbx[4 * r + 1], ul[1]);
                     pbx[4 * r + 2] = __fadd_ru(pbx[4 * r + 2], uh[0]);
                     pbx[4 * r + 3] = __fadd_ru(pbx[4 * r + 3], uh[1]);
                 }
-        if (a.rho > 0.f) {
-            for (int r = warp; r < RB; r += NT / 32) {
-                const int box = box0 + r;
-                float v = 0.f;
-                if (box < nlive)
-                    for (int j = lane; j < k; j += 32)
-                        v = __fadd_rd(v, sq_min_rd(a.lo[(size_t)box * d + t * k + j], a.hi[(size_t)box * d + t * k + j]));
-                v = warp_sum_rd(v);
-                if (lane == 0) lbacc[r] = __fadd_rd(lbacc[r], __fmul_rd(a.rho, v));
             }
         }
-        __syncthreads();
-        int cur = 0;
+        if (t == H) break;
+        if (ahead) load_u(t + 1);
+        int any = group_or(grp, TG, safe | (int)bad);
+        cur = 0;
         for (int l = 1; l <= L; ++l) {
-            const int Kp = pad4(N.dims[l - 1]), Np = pad4(N.dims[l]), dl = N.dims[l];
-            // 2 rows x 4 columns per thread: a 16-row tile of a 128-wide layer is then one item per thread
-            // (2 x 8 left half the threads idle: 21% slower on both the pushing and manipulation networks)
+            const int Kp = pad4(N.dims[l - 1]), Np = pad4(N.dims[l]);
             IbpSink o;
             const size_t base = (size_t)box0 * H + t;
-            o.pre_lo = a.pre_lo + base * sumh;
-            o.pre_hi = a.pre_hi + base * sumh;
-            o.S = a.S + base * (sumh + s);
+            o.pre_lo = a.pre_lo + base * sumh + (l < L ? N.hoff[l] : 0);
+            o.pre_hi = a.pre_hi + base * sumh + (l < L ? N.hoff[l] : 0);
+            o.S = a.S ? a.S + base * (sumh + s) + (l < L ? N.hoff[l] : sumh) : nullptr;
             o.rstride_h = (size_t)H * sumh;
             o.rstride_s = (size_t)H * (sumh + s);
-            o.hoff = l < L ? N.hoff[l] : 0;
-            o.soff = l < L ? N.hoff[l] : sumh;
-            o.dl = dl;
+            o.dl = N.dims[l];
             o.nrows = nlive - box0;
             o.hidden = l < L;
-            // (an output layer of 8 or 16 columns: 1 x 2 tiles, twice the threads of 1 x 4 on its K-long sums)
-            if (Np >= 64)
-                ibp_dense<2, 4>(blo[cur], bhi[cur], ld, img + N.fwd_w[l], img + N.fwd_b[l], Kp, Np, blo[cur ^ 1],
-                                bhi[cur ^ 1], o);
-            else if (Np >= 32)
-                ibp_dense<1, 4>(blo[cur], bhi[cur], ld, img + N.fwd_w[l], img + N.fwd_b[l], Kp, Np, blo[cur ^ 1],
-                                bhi[cur ^ 1], o);
-            else
-                ibp_dense<1, 2>(blo[cur], bhi[cur], ld, img + N.fwd_w[l], img + N.fwd_b[l], Kp, Np, blo[cur ^ 1],
-                                bhi[cur ^ 1], o);
-            __syncthreads();
+            o.vec_h = (vec_h >> l) & 1;
+            o.vec_s = (vec_s >> l) & 1;
+            o.full = (rb * Np) % 512 == 0;
+            // the input's masks, the output's, and the ones to clear for the next layer (read before the last barrier)
+            const uint32_t *mk = masks + (size_t)mcur * 8 * rb;
+            mcur = mcur == 2 ? 0 : mcur + 1;
+            o.mask = masks + (size_t)mcur * 8 * rb;
+            {
+                uint32_t *clear = masks + (size_t)(mcur == 2 ? 0 : mcur + 1) * 8 * rb;
+                for (int i = tid; i < 8 * rb; i += TG) clear[i] = 0u;
+            }
+            const float *in_l = buf_lo(cur), *in_h = buf_hi(cur), *Wt = img + N.fwd_w[l], *bias = img + N.fwd_b[l];
+            float *zl = buf_lo(cur ^ 1), *zh = buf_hi(cur ^ 1);
+            if (any) {
+                bad = ibp_dense_any(tid, TG, l == 1, in_l, in_h, ld, rb, Wt, bias, Kp, Np, zl, zh, o);
+            } else if (!STREAM && l > 1 && rb * Np <= 2 * TG && Np < 64) {
+                bad = ibp_dense_narrow(tid, TG, in_l, in_h, ld, rb, Wt, bias, Kp, Np, zl, zh, o);
+            } else if (STREAM) {
+                // the largest tile whose items still cover the threads: 32 rows of 256, 128 or 32 columns
+                if (l == 1) {
+                    if (Np > 128) bad = ibp_dense_stream<4, 4, true>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                    else if (Np > 32) bad = ibp_dense_stream<2, 4, true>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                    else bad = ibp_dense_stream<1, 2, true>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                } else {
+                    if (Np > 128) bad = ibp_dense_stream<4, 4, false>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                    else if (Np > 32) bad = ibp_dense_stream<2, 4, false>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                    else bad = ibp_dense_stream<1, 2, false>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                }
+            } else {
+                switch ((l == 1 ? 4 : 0) + ((tiles >> (2 * l)) & 3)) {
+                    case 0: bad = ibp_dense<4, 4, false>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                    case 1: bad = ibp_dense<2, 4, false>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                    case 2: bad = ibp_dense<1, 4, false>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                    case 3: bad = ibp_dense<1, 2, false>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                    case 4:
+                    case 5: bad = ibp_dense<2, 4, true>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                    case 6: bad = ibp_dense<1, 4, true>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                    default: bad = ibp_dense<1, 2, true>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
+                }
+            }
+            any = group_or(grp, TG, safe | (int)bad);
             cur ^= 1;
         }
-        // x_{t+1} in [x_t] + [z_L]; interval bound of ||x_{t+1} - g||^2
-        for (int r = warp; r < RB; r += NT / 32) {
-            const int box = box0 + r;
-            float v = 0.f;
-            for (int i = lane; i < s; i += 32) {
-                const float nl = __fadd_rd(xl[r * s4 + i], blo[cur][r * ld + i]);
-                const float nh = __fadd_ru(xu[r * s4 + i], bhi[cur][r * ld + i]);
-                xl[r * s4 + i] = nl;
-                xu[r * s4 + i] = nh;
-                if (box < nlive && a.x_lo) {
-                    a.x_lo[((size_t)box * (H + 1) + t + 1) * s + i] = nl;
-                    a.x_hi[((size_t)box * (H + 1) + t + 1) * s + i] = nh;
-                }
-                const float g = a.goal[i];
-                if (a.cost.kind == 0) {
-                    v = __fadd_rd(v, sq_min_rd(__fsub_rd(nl, g), __fsub_ru(nh, g)));
-                } else {
-                    // distance from g to the interval, rounded down, squared rounded down
-                    const float e = fmaxf(fmaxf(__fsub_rd(nl, g), __fsub_rd(g, nh)), 0.f);
-                    v = __fmaf_rd(e, e, v);
-                }
-            }
-            v = warp_sum_rd(v);
-            if (a.cost.kind == 1) {
-                // w_t times the distance from g to the box, then the penalties at their minima (each rounded down)
-                __syncwarp();
-                float pen = 0.f;
-                const int nq = s / 2 + 1;
-                for (int q = lane; q < a.cost.n_obs * nq; q += 32) {
-                    const int o = q / nq, kp = q % nq - 1;
-                    pen = __fadd_rd(pen, kp < 0 ? penalty_min_rd(a.cost, o, pbx[4 * r], pbx[4 * r + 2], pbx[4 * r + 1],
-                                                                 pbx[4 * r + 3])
-                                                : penalty_min_rd(a.cost, o, xl[r * s4 + 2 * kp], xu[r * s4 + 2 * kp],
-                                                                 xl[r * s4 + 2 * kp + 1], xu[r * s4 + 2 * kp + 1]));
-                }
-                pen = warp_sum_rd(pen);
-                v = __fadd_rd(__fmul_rd(a.cost.w[t], __fsqrt_rd(v)), pen);
-            }
-            if (lane == 0) lbacc[r] = __fadd_rd(lbacc[r], v);
-        }
-        __syncthreads();
     }
-    if (a.lb_ibp)
-        for (int r = threadIdx.x; r < RB; r += NT)
+    __syncwarp();
+    if (a.lb_ibp && lane == 0)
+        for (int r = warp; r < rb; r += TG / 32)
             if (box0 + r < nlive) a.lb_ibp[box0 + r] = lbacc[r];
 }
 
@@ -918,11 +1267,100 @@ static cudaError_t launch_rows_kernel(K kern_smem, K kern_glob, size_t img_bytes
     return cudaGetLastError();
 }
 
-cudaError_t launch_ibp(const BoundArgs &a, int, cudaStream_t st)
+// Cycles one input of a layer takes a scheduler of k_ibp with groups of rb rows, and the tile (0: 4 x 4, 1: 2 x 4,
+// 2: 1 x 4, 3: 1 x 2 outputs a thread) that takes the fewest: the FMAs of the tile, the sign split of its weights (the
+// ALU pipe has half the FMA pipe's width) and its loads, times the warps' passes; a tile that leaves a group fewer
+// than four warps leaves schedulers without one.
+static int ibp_tile(int rb, int Np, int &tile)
+{
+    static const int tr[4] = {4, 2, 1, 1}, tn[4] = {4, 4, 4, 2}, cost[4] = {50, 30, 22, 13};
+    int best = -1;
+    for (int i = 0; i < 4; ++i) {
+        if (rb % tr[i]) continue;
+        const int warps = ((rb / tr[i]) * (Np / tn[i]) + 31) / 32;
+        const int c = (warps > 4 ? (warps + 3) / 4 : 1) * cost[i] * kIbpGroups * (warps < 4 ? 3 : 4) / 4;
+        if (best < 0 || c < best) {
+            best = c;
+            tile = i;
+        }
+    }
+    return best;
+}
+
+// Boxes per group of k_ibp over n boxes: the count up to `most` whose waves of tiles take the least time (per layer
+// its inputs' cycles plus about 700 for the barrier, the stores and the step's share of the rest).
+static int ibp_rows(const NetDesc &N, int n, int num_sms, int most, int &tiles)
+{
+    int best = most;
+    long long best_cost = -1;
+    for (int rb = most; rb >= 1; --rb) {
+        const int per = rb * kIbpGroups;
+        const long long waves = ((n + per - 1) / per + num_sms - 1) / num_sms;
+        long long c = 0;
+        int code = 0;
+        for (int l = 1; l <= N.L; ++l) {
+            int tile;
+            c += 700 + 16 * rb + (long long)pad4(N.dims[l - 1]) * ibp_tile(rb, pad4(N.dims[l]), tile);
+            code |= tile << (2 * l);
+        }
+        if (best_cost < 0 || waves * c < best_cost) {
+            best_cost = waves * c;
+            best = rb;
+            tiles = code;
+        }
+    }
+    return best;
+}
+
+static int sm_count()
+{
+    int dev, v = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v;
+}
+
+// Which layers' columns can be stored four at a time: bit l for layer l of the [n][H][sumh] arrays (vec_h) and of S
+// (vec_s).
+static void ibp_vec(const BoundArgs &a, int &vec_h, int &vec_s)
 {
     const NetDesc &N = a.net;
-    size_t rest = (4 * (size_t)RB * N.maxw_p + 2 * (size_t)RB * pad4(N.s) + 5 * (size_t)RB) * sizeof(float);
-    return launch_rows_kernel(k_ibp<true>, k_ibp<false>, (size_t)N.img_floats * 4, rest, a.n, a, st);
+    auto al = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
+    vec_h = vec_s = 0;
+    for (int l = 1; l <= N.L; ++l) {
+        const int off = l < N.L ? N.hoff[l] : N.sumh;
+        if (N.sumh % 4 == 0 && off % 4 == 0 && al(a.pre_lo) && al(a.pre_hi)) vec_h |= 1 << l;
+        if ((N.sumh + N.s) % 4 == 0 && off % 4 == 0 && al(a.S)) vec_s |= 1 << l;
+    }
+}
+
+cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st)
+{
+    if (a.n <= 0) return cudaSuccess;
+    const NetDesc &N = a.net;
+    const int budget = max_optin_smem();
+    if (num_sms <= 0) num_sms = sm_count();
+    int vec_h, vec_s;
+    ibp_vec(a, vec_h, vec_s);
+    const size_t img = N.img_floats;
+    int most = 8;
+    while (most >= 1 && (img + kIbpGroups * ibp_rest_floats(N, most)) * 4 > (size_t)budget) --most;
+    if (most >= 4) {
+        int tiles = 0;
+        const int rb = ibp_rows(N, a.n, num_sms, most, tiles), per = rb * kIbpGroups;
+        const size_t smem = (img + kIbpGroups * ibp_rest_floats(N, rb)) * 4;
+        cudaError_t e = cudaFuncSetAttribute(k_ibp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_ibp<false><<<(a.n + per - 1) / per, kIbpNT, smem, st>>>(a, rb, tiles, vec_h, vec_s, a.unchecked);
+    } else {
+        const int rb = kIbpStreamRows;
+        const size_t smem = ((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, rb)) * 4;
+        if (smem > (size_t)budget) return cudaErrorInvalidConfiguration;
+        cudaError_t e = cudaFuncSetAttribute(k_ibp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_ibp<true><<<(a.n + rb - 1) / rb, kIbpNT, smem, st>>>(a, rb, 0, vec_h, vec_s, a.unchecked);
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_crown(const BoundArgs &a, int, cudaStream_t st)

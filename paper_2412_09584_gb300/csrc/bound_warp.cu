@@ -516,8 +516,8 @@ static cudaError_t launch_warp_variant(const BoundArgs &a, int steps, float lr, 
 // Interval bound propagation (outward-rounded FP32) through the H-step unrolled
 // network, one warp per box: lane q holds the interval of inputs and outputs
 // q, q + 32, ...; per output the three directed-rounding sums (lower, upper,
-// and S = sum_j |W_kj| max|a_j|) run over the inputs in order from the bias, as
-// in k_ibp, so the bounds are bit-identical to it.  Writes the pre-activation
+// and the one S = sum_j |W_kj| max|a_j| is formed from) run over the inputs in
+// order from the bias, as in k_ibp, so the bounds are bit-identical to it.  Writes the pre-activation
 // bounds, the state intervals, S and (nullable) the interval bound of the cost.
 template <int P, bool WSMEM>
 __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_ibp_warp(BoundArgs a)
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_
                     for (int kl = 0; kl < kn; ++kl) {
                         const float il = __shfl_sync(0xFFFFFFFFu, zl[pk], kl);
                         const float ih = __shfl_sync(0xFFFFFFFFu, zu[pk], kl);
-                        const float am = fmaxf(fabsf(il), fabsf(ih));
+                        const float am = l == 1 ? fmaxf(fabsf(il), fabsf(ih)) : il;
 #pragma unroll
                         for (int q = 0; q < P; ++q) {
                             if (lane + 32 * q < Np) {
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_
                 for (int q = 0; q < P; ++q) {
                     const int j = lane + 32 * q;
                     if (j < dl) {
-                        S[(size_t)t * sw + soff + j] = as_[q];
+                        S[(size_t)t * sw + soff + j] = l == 1 ? as_[q] : ibp_s(al_[q], ah_[q], bias[j], as_[q]);
                         if (l < L) {
                             pl[(size_t)t * sumh + N.hoff[l] + j] = al_[q];
                             ph[(size_t)t * sumh + N.hoff[l] + j] = ah_[q];

@@ -97,13 +97,15 @@ struct BoundArgs {
     const float *x0, *goal, *lo, *hi;
     int n;
     const int *d_n;
+    int unchecked;           // the weights were not checked to be finite (a network handed over on the device)
     int row0;                // the launch's first row within the caller's arrays (chunked calls; d_n counts from 0)
     int H, d;
     float rho;
     // interval bounds (written by k_ibp, read by k_crown / k_alpha_fwd)
     float *pre_lo, *pre_hi;  // [n][H][sumh]
     float *x_lo, *x_hi;      // [n][H+1][s]
-    float *S;                // [n][H][sumh + s]: per row of each layer, sum_j |W_kj| max|a_j| over the input box
+    float *S;                // [n][H][sumh + s] (nullable): per row of each layer, an upper bound of sum_j |W_kj| max|a_j|
+                             // over the input box
     float *lb_ibp;           // [n] (nullable)
     // CROWN
     const float *alpha;      // [n][H][sumh] (nullable: adaptive)
@@ -222,6 +224,14 @@ __device__ __forceinline__ float obstacle_state_lin_row(const CostDesc &c, int t
         }
     }
     return cst;
+}
+
+// S of a later layer from its sums: with 0 <= a_lo <= a_hi, sum |w| a_hi = (upper - b) + (b - lower) + sum |w| a_lo
+// in exact arithmetic; upper and lower are rounded outward, so the same sum rounded up bounds it from above (and is
+// as tight as adding |w| a_hi term by term: the two parts' roundings are relative to sums that add up to S).
+__device__ __forceinline__ float ibp_s(float lo, float hi, float b, float v)
+{
+    return __fadd_ru(__fadd_ru(__fsub_ru(hi, b), __fsub_ru(b, lo)), v);
 }
 
 struct AdamStep {
