@@ -567,8 +567,10 @@ int bab_prune_branch_batch(bab_ctx *ctx, int d_stride, const int *horizon, int m
  * FP32 rollout variants, and the fused alpha loop against the separate
  * launches, give bit-identical results: each output is summed in the same
  * order whatever the tile).
- *   BAB_KERNEL_ROLLOUT_FP32  0: 64 samples x 256 threads, one CTA per SM;
- *                            1: 64 x 256 with <= 128 registers; 2: 32 x 128.
+ *   BAB_KERNEL_ROLLOUT_FP32  0 (and -1): register tiles of 64 samples (per-box
+ *                            tiles, one CTA per SM, for batched problems and
+ *                            search-integrated bounds); per-box tiles of
+ *                            1: 64 samples x 256 threads, 2: 32 x 128.
  *   BAB_KERNEL_ALPHA_FUSED   -2: separate bound / adjoint / Adam launches;
  *                            0, 1, 2: one launch, 2, 4 or 8 boxes per CTA with
  *                            all per-box state in shared memory (small

@@ -337,6 +337,9 @@ __device__ __forceinline__ void dense_rows_auto(const float *in, int ldi, const 
 // variant < 0 picks by shared-memory size; rollout_fp32_variants() variants exist (the autotuner times them)
 cudaError_t launch_rollout_fp32(const RolloutArgs &a, int variant, int num_sms, cudaStream_t st);
 int rollout_fp32_variants();
+// FP32 rollouts of one problem with register tiles (rollout_rows.cu); keys filled by the caller
+bool rollout_rows_supported(const RolloutArgs &a, size_t budget);
+cudaError_t launch_rollout_rows(const RolloutArgs &a, int num_sms, size_t budget, cudaStream_t st);
 cudaError_t launch_rollout_tc(RolloutArgs a, int split, int nslot_pref, int num_sms, cudaStream_t st);
 // the synthetic objective sum 5 u^2 + cos(50 u): sampled search (uniform, or the cross-entropy mode with
 // cem_mu / cem_sigma and costs), sound interval bound, FP64 incumbent
