@@ -208,16 +208,51 @@ __global__ void k_rollout_finalize(RolloutArgs a)
 }
 
 // Incumbent update: the box with the smallest ub (lowest index on ties) has its best_u re-evaluated in FP64; if the
-// value beats *inc_val, it becomes the incumbent.  The FP64 rate of one SM (about one multiply-add per clock) sets
-// the pace of a one-CTA evaluation, so a large network's row is evaluated by a cluster of kIncCTAs CTAs (a small
-// one's by a cluster of one, which leaves the other SMs to the bounds that run beside it): every CTA keeps the whole
-// layer input in its shared memory, computes its share of each layer's outputs (each output's sum split over ks
-// lanes, strided over the inputs, and added across them by shuffles) and writes them into every CTA's shared memory
-// (distributed shared memory); a cluster barrier closes each layer and each step's cost.  The control flow depends
-// only on values every CTA of the cluster computes alike, so all of them reach the same barriers.
+// value beats *inc_val, it becomes the incumbent.  One row is a chain of H x L layers, so what bounds it is the FP64
+// rate of the SMs it runs on (two multiply-adds per clock each) and, once that is spread, each layer's latency.  A
+// cluster of kIncCTAs CTAs shares every layer's outputs (one CTA for the smallest networks): each CTA keeps its rows of
+// every layer's weights in shared memory as doubles for all steps, an output's sum is split over ks lanes (strided over
+// the inputs, added by shuffles), lane by lane written into the CTAs' shared memory (distributed shared memory), and
+// one cluster barrier closes the layer.  The outputs alternate between two buffers without restarting at a step: a CTA
+// at most one layer ahead then writes the buffer that nobody reads.  The control flow depends only on values every CTA
+// of the cluster computes alike, so all of them reach the same barriers.
+// Pushing network (20 steps): 603 -> 146 us (one CTA before); object manipulation (40 steps): 1136 -> 488 us (the
+// weights read from L2 at every step before); tiny network (5 steps), one CTA: 39 -> 28 us.
 constexpr int kIncCTAs = 16;  // a non-portable cluster size; 8 where the GPU cannot place 16
+constexpr int kIncThreads = 256;
+constexpr int kIncActions = 1024;  // action coordinates kept in shared memory (a longer plan is read as it goes)
 
-__global__ void __launch_bounds__(256) k_incumbent_fp64(RolloutArgs a)
+// Lanes per output of a layer with ni inputs of which a CTA computes `chunk` outputs: the power of two that takes the
+// fewest clocks.  A warp's FP64 instruction holds the SM's FP64 unit for 16 clocks (and a warp waits longer than that
+// for its own result), the additions across lanes like the multiply-adds, so few lanes are best.
+__host__ __device__ inline int incumbent_lanes(int chunk, int ni)
+{
+    int best = 1, cost = 1 << 30;
+    for (int ks = 1, lg = 0; ks <= 32 && chunk * ks <= kIncThreads; ks *= 2, ++lg) {
+        const int warps = (chunk * ks + 31) / 32, c = ((ni + ks - 1) / ks + 4 + lg) * (warps > 2 ? 16 * warps : 40);
+        if (c < cost) {
+            cost = c;
+            best = ks;
+        }
+    }
+    return best;
+}
+
+// doubles of shared memory a CTA of a cluster of ncta needs: its rows of every layer's weights (ni + lanes apart, so
+// that the outputs of a warp read different banks) and their biases
+__host__ __device__ inline size_t incumbent_doubles(const NetDesc &N, int ncta)
+{
+    size_t f = 0;
+    for (int l = 1; l <= N.L; ++l) {
+        const int chunk = (N.dims[l] + ncta - 1) / ncta;
+        f += (size_t)chunk * (N.dims[l - 1] + incumbent_lanes(chunk, N.dims[l - 1]) + 1);
+    }
+    return f;
+}
+
+// WSMEM: the CTA's rows fit in shared memory (else they are read through L2).
+template <bool WSMEM>
+__global__ void __launch_bounds__(kIncThreads) k_incumbent_fp64(RolloutArgs a)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -232,23 +267,43 @@ __global__ void __launch_bounds__(256) k_incumbent_fp64(RolloutArgs a)
     const float rho = problem_rho(a.batch, pb, a.rho);
     double *inc_val = a.inc_val + pb;
     float *inc_u = a.inc_u + (size_t)pb * a.d;
-    __shared__ unsigned long long red[8];
-    __shared__ double act[2][kMaxWidth + 4];
-    __shared__ double xs[kMaxWidth];
+    extern __shared__ double wsh[];  // WSMEM: per layer this CTA's rows [chunk][ni], then their biases [chunk]
+    __shared__ unsigned long long red[kIncThreads / 32];
+    __shared__ double act[2][kMaxWidth];
+    __shared__ double xin[kMaxWidth], xs[kMaxWidth], gl[kMaxWidth];
+    __shared__ float us[kIncActions];
     __shared__ double f_sh;
-    __shared__ int row_sh;
+    __shared__ int row_sh, ks_sh[kMaxLayers + 1];
     const int lane = threadIdx.x & 31;
+    if (threadIdx.x >= 1 && (int)threadIdx.x <= N.L)
+        ks_sh[threadIdx.x] = incumbent_lanes((N.dims[threadIdx.x] + ncta - 1) / ncta, N.dims[threadIdx.x - 1]);
     unsigned long long best = ~0ull;
-    for (int i = threadIdx.x; i < nlive; i += blockDim.x)
+#pragma unroll 8
+    for (int i = threadIdx.x; i < nlive; i += kIncThreads)
         if (row_problem(a.batch, i) == pb)
             best = umin64(best, ((unsigned long long)float_order(a.ub[i]) << 32) | (unsigned)i);
+    if (WSMEM) {
+        double *w = wsh;
+        for (int l = 1; l <= N.L; ++l) {
+            const int no = N.dims[l], ni = N.dims[l - 1], chunk = (no + ncta - 1) / ncta, q0 = rank * chunk;
+            const int mine = min(chunk, no - q0), ldw = ni + incumbent_lanes(chunk, ni);  // (mine may be <= 0)
+#pragma unroll 4
+            for (int i = threadIdx.x; i < mine * ni; i += kIncThreads) {
+                const int r = i / ni;
+                w[r * ldw + (i - r * ni)] = (double)raw[N.raw_w[l] + (size_t)q0 * ni + i];
+            }
+            w += chunk * ldw;
+            for (int i = threadIdx.x; i < mine; i += kIncThreads) w[i] = (double)raw[N.raw_b[l] + q0 + i];
+            w += chunk;
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best = umin64(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
     if (lane == 0) red[threadIdx.x >> 5] = best;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long b = red[0];
-        for (int w = 1; w < 8; ++w) b = umin64(b, red[w]);
+        for (int w = 1; w < kIncThreads / 32; ++w) b = umin64(b, red[w]);
         row_sh = (b == ~0ull) ? -1 : (int)(b & 0xFFFFFFFFu);
         f_sh = 0.0;
     }
@@ -257,64 +312,101 @@ __global__ void __launch_bounds__(256) k_incumbent_fp64(RolloutArgs a)
     if (row < 0) return;  // the same in every CTA of the cluster
     const float *u = a.best_u + (size_t)row * a.d;
     const int s = N.s, k = N.k;
-    double px = (double)a.cost.p0x, py = (double)a.cost.p0y;  // pusher position (obstacle cost; thread 0)
-    for (int i = threadIdx.x; i < s; i += blockDim.x) xs[i] = (double)x0[i];
-    __syncthreads();
+    double px = (double)a.cost.p0x, py = (double)a.cost.p0y;  // pusher position (obstacle cost; lane 0)
+    double f = 0.0;  // the first warp's partial sums of the objective, added up at the end
+    const bool u_sh = Hb * k <= kIncActions;
+    if (u_sh)
+        for (int j = threadIdx.x; j < Hb * k; j += kIncThreads) us[j] = u[j];
+    for (int i = threadIdx.x; i < s; i += kIncThreads) gl[i] = (double)goal[i];
+    for (int i = threadIdx.x; i < s; i += kIncThreads) xs[i] = (double)x0[i];
+    for (int c = threadIdx.x; c < s + k; c += kIncThreads) xin[c] = c < s ? (double)x0[c] : (Hb > 0 ? (double)u[c - s] : 0.0);
+    if (ncta > 1) cluster.sync();  // every CTA of the cluster runs before its shared memory is written
+    else __syncthreads();
+    int cur = 0;  // the buffer the next layer writes
     for (int t = 0; t < Hb; ++t) {
-        for (int c = threadIdx.x; c < s + k; c += blockDim.x)
-            act[0][c] = c < s ? xs[c] : (double)u[t * k + (c - s)];
-        __syncthreads();
-        int cur = 0;
+        const double *w = wsh;
         for (int l = 1; l <= N.L; ++l) {
             const int no = N.dims[l], ni = N.dims[l - 1];
-            const float *W = raw + N.raw_w[l];
-            const float *b = raw + N.raw_b[l];
-            // this CTA's outputs q0 .. q0 + chunk - 1 (chunk <= 256, the widest layer): cp >= chunk slots of ks
-            // lanes each (ks a power of two, at most 32, cp ks <= 256 threads)
+            const double *in = l == 1 ? xin : act[cur ^ 1];
+            // this CTA's outputs q0 .. q0 + chunk - 1 (chunk <= 256, the widest layer), ks lanes each
             const int chunk = (no + ncta - 1) / ncta, q0 = rank * chunk;
-            int cp = 1;
-            while (cp < chunk) cp *= 2;
-            const int ks = 256 / cp > 32 ? 32 : 256 / cp;
+            const int ks = ks_sh[l], ldw = ni + ks;
             const int ql = (int)threadIdx.x / ks, sl = (int)threadIdx.x % ks, q = q0 + ql;
             const bool mine = ql < chunk && q < no;
-            double part = 0.0;
-            if (mine)
-                for (int c = sl; c < ni; c += ks) part = fma((double)W[(size_t)q * ni + c], act[cur][c], part);
-            for (int o = ks / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
-            if (mine && sl == 0) {
-                double v = (double)b[q] + part;
-                if (l < N.L && v < 0.0) v = 0.0;
-                for (int r2 = 0; r2 < ncta; ++r2) cluster.map_shared_rank(&act[cur ^ 1][0], r2)[q] = v;
+            if (((int)threadIdx.x & ~31) < chunk * ks) {  // (whole warps)
+                double pt[4] = {0.0, 0.0, 0.0, 0.0};
+                if (mine) {
+                    if (WSMEM) {
+                        const double *wq = w + ql * ldw;
+                        int c = sl;
+                        for (; c + 3 * ks < ni; c += 4 * ks)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) pt[e] = fma(wq[c + e * ks], in[c + e * ks], pt[e]);
+                        for (; c < ni; c += ks) pt[0] = fma(wq[c], in[c], pt[0]);
+                    } else {
+                        const float *wq = raw + N.raw_w[l] + (size_t)q * ni;
+#pragma unroll 4
+                        for (int c = sl; c < ni; c += ks) pt[0] = fma((double)wq[c], in[c], pt[0]);
+                    }
+                }
+                double part = (pt[0] + pt[1]) + (pt[2] + pt[3]);
+                for (int o = ks / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
+                if (mine) {
+                    double v = (WSMEM ? w[chunk * ldw + ql] : (double)raw[N.raw_b[l] + q]) + part;
+                    if (l < N.L && v < 0.0) v = 0.0;
+                    // (every lane of the output holds the sum: lane r2 writes CTA r2's copy)
+                    if (ncta == 1) {
+                        if (sl == 0) act[cur][q] = v;
+                    } else {
+                        for (int r2 = sl; r2 < ncta; r2 += ks) cluster.map_shared_rank(&act[cur][0], r2)[q] = v;
+                    }
+                }
             }
-            cluster.sync();  // every CTA's copy of the layer output complete
+            w += chunk * (ldw + 1);
+            if (ncta > 1) cluster.sync();  // every CTA's copy of the layer output complete
+            else __syncthreads();
             cur ^= 1;
         }
-        if (threadIdx.x == 0) {
-            double f = f_sh;
-            for (int i = 0; i < s; ++i) xs[i] += act[cur][i];
-            if (a.cost.kind == 0) {
-                for (int i = 0; i < s; ++i) {
-                    const double e = xs[i] - (double)goal[i];
-                    f += e * e;
+        // x_{t+1}, its cost and the next input row (every CTA its own copy)
+        const double *z = act[cur ^ 1];
+        if (threadIdx.x < 32) {
+            for (int i = lane; i < s; i += 32) {
+                const double x = xs[i] + z[i];
+                xs[i] = x;
+                xin[i] = x;
+                if (a.cost.kind == 0) {
+                    const double e = x - gl[i];
+                    f = fma(e, e, f);
                 }
-            } else {
-                px += (double)u[t * k];
-                py += (double)u[t * k + 1];
-                f += obstacle_cost_f64(a.cost, t + 1, s, xs, goal, px, py);
             }
-            for (int j = 0; j < k; ++j) {
-                const double uu = (double)u[t * k + j];
-                f += (double)rho * uu * uu;
+            for (int j = lane; j < k; j += 32) {
+                const double uu = (double)(u_sh ? us[t * k + j] : u[t * k + j]);
+                f = fma((double)rho * uu, uu, f);
             }
-            f_sh = f;
+            if (a.cost.kind != 0) {
+                __syncwarp();
+                if (lane == 0) {
+                    px += (double)u[t * k];
+                    py += (double)u[t * k + 1];
+                    f += obstacle_cost_f64(a.cost, t + 1, s, xs, goal, px, py);
+                }
+            }
+        } else if (t + 1 < Hb) {
+            for (int j = (int)threadIdx.x - 32; j < k; j += kIncThreads - 32)
+                xin[s + j] = (double)(u_sh ? us[(t + 1) * k + j] : u[(t + 1) * k + j]);
         }
-        cluster.sync();  // the output read before the next step's first layer overwrites it
+        __syncthreads();
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xFFFFFFFFu, f, o);
     if (rank != 0) return;
-    if (threadIdx.x == 0) row_sh = (f_sh < *inc_val) ? 1 : 0;
+    if (threadIdx.x == 0) {
+        f_sh = f;
+        row_sh = (f < *inc_val) ? 1 : 0;
+    }
     __syncthreads();
     if (row_sh) {
-        for (int j = threadIdx.x; j < a.d; j += blockDim.x) inc_u[j] = u[j];
+        for (int j = threadIdx.x; j < a.d; j += kIncThreads) inc_u[j] = u[j];
         if (threadIdx.x == 0) *inc_val = f_sh;
     }
 }
@@ -443,41 +535,33 @@ void launch_rollout_finalize(const RolloutArgs &a, cudaStream_t st)
     if (a.n > 0) k_rollout_finalize<<<a.n, 128, 0, st>>>(a);
 }
 
-void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
+template <bool WSMEM>
+static bool incumbent_placed(int ncta, size_t smem)
 {
-    if (a.n <= 0) return;
-    // a cluster of kIncCTAs (else 8) for rows of more than 2 M multiply-adds (at about one FP64 multiply-add per
-    // clock, a millisecond on one SM), else one CTA per problem
-    const NetDesc &N = a.net;
-    long long macs = 0;
-    for (int l = 1; l <= N.L; ++l) macs += (long long)N.dims[l] * N.dims[l - 1];
-    int ncta = macs * a.H > 2000000 ? kIncCTAs : 1;
-    // whether this GPU places a 16-CTA cluster of the kernel (non-portable size): decided at the first large launch,
-    // which runs eagerly before any graph capture, and kept (one device per process)
-    static int big_ok = -1;
-    if (ncta > 8 && big_ok < 0) {
-        big_ok = 0;
-        if (cudaFuncSetAttribute(k_incumbent_fp64, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-            cudaLaunchConfig_t q = {};
-            q.gridDim = dim3((unsigned)ncta);
-            q.blockDim = dim3(256);
-            cudaLaunchAttribute qa[1];
-            qa[0].id = cudaLaunchAttributeClusterDimension;
-            qa[0].val.clusterDim.x = (unsigned)ncta;
-            qa[0].val.clusterDim.y = 1;
-            qa[0].val.clusterDim.z = 1;
-            q.attrs = qa;
-            q.numAttrs = 1;
-            int nclusters = 0;
-            big_ok = cudaOccupancyMaxActiveClusters(&nclusters, k_incumbent_fp64, &q) == cudaSuccess && nclusters >= 1;
-        }
-        cudaGetLastError();
-    }
-    if (ncta > 8 && !big_ok) ncta = 8;
+    cudaLaunchConfig_t q = {};
+    q.gridDim = dim3((unsigned)ncta);
+    q.blockDim = dim3(kIncThreads);
+    q.dynamicSmemBytes = smem;
+    cudaLaunchAttribute qa[1];
+    qa[0].id = cudaLaunchAttributeClusterDimension;
+    qa[0].val.clusterDim.x = (unsigned)ncta;
+    qa[0].val.clusterDim.y = 1;
+    qa[0].val.clusterDim.z = 1;
+    q.attrs = qa;
+    q.numAttrs = 1;
+    int nclusters = 0;
+    const bool ok = cudaOccupancyMaxActiveClusters(&nclusters, k_incumbent_fp64<WSMEM>, &q) == cudaSuccess && nclusters >= 1;
+    cudaGetLastError();
+    return ok;
+}
+
+template <bool WSMEM>
+static void incumbent_run(const RolloutArgs &a, int ncta, size_t smem, cudaStream_t st)
+{
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ncta * (a.batch.P > 1 ? a.batch.P : 1)));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
+    cfg.blockDim = dim3(kIncThreads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -486,7 +570,36 @@ void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_incumbent_fp64, a);
+    cudaLaunchKernelEx(&cfg, k_incumbent_fp64<WSMEM>, a);
+}
+
+void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
+{
+    if (a.n <= 0) return;
+    // One CTA where a step is at most 4096 multiply-adds (2048 clocks of one SM's FP64 rate, about the layers' cluster
+    // barriers) or many problems are evaluated side by side and each is small; else a cluster of kIncCTAs, or of 8 where
+    // the GPU does not place 16.
+    const NetDesc &N = a.net;
+    long long macs = 0;
+    for (int l = 1; l <= N.L; ++l) macs += (long long)N.dims[l] * N.dims[l - 1];
+    int ncta = macs > (a.batch.P > 1 ? 65536 : 4096) ? kIncCTAs : 1;
+    // whether this GPU places a 16-CTA cluster (non-portable size) with the most shared memory the kernel takes:
+    // decided at the first launch, which runs eagerly before any graph capture, and kept (one device per process)
+    constexpr size_t kMaxSmem = 200 * 1024;
+    static const bool big_ok = [] {
+        bool ok = true;
+        for (int w = 0; w < 2; ++w) {
+            auto kern = w ? k_incumbent_fp64<true> : k_incumbent_fp64<false>;
+            ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+            if (w) ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) == cudaSuccess;
+        }
+        cudaGetLastError();
+        return ok && incumbent_placed<true>(kIncCTAs, kMaxSmem) && incumbent_placed<false>(kIncCTAs, 0);
+    }();
+    if (ncta > 8 && !big_ok) ncta = 8;
+    const size_t smem = incumbent_doubles(N, ncta) * sizeof(double);
+    if (smem <= kMaxSmem) incumbent_run<true>(a, ncta, smem, st);
+    else incumbent_run<false>(a, ncta, 0, st);
 }
 
 }  // namespace bab
