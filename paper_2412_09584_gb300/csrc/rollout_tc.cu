@@ -1080,86 +1080,162 @@ __global__ void __launch_bounds__(256) k_rescore_fp32(RolloutArgs a)
     }
 }
 
-// BF16 mode, one problem, top-k re-score of a large network: the boxes of the top-k list, one per thread-block
-// cluster at a time.  Each of the cluster's CTAs stages its share of each layer's columns of W_l^T (at most 32) in
-// shared memory, computes those outputs one per thread (the same sums, in the same order, as k_rescore_fp32 and
-// k_rescore_rows: from the bias over the inputs in order) and writes them into every CTA's shared memory
-// (distributed shared memory); a cluster barrier closes each layer and each step's cost.  The list and its count
-// are the same for every CTA, so all of them reach the same barriers.
-constexpr int kRescoreCTAs = 8;
+// BF16 mode, one problem, top-k re-score of a large network: the boxes of the top-k list, nbox (at most kRescoreBoxes)
+// per thread-block cluster at a time, a warp each in every CTA.  Each of the cluster's CTAs keeps its share of every layer's
+// columns of W_l^T (at most 32) in shared memory for all steps and boxes, computes those outputs one per lane (the same
+// sums, in the same order, as k_rescore_fp32 and k_rescore_rows: from the bias over the inputs in order) and writes them
+// into every CTA's shared memory (distributed shared memory); a cluster barrier closes each layer.  The outputs alternate
+// between two buffers without restarting at a step, so a CTA one layer ahead writes the buffer that nobody reads.  The
+// list and its count are the same for every CTA, so all of them reach the same barriers.
+// What bounds it: the chain of 200 layers (40 steps of the object-manipulation network), each a dependent FMA chain of
+// up to 256 inputs and a cluster barrier.  64 boxes: 1710 us with every layer's columns staged from L2 at every step
+// and one box per cluster -> 401 us.
+constexpr int kRescoreCTAs = 8, kRescoreBoxes = 8, kRescoreClThreads = 32 * kRescoreBoxes;
+
+// Floats of shared memory for a CTA's columns of every layer, [inputs][columns] and their biases each.
+__host__ __device__ inline size_t rescore_cl_floats(const NetDesc &N)
+{
+    size_t f = 0;
+    for (int l = 1; l <= N.L; ++l) f += (size_t)(N.dims[l - 1] + 1) * ((N.dims[l] + kRescoreCTAs - 1) / kRescoreCTAs);
+    return f;
+}
+
 template <bool OBST>
-__global__ void __launch_bounds__(256) k_rescore_cl(RolloutArgs a)
+__global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a, int nbox)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank(), ncta = (int)cluster.num_blocks();
-    const int cl = (int)blockIdx.x / ncta, ncl = (int)gridDim.x / ncta;
-    extern __shared__ float wsl[];  // [inputs][32]: this CTA's columns of W_l^T
-    __shared__ float act[2][kMaxWidth + 4];
-    __shared__ float xs[kMaxWidth];
-    __shared__ float f_sh;
+    const int rank = (int)cluster.block_rank();
+    const int cl = (int)blockIdx.x / kRescoreCTAs, ncl = (int)gridDim.x / kRescoreCTAs;
+    extern __shared__ float wsl[];  // per layer this CTA's columns of W_l^T
+    __shared__ float4 act4[kRescoreBoxes][2][kMaxWidth / 4];
+    __shared__ float4 xin4[kRescoreBoxes][kMaxWidth / 4];
+    __shared__ float xs_[kRescoreBoxes][kMaxWidth], es_[kRescoreBoxes][kMaxWidth];
     const NetDesc &N = a.net;
     const int s = N.s, k = N.k, d = a.d;
+    const int lane = threadIdx.x & 31, slot = threadIdx.x >> 5;
     const int count = (int)a.topk_t[3];
-    const float *fwd = a.fwd;
-    const float *x0 = a.x0, *goal = a.goal;
+    if (cl * nbox >= count) return;  // the same in every CTA of the cluster
+    {
+        float *w = wsl;
+        for (int l = 1; l <= N.L; ++l) {
+            const int no = N.dims[l], ni = N.dims[l - 1], Np = pad4(no);
+            const int chunk = (no + kRescoreCTAs - 1) / kRescoreCTAs, q0 = rank * chunk;
+            const float *Wt = a.fwd + N.fwd_w[l];
+#pragma unroll 8
+            for (int i = threadIdx.x; i < ni * chunk; i += kRescoreClThreads) {
+                const int c = i / chunk, j = i - c * chunk;
+                w[i] = q0 + j < no ? __ldg(Wt + (size_t)c * Np + q0 + j) : 0.f;
+            }
+            w += ni * chunk;
+            for (int j = threadIdx.x; j < chunk; j += kRescoreClThreads) w[j] = q0 + j < no ? a.fwd[N.fwd_b[l] + q0 + j] : 0.f;
+            w += chunk;
+        }
+    }
+    // (the warps beyond the boxes' have helped stage the weights; they go on to the barriers only)
+    const bool works = slot < nbox;
+    const int sl = works ? slot : 0;
+    float *xin = reinterpret_cast<float *>(xin4[sl]), *xs = xs_[sl], *es = es_[sl];
     const float rho = a.rho;
-    for (int e = cl; e < count; e += ncl) {
-        const int box = a.topk_list[e];
-        const unsigned long long key = a.keys[box];
-        const uint32_t m = (uint32_t)(key & 0xFFFFFFFFu);
+    for (int e0 = cl * nbox; e0 < count; e0 += ncl * nbox) {
+        const bool live = works && e0 + slot < count;
+        const int box = a.topk_list[live ? e0 + slot : e0];  // (an idle slot repeats the first box)
+        const uint32_t m = (uint32_t)(a.keys[box] & 0xFFFFFFFFu);
         const uint64_t hb = box_hash(a.seed, a.id[box]);
         const float *blo = a.lo + (size_t)box * d, *bhi = a.hi + (size_t)box * d;
-        for (int i = threadIdx.x; i < s; i += blockDim.x) xs[i] = x0[i];
-        if (threadIdx.x == 0) f_sh = 0.f;
-        float px = OBST ? a.cost.p0x : 0.f, py = OBST ? a.cost.p0y : 0.f;  // pusher position (thread 0)
-        __syncthreads();
+        auto draw = [&](int t) {
+            // the actions u_t at their place of the input row
+            for (int j = lane; j < k; j += 32)
+                xin[s + j] = draw_sample(hb, m, (uint32_t)(t * k + j), blo[t * k + j], bhi[t * k + j]);
+        };
+        if (works) {
+            for (int i = lane; i < s; i += 32) xin[i] = xs[i] = a.x0[i];
+            draw(0);
+        }
+        float f = 0.f, px = OBST ? a.cost.p0x : 0.f, py = OBST ? a.cost.p0y : 0.f;
+        cluster.sync();  // the weights staged; the cluster's CTAs running, the last boxes' buffers free
+        int cur = 0;
         for (int t = 0; t < a.H; ++t) {
-            for (int c = threadIdx.x; c < s + k; c += blockDim.x)
-                act[0][c] = c < s ? xs[c]
-                                  : draw_sample(hb, m, (uint32_t)(t * k + c - s), blo[t * k + c - s], bhi[t * k + c - s]);
-            __syncthreads();
-            int cur = 0;
+            const float *w = wsl;
             for (int l = 1; l <= N.L; ++l) {
-                const int no = N.dims[l], ni = N.dims[l - 1], Np = pad4(no);
-                const int chunk = (no + ncta - 1) / ncta, q0 = rank * chunk;  // chunk <= 32: widths <= 256
-                const float *Wt = fwd + N.fwd_w[l];
-                for (int i = threadIdx.x; i < ni * 32; i += blockDim.x) {
-                    const int c = i >> 5, j = i & 31;
-                    wsl[i] = (j < chunk && q0 + j < no) ? __ldg(Wt + (size_t)c * Np + q0 + j) : 0.f;
-                }
-                __syncthreads();
-                const int q = q0 + (int)threadIdx.x;
-                if ((int)threadIdx.x < chunk && q < no) {
-                    float acc = fwd[N.fwd_b[l] + q];
-                    for (int c = 0; c < ni; ++c) acc = fmaf(wsl[c * 32 + threadIdx.x], act[cur][c], acc);
+                const int no = N.dims[l], ni = N.dims[l - 1];
+                const int chunk = (no + kRescoreCTAs - 1) / kRescoreCTAs, q = rank * chunk + lane;  // chunk <= 32
+                const float4 *in = l == 1 ? xin4[sl] : act4[sl][cur ^ 1];
+                if (works && lane < chunk && q < no) {
+                    float acc = w[ni * chunk + lane];
+                    // 16 inputs at a time, the next 16 loaded under this chain of multiply-adds
+                    const float *wq = w + lane;
+                    float wa[16], wb[16];
+                    float4 xa[4], xb[4];
+                    auto load = [&](float (&wr)[16], float4 (&xr)[4], int c0) {
+                        const float *pw = wq + c0 * chunk;
+#pragma unroll
+                        for (int cc = 0; cc < 16; ++cc, pw += chunk) wr[cc] = *pw;
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) xr[cc] = in[(c0 >> 2) + cc];
+                    };
+                    auto add = [&](const float (&wr)[16], const float4 (&xr)[4]) {
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) {
+                            acc = fmaf(wr[4 * cc], xr[cc].x, acc);
+                            acc = fmaf(wr[4 * cc + 1], xr[cc].y, acc);
+                            acc = fmaf(wr[4 * cc + 2], xr[cc].z, acc);
+                            acc = fmaf(wr[4 * cc + 3], xr[cc].w, acc);
+                        }
+                    };
+                    const int whole = ni & ~15;
+                    if (whole > 0) load(wa, xa, 0);
+                    int c = 0;
+                    for (; c + 32 <= whole; c += 32) {
+                        load(wb, xb, c + 16);
+                        add(wa, xa);
+                        if (c + 32 < whole) load(wa, xa, c + 32);
+                        add(wb, xb);
+                    }
+                    if (c < whole) {
+                        add(wa, xa);
+                        c += 16;
+                    }
+                    for (; c < ni; ++c) acc = fmaf(wq[c * chunk], reinterpret_cast<const float *>(in)[c], acc);
                     const float v = (l < N.L) ? fmaxf(acc, 0.f) : acc;
-                    for (int r2 = 0; r2 < ncta; ++r2) cluster.map_shared_rank(&act[cur ^ 1][0], r2)[q] = v;
+                    float *out = reinterpret_cast<float *>(act4[sl][cur]);
+#pragma unroll
+                    for (int r2 = 0; r2 < kRescoreCTAs; ++r2) cluster.map_shared_rank(out, r2)[q] = v;
                 }
-                cluster.sync();  // every CTA's copy of the layer output complete, the staged columns free again
+                w += (ni + 1) * chunk;
+                cluster.sync();  // every CTA's copy of the layer output complete
                 cur ^= 1;
             }
-            if (threadIdx.x == 0) {
-                float f = f_sh;
+            if (!works) continue;
+            // the step's action cost, then the state cost, each in index order (every CTA its own copy; lane 0's sums)
+            const float *z = reinterpret_cast<const float *>(act4[sl][cur ^ 1]);
+            for (int i = lane; i < s; i += 32) {
+                const float x = xs[i] + z[i];
+                xs[i] = x;
+                es[i] = x - a.goal[i];
+            }
+            __syncwarp();
+            if (lane == 0) {
                 for (int j = 0; j < k; ++j) {
-                    const float u = draw_sample(hb, m, (uint32_t)(t * k + j), blo[t * k + j], bhi[t * k + j]);
+                    const float u = xin[s + j];
                     f = fmaf(rho * u, u, f);
                     if (OBST && j == 0) px = __fadd_rn(px, u);
                     if (OBST && j == 1) py = __fadd_rn(py, u);
                 }
                 float c = 0.f;
-                for (int i = 0; i < s; ++i) {
-                    xs[i] = xs[i] + act[cur][i];
-                    const float ee = xs[i] - goal[i];
-                    c = fmaf(ee, ee, c);
-                }
-                if (OBST) c = obstacle_cost_f32(a.cost, t + 1, s, xs, goal, px, py);
-                f_sh = f + c;
+                if (OBST) c = obstacle_cost_f32(a.cost, t + 1, s, xs, a.goal, px, py);
+                else
+                    for (int i = 0; i < s; ++i) c = fmaf(es[i], es[i], c);
+                f = f + c;
             }
-            cluster.sync();  // the output read before the next step's first layer overwrites it
+            __syncwarp();
+            for (int i = lane; i < s; i += 32) xin[i] = xs[i];
+            if (t + 1 < a.H) draw(t + 1);
+            __syncwarp();
         }
-        if (rank == 0 && threadIdx.x == 0) a.ub[box] = f_sh;  // best_u was written by the finalize kernel
+        if (rank == 0 && lane == 0 && live) a.ub[box] = f;  // best_u was written by the finalize kernel
     }
+    cluster.sync();  // no CTA leaves while another may still write its shared memory
 }
 
 // BF16 mode, one problem, every box re-scored: the same FP32 re-score as k_rescore_fp32 for a tile of RR boxes
@@ -1262,13 +1338,19 @@ static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
     const NetDesc &N = a.net;
     long long macs = 0;
     for (int l = 1; l <= N.L; ++l) macs += (long long)N.dims[l] * N.dims[l - 1];
-    if (a.batch.P <= 1 && a.topk > 0 && macs * a.H > 2000000) {
-        // a large network's top k: a cluster of kRescoreCTAs per listed box
+    const size_t cl_smem = rescore_cl_floats(N) * sizeof(float);
+    if (a.batch.P <= 1 && a.topk > 0 && macs * a.H > 2000000 && cl_smem <= 200 * 1024) {
+        // a large network's top k: a cluster of kRescoreCTAs per nbox listed boxes, as many as make one wave of clusters
+        // (this GPU holds 15 at one CTA per SM), at most a warp each
+        auto kern = a.cost.kind == 1 ? k_rescore_cl<true> : k_rescore_cl<false>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem);
+        if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
-        const int ncl = a.topk < 64 ? a.topk : 64;
-        cfg.gridDim = dim3((unsigned)(kRescoreCTAs * ncl));
-        cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = (size_t)N.maxw_p * 32 * sizeof(float);
+        const int nbox = a.topk > 15 * kRescoreBoxes ? kRescoreBoxes : (a.topk + 14) / 15;
+        const int ncl = (a.topk + nbox - 1) / nbox;
+        cfg.gridDim = dim3((unsigned)(kRescoreCTAs * (ncl < 15 ? ncl : 15)));
+        cfg.blockDim = dim3(kRescoreClThreads);
+        cfg.dynamicSmemBytes = cl_smem;
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1277,8 +1359,7 @@ static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return a.cost.kind == 1 ? cudaLaunchKernelEx(&cfg, k_rescore_cl<true>, a)
-                                : cudaLaunchKernelEx(&cfg, k_rescore_cl<false>, a);
+        return cudaLaunchKernelEx(&cfg, kern, a, nbox);
     }
     if (a.batch.P > 1 || a.topk > 0) {
         // each box reads its own problem's image; with a top-k selection all but k boxes return at once
