@@ -736,11 +736,12 @@ __host__ __device__ inline size_t fwd_rows_floats(const NetDesc &N, int rb)
 
 // Theorem 1 backward propagation of the tangent-linearised cost through all H
 // steps, then Theorem 2 in box form, for rows 0 .. nrows-1 of the view (rows
-// nrows .. RBT-1 are padding).  img: backward image; p: crown_rows_floats of
-// shared memory.
+// nrows .. RBT-1 are padding), by NTT consecutive threads of the CTA (group grp
+// of them).  img: backward image; p: crown_rows_floats of shared memory.
 template <int RBT, int NTT>
-__device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const RowsView &v, int nrows)
+__device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const RowsView &v, int nrows, int grp = 0)
 {
+    const int tid = threadIdx.x % NTT;
     const NetDesc &N = a.net;
     const int s = N.s, k = N.k, L = N.L, d = a.d, H = a.H, sumh = N.sumh, sw = sumh + s;
     const int ld = N.maxw_p, s4 = pad4(s), d4 = pad4(d);
@@ -752,7 +753,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
     float *cst = p; p += RBT;
     float *mg = p; p += RBT;
     float *Pu = p; p += 4 * RBT;  // obstacle cost: per row the pusher coefficient of the actions (2) and its |sum| (2)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = tid & 31, warp = tid >> 5;
     const bool obst = a.cost.kind == 1;
     const bool has_alpha = v.alpha != nullptr;
     const int ts = a.t_stop;              // early stop: propagate back to x_ts only
@@ -760,7 +761,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
 
     // early stop: the cost terms at steps 1 .. ts on their intervals, no coefficient of u before ts
     if (ts > 0) {
-        for (int i = threadIdx.x; i < RBT * d4; i += NTT) mu[i] = 0.f;
+        for (int i = tid; i < RBT * d4; i += NTT) mu[i] = 0.f;
         for (int r = warp; r < RBT; r += NTT / 32) {
             float c = 0.f;
             if (r < nrows)
@@ -812,7 +813,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
             mg[r] = 0.f;
         }
     }
-    __syncthreads();
+    group_barrier(grp, NTT);
 
     for (int t = H - 1; t >= ts; --t) {
         // last layer: A = lam on z_L (rows of W_L), constant lam . b_L
@@ -836,9 +837,9 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                     mg[r] = __fmaf_ru(N.gam[L], e, mg[r]);
                 }
             }
-            __syncthreads();
-            dense_rows_auto<RBT, NTT>(Ab[0], ld, img + N.bwd_w[L], nullptr, NpL, pad4(N.dims[L - 1]), Ab[1], ld, false);
-            __syncthreads();
+            group_barrier(grp, NTT);
+            dense_rows_auto<RBT, NTT>(Ab[0], ld, img + N.bwd_w[L], nullptr, NpL, pad4(N.dims[L - 1]), Ab[1], ld, false, tid);
+            group_barrier(grp, NTT);
         }
         int cur = 1;
         for (int l = L - 1; l >= 1; --l) {
@@ -875,10 +876,10 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                     mg[r] = __fadd_ru(mg[r], __fmaf_ru(N.gam[l], eg, __fmul_ru(kTwoU, er)));
                 }
             }
-            __syncthreads();
+            group_barrier(grp, NTT);
             dense_rows_auto<RBT, NTT>(Ab[cur], ld, img + N.bwd_w[l], nullptr, Npl, pad4(N.dims[l - 1]), Ab[cur ^ 1],
-                                      ld, false);
-            __syncthreads();
+                                      ld, false, tid);
+            group_barrier(grp, NTT);
             cur ^= 1;
         }
         // A is on [x_t | u_t]: mu_t = A_u; lam <- lam + A_x (+ tangent of ||x_t - g||^2 for t >= 1)
@@ -949,7 +950,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 mg[r] = __fadd_ru(mg[r], e);
             }
         }
-        __syncthreads();
+        group_barrier(grp, NTT);
     }
 
     // lam . x0, then Theorem 2 in box form: sum_j min_{u in [lo, hi]} mu_j u + rho u^2
@@ -1012,8 +1013,9 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
 // not needed again in this pass); otherwise the gradient goes to v.grad.
 template <int RBT, int NTT>
 __device__ void fwd_rows(const BoundArgs &a, const float *img, float *p, const RowsView &v, int nrows,
-                         const AdamStep *adam)
+                         const AdamStep *adam, int grp = 0)
 {
+    const int tid = threadIdx.x % NTT;
     const NetDesc &N = a.net;
     const int s = N.s, k = N.k, L = N.L, d = a.d, H = a.H, sumh = N.sumh;
     const int ld = N.maxw_p, s4 = pad4(s);
@@ -1023,26 +1025,26 @@ __device__ void fwd_rows(const BoundArgs &a, const float *img, float *p, const R
     float *xs = p; p += RBT * s4;
     const bool has_alpha = v.alpha != nullptr;
     const int Kp1 = pad4(s + k);
-    for (int i = threadIdx.x; i < RBT * s; i += NTT) xs[(i / s) * s4 + i % s] = a.x0[i % s];
-    __syncthreads();
+    for (int i = tid; i < RBT * s; i += NTT) xs[(i / s) * s4 + i % s] = a.x0[i % s];
+    group_barrier(grp, NTT);
     for (int t = 0; t < H; ++t) {
-        for (int i = threadIdx.x; i < RBT * Kp1; i += NTT) {
+        for (int i = tid; i < RBT * Kp1; i += NTT) {
             const int r = i / Kp1, c = i % Kp1;
             float val = 0.f;
             if (c < s) val = xs[r * s4 + c];
             else if (c < s + k && r < nrows) val = v.ustar[(size_t)r * d + t * k + (c - s)];
             Z[0][r * ld + c] = val;
         }
-        __syncthreads();
+        group_barrier(grp, NTT);
         int cur = 0;
         for (int l = 1; l <= L; ++l) {
             dense_rows_auto<RBT, NTT>(Z[cur], ld, img + N.fwd_w[l], img + N.fwd_b[l], pad4(N.dims[l - 1]),
-                                      pad4(N.dims[l]), Z[cur ^ 1], ld, false);
-            __syncthreads();
+                                      pad4(N.dims[l]), Z[cur ^ 1], ld, false, tid);
+            group_barrier(grp, NTT);
             cur ^= 1;
             if (l < L) {
                 const int dl = N.dims[l];
-                for (int i = threadIdx.x; i < RBT * dl; i += NTT) {
+                for (int i = tid; i < RBT * dl; i += NTT) {
                     const int r = i / dl, q = i % dl;
                     if (r >= nrows) continue;
                     const size_t idx = ((size_t)r * H + t) * sumh + N.hoff[l] + q;
@@ -1056,55 +1058,45 @@ __device__ void fwd_rows(const BoundArgs &a, const float *img, float *p, const R
                     else v.grad[idx] = g;
                     Z[cur][r * ld + q] = fmaf(D, z, c);
                 }
-                __syncthreads();
+                group_barrier(grp, NTT);
             }
         }
-        for (int i = threadIdx.x; i < RBT * s; i += NTT) {
+        for (int i = tid; i < RBT * s; i += NTT) {
             const int r = i / s, c = i % s;
             xs[r * s4 + c] += Z[cur][r * ld + c];
         }
+        group_barrier(grp, NTT);
+    }
+}
+
+// CROWN (FWD: the forward pass of its adjoint) over RBT boxes per group of warps: the image in shared memory (WSMEM,
+// else read through L2) is shared by kRowGroups groups with their own buffers and barriers, so that one group's interval
+// loads and row reductions run under another's products.
+constexpr int kRowGroups = 4, kRowGroupThreads = NT / kRowGroups;
+
+template <int RBT, bool WSMEM, bool FWD>
+__global__ void __launch_bounds__(NT, 1) k_rows(BoundArgs a, int stride)
+{
+    extern __shared__ float4 smem4[];
+    float *sm = reinterpret_cast<float *>(smem4);
+    const NetDesc &N = a.net;
+    const int nlive = live_count(a.n, a.d_n, a.row0);
+    if ((int)blockIdx.x * kRowGroups * RBT >= nlive) return;
+    const float *img = FWD ? a.fwd : a.bwd;
+    float *p = sm;
+    if (WSMEM) {
+        for (int i = threadIdx.x; i < N.img_floats / 4; i += NT) smem4[i] = reinterpret_cast<const float4 *>(img)[i];
+        img = sm;
+        p += N.img_floats;
         __syncthreads();
     }
-}
-
-template <bool WSMEM>
-__global__ void __launch_bounds__(NT) k_crown(BoundArgs a)
-{
-    extern __shared__ float4 smem4[];
-    float *sm = reinterpret_cast<float *>(smem4);
-    const NetDesc &N = a.net;
-    const float *img = a.bwd;
-    float *p = sm;
-    if (WSMEM) {
-        for (int i = threadIdx.x; i < N.img_floats / 4; i += NT) smem4[i] = reinterpret_cast<const float4 *>(a.bwd)[i];
-        img = sm;
-        p += N.img_floats;
-    }
-    const int nlive = live_count(a.n, a.d_n, a.row0);
-    const int box0 = blockIdx.x * RB;
+    const int grp = threadIdx.x / kRowGroupThreads;
+    const int box0 = ((int)blockIdx.x * kRowGroups + grp) * RBT;
     if (box0 >= nlive) return;
-    const int nrows = min(RB, nlive - box0);
-    crown_rows<RB, NT>(a, img, p, global_view(a, box0), nrows);
-}
-
-template <bool WSMEM>
-__global__ void __launch_bounds__(NT) k_alpha_fwd(BoundArgs a)
-{
-    extern __shared__ float4 smem4[];
-    float *sm = reinterpret_cast<float *>(smem4);
-    const NetDesc &N = a.net;
-    const float *img = a.fwd;
-    float *p = sm;
-    if (WSMEM) {
-        for (int i = threadIdx.x; i < N.img_floats / 4; i += NT) smem4[i] = reinterpret_cast<const float4 *>(a.fwd)[i];
-        img = sm;
-        p += N.img_floats;
-    }
-    const int nlive = live_count(a.n, a.d_n, a.row0);
-    const int box0 = blockIdx.x * RB;
-    if (box0 >= nlive) return;
-    const int nrows = min(RB, nlive - box0);
-    fwd_rows<RB, NT>(a, img, p, global_view(a, box0), nrows, nullptr);
+    const int nrows = min(RBT, nlive - box0);
+    p += (size_t)grp * stride;
+    if (FWD) fwd_rows<RBT, kRowGroupThreads>(a, img, p, global_view(a, box0), nrows, nullptr, grp);
+    else crown_rows<RBT, kRowGroupThreads>(a, img, p, global_view(a, box0), nrows, grp);
 }
 
 // ---------------------------------------------------------------------------
@@ -1252,21 +1244,6 @@ static int max_optin_smem()
     return v - 1024;
 }
 
-template <typename K>
-static cudaError_t launch_rows_kernel(K kern_smem, K kern_glob, size_t img_bytes, size_t rest_bytes, int n,
-                                      const BoundArgs &a, cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    const int budget = max_optin_smem();
-    const bool wsmem = img_bytes + rest_bytes <= (size_t)budget;
-    const size_t smem = (wsmem ? img_bytes : 0) + rest_bytes;
-    if (smem > (size_t)budget) return cudaErrorInvalidConfiguration;
-    K kern = wsmem ? kern_smem : kern_glob;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<(n + RB - 1) / RB, NT, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
 // Cycles one input of a layer takes a scheduler of k_ibp with groups of rb rows, and the tile (0: 4 x 4, 1: 2 x 4,
 // 2: 1 x 4, 3: 1 x 2 outputs a thread) that takes the fewest: the FMAs of the tile, the sign split of its weights (the
 // ALU pipe has half the FMA pipe's width) and its loads, times the warps' passes; a tile that leaves a group fewer
@@ -1363,29 +1340,58 @@ cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_crown(const BoundArgs &a, int, cudaStream_t st)
+// Rows per group of k_rows: the smallest of 1, 2, 4, 8 with which one wave of CTAs holds all boxes (a step takes a group
+// about the same time with one row as with two), at most what fits in shared memory; 8 beyond one wave.
+template <bool FWD>
+static cudaError_t launch_rows(const BoundArgs &a, int num_sms, cudaStream_t st)
 {
+    if (a.n <= 0) return cudaSuccess;
     const NetDesc &N = a.net;
-    size_t rest = crown_rows_floats(N, RB, a.d) * sizeof(float);
-    return launch_rows_kernel(k_crown<true>, k_crown<false>, (size_t)N.img_floats * 4, rest, a.n, a, st);
+    const size_t budget = (size_t)max_optin_smem(), img = (size_t)N.img_floats * 4;
+    auto floats = [&](int rb) { return FWD ? fwd_rows_floats(N, rb) : crown_rows_floats(N, rb, a.d); };
+    auto group = [&](int rb) { return ((floats(rb) + 3) & ~size_t(3)) * 4; };
+    if (floats(RB) * 4 > budget) return cudaErrorInvalidConfiguration;  // (the working set of a tile of RB boxes)
+    if (num_sms <= 0) num_sms = sm_count();
+    int rb = 1;
+    while (rb < 8 && (long long)num_sms * kRowGroups * rb < a.n) rb *= 2;
+    // (fewer rows rather than the image out of shared memory)
+    const size_t beside = img + kRowGroups * group(1) <= budget ? img : 0;
+    while (rb > 1 && beside + kRowGroups * group(rb) > budget) rb /= 2;
+    const bool wsmem = img + kRowGroups * group(rb) <= budget;
+    const size_t smem = (wsmem ? img : 0) + kRowGroups * group(rb);
+    auto run = [&](auto kern) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int per = kRowGroups * rb;
+        kern<<<(a.n + per - 1) / per, NT, smem, st>>>(a, (int)(group(rb) / 4));
+        return cudaGetLastError();
+    };
+    switch (rb) {
+        case 1: return wsmem ? run(k_rows<1, true, FWD>) : run(k_rows<1, false, FWD>);
+        case 2: return wsmem ? run(k_rows<2, true, FWD>) : run(k_rows<2, false, FWD>);
+        case 4: return wsmem ? run(k_rows<4, true, FWD>) : run(k_rows<4, false, FWD>);
+        default: return wsmem ? run(k_rows<8, true, FWD>) : run(k_rows<8, false, FWD>);
+    }
 }
+
+cudaError_t launch_crown(const BoundArgs &a, int num_sms, cudaStream_t st) { return launch_rows<false>(a, num_sms, st); }
 
 cudaError_t preload_ibp_crown()
 {
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, k_ibp<true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_ibp<false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_crown<true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_crown<false>);
-    return e;
+    const void *kerns[] = {(const void *)k_ibp<true>, (const void *)k_ibp<false>,
+                           (const void *)k_rows<1, true, false>, (const void *)k_rows<1, false, false>,
+                           (const void *)k_rows<2, true, false>, (const void *)k_rows<2, false, false>,
+                           (const void *)k_rows<4, true, false>, (const void *)k_rows<4, false, false>,
+                           (const void *)k_rows<8, true, false>, (const void *)k_rows<8, false, false>};
+    for (const void *k : kerns) {
+        cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-cudaError_t launch_alpha_fwd(const BoundArgs &a, int, cudaStream_t st)
-{
-    const NetDesc &N = a.net;
-    size_t rest = fwd_rows_floats(N, RB) * sizeof(float);
-    return launch_rows_kernel(k_alpha_fwd<true>, k_alpha_fwd<false>, (size_t)N.img_floats * 4, rest, a.n, a, st);
-}
+cudaError_t launch_alpha_fwd(const BoundArgs &a, int num_sms, cudaStream_t st) { return launch_rows<true>(a, num_sms, st); }
 
 static size_t fused_smem(const NetDesc &N, int rb, int H, int d)
 {

@@ -258,27 +258,43 @@ struct AdamTable {
     float bc1[kAdamTable], bc2[kAdamTable];
 };
 
+// Paired FP32 FMA, per element the scalar fmaf.
+__device__ __forceinline__ unsigned long long ffma2_rn(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pack_f32x2(float x, float y)
+{
+    return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
+}
+
 // out[r][c] = act(sum_k in[r][k] * B[k][c] + bias[c]) for r < R, c < Np, where
-// B is [Kp][Np] row-major (a forward image Wt_l, or a backward image W_l).
+// B is [Kp][Np] row-major (a forward image Wt_l, or a backward image W_l), by
+// NT threads (tid: this one's number among them).  Each output is the FMA chain
+// over k from the bias; two columns run as one FMA pair (TN = 1: one output).
 // Kp % 4 == 0 and Np % 4 == 0; bias may be null.
 template <int R, int NT, int TR, int TN>
 __device__ __forceinline__ void dense_rows(const float *__restrict__ in, int ldi, const float *__restrict__ B,
                                            const float *__restrict__ bias, int Kp, int Np, float *__restrict__ out,
-                                           int ldo, bool relu)
+                                           int ldo, bool relu, int tid)
 {
+    constexpr int TP = (TN + 1) / 2;
     const int ngc = (Np + TN - 1) / TN;
     const int items = (R / TR) * ngc;
-    for (int it = threadIdx.x; it < items; it += NT) {
+    for (int it = tid; it < items; it += NT) {
         const int cg = it % ngc, rg = it / ngc;
         const int c0 = cg * TN, r0 = rg * TR;
-        float acc[TR][TN];
-        float bv[TN];
+        unsigned long long acc[TR][TP];
 #pragma unroll
-        for (int j = 0; j < TN; ++j) bv[j] = (bias && c0 + j < Np) ? bias[c0 + j] : 0.f;
+        for (int j = 0; j < TP; ++j) {
+            const int c = c0 + 2 * j;
+            const unsigned long long b2 = pack_f32x2(bias && c < Np ? bias[c] : 0.f,
+                                                     bias && TN > 1 && c + 1 < Np ? bias[c + 1] : 0.f);
 #pragma unroll
-        for (int i = 0; i < TR; ++i)
-#pragma unroll
-            for (int j = 0; j < TN; ++j) acc[i][j] = bv[j];
+            for (int i = 0; i < TR; ++i) acc[i][j] = b2;
+        }
         const bool full = (c0 + TN <= Np);
         for (int k = 0; k < Kp; k += 4) {
             float4 xv[TR];
@@ -286,26 +302,35 @@ __device__ __forceinline__ void dense_rows(const float *__restrict__ in, int ldi
             for (int i = 0; i < TR; ++i) xv[i] = *reinterpret_cast<const float4 *>(in + (r0 + i) * ldi + k);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                float w[TN];
+                float w[2 * TP];
                 const float *wr = B + (size_t)(k + kk) * Np + c0;
-                if (full) {
+                if (TN >= 4 && full) {
 #pragma unroll
                     for (int j = 0; j < TN; j += 4) {
                         float4 q = *reinterpret_cast<const float4 *>(wr + j);
                         w[j] = q.x;
-                        w[j + 1] = q.y;
-                        w[j + 2] = q.z;
-                        w[j + 3] = q.w;
+                        w[(j + 1) % (2 * TP)] = q.y;
+                        w[(j + 2) % (2 * TP)] = q.z;
+                        w[(j + 3) % (2 * TP)] = q.w;
                     }
+                } else if (TN == 2) {
+                    const float2 q = *reinterpret_cast<const float2 *>(wr);
+                    w[0] = q.x;
+                    w[1] = q.y;
                 } else {
 #pragma unroll
-                    for (int j = 0; j < TN; ++j) w[j] = (c0 + j < Np) ? wr[j] : 0.f;
+                    for (int j = 0; j < 2 * TP; ++j) w[j] = (j < TN && c0 + j < Np) ? wr[j] : 0.f;
                 }
 #pragma unroll
                 for (int i = 0; i < TR; ++i) {
                     const float xs = kk == 0 ? xv[i].x : kk == 1 ? xv[i].y : kk == 2 ? xv[i].z : xv[i].w;
+                    if (TN == 1) {
+                        acc[i][0] = __float_as_uint(fmaf(xs, w[0], __uint_as_float((uint32_t)acc[i][0])));
+                    } else {
+                        const unsigned long long x2 = pack_f32x2(xs, xs);
 #pragma unroll
-                    for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(xs, w[j], acc[i][j]);
+                        for (int j = 0; j < TP; ++j) acc[i][j] = ffma2_rn(x2, pack_f32x2(w[2 * j], w[2 * j + 1]), acc[i][j]);
+                    }
                 }
             }
         }
@@ -314,7 +339,7 @@ __device__ __forceinline__ void dense_rows(const float *__restrict__ in, int ldi
 #pragma unroll
             for (int j = 0; j < TN; ++j)
                 if (c0 + j < Np) {
-                    const float v = acc[i][j];
+                    const float v = __uint_as_float((uint32_t)(j & 1 ? acc[i][j / 2] >> 32 : acc[i][j / 2]));
                     out[(r0 + i) * ldo + c0 + j] = relu ? fmaxf(v, 0.f) : v;
                 }
     }
@@ -323,14 +348,23 @@ __device__ __forceinline__ void dense_rows(const float *__restrict__ in, int ldi
 // Picks the register block so that the tile's items cover the threads.
 template <int R, int NT>
 __device__ __forceinline__ void dense_rows_auto(const float *in, int ldi, const float *B, const float *bias, int Kp,
-                                                int Np, float *out, int ldo, bool relu)
+                                                int Np, float *out, int ldo, bool relu, int tid = threadIdx.x)
 {
     if (R >= 4 && (R / 4) * ((Np + 7) / 8) >= NT / 2)
-        dense_rows<R, NT, (R >= 4 ? 4 : 1), 8>(in, ldi, B, bias, Kp, Np, out, ldo, relu);
+        dense_rows<R, NT, (R >= 4 ? 4 : 1), 8>(in, ldi, B, bias, Kp, Np, out, ldo, relu, tid);
     else if (R >= 2 && (R / 2) * ((Np + 3) / 4) >= NT / 2)
-        dense_rows<R, NT, (R >= 2 ? 2 : 1), 4>(in, ldi, B, bias, Kp, Np, out, ldo, relu);
+        dense_rows<R, NT, (R >= 2 ? 2 : 1), 4>(in, ldi, B, bias, Kp, Np, out, ldo, relu, tid);
+    else if (R * Np >= 2 * NT)
+        dense_rows<R, NT, 1, 4>(in, ldi, B, bias, Kp, Np, out, ldo, relu, tid);
     else
-        dense_rows<R, NT, 1, 4>(in, ldi, B, bias, Kp, Np, out, ldo, relu);
+        // few outputs: one a thread, so that the chain over k is all a thread does
+        dense_rows<R, NT, 1, 1>(in, ldi, B, bias, Kp, Np, out, ldo, relu, tid);
+}
+
+// Barrier of one group of nt threads of a CTA (groups are numbered from 0; barrier 0 is the CTA's own).
+__device__ __forceinline__ void group_barrier(int g, int nt)
+{
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(g + 1), "r"(nt) : "memory");
 }
 
 // host launchers (return the first CUDA error)
