@@ -1,13 +1,18 @@
 // branch.cu -- Pruner, batch_pick_out and batch_split of Algorithm 2
 // (Section 3 overview and Section 3.1), bit-exact and deterministic.
 //
-//   k_branch_plan   one CTA: the FP64 prune test, the pick-out selection (exact
-//                   k-th smallest of the composite keys (order(ub), id) and
-//                   (order(lb), id) by 8-bit radix selection), and the stable
-//                   ranks of picked and unpicked survivors (warp ballots).
-//   k_branch_write  one warp per pool row: the widest coordinate (warp
-//                   argmax, lowest index on ties), the FP32 midpoint, and the
+//   k_branch_plan_cl  one problem: a thread-block cluster plans the pool (the FP64
+//                   prune test, the pick-out selection as the exact k-th smallest
+//                   of the composite keys (order(ub), id) and (order(lb), id) by
+//                   8-bit radix selection, the stable ranks of picked and unpicked
+//                   survivors by warp ballots); k_branch_plan_small the same for
+//                   at most 256 rows, by counting.
+//   k_branch_plan   several problems: the same with one CTA per problem.
+//   k_branch_write  a few lanes per pool row: the widest coordinate (argmax over the
+//                   lanes, lowest index on ties), the FP32 midpoint, and the
 //                   coalesced writes of two children or of the unpicked row.
+#include <cooperative_groups.h>
+
 #include "bab_internal.cuh"
 #include "kernels.cuh"
 #include "select.cuh"
@@ -16,6 +21,18 @@ namespace bab {
 
 constexpr int kPlanThreads = 1024;
 constexpr int kPickFlag = 1 << 30;
+
+// Problem pb's quota, and the part of it that is taken by upper bound.
+__device__ __forceinline__ void plan_quota(const BranchArgs &a, int pb, int &n_pick, int &n1)
+{
+    n_pick = a.n_pick;
+    n1 = a.n1;
+    if (a.n_pick_dev) {
+        n_pick = a.n_pick_dev[pb] < 0 ? 0 : a.n_pick_dev[pb];
+        n1 = (int)ceil((double)a.eta * n_pick);
+        n1 = n1 > n_pick ? n_pick : n1;
+    }
+}
 
 __global__ void __launch_bounds__(kPlanThreads) k_branch_plan(BranchArgs a)
 {
@@ -31,12 +48,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan(BranchArgs a)
     const BatchDesc &B = a.batch;
     auto mine = [&](int i) { return B.prob == nullptr || row_problem(B, i) == pb; };
     const double inc = a.inc_val[pb];
-    int n_pick = a.n_pick, n1 = a.n1;
-    if (a.n_pick_dev) {
-        n_pick = a.n_pick_dev[pb] < 0 ? 0 : a.n_pick_dev[pb];
-        n1 = (int)ceil((double)a.eta * n_pick);
-        n1 = n1 > n_pick ? n_pick : n1;
-    }
+    int n_pick, n1;
+    plan_quota(a, pb, n_pick, n1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     // prune (strict, in FP64; a NaN bound is kept and latched as BAB_ERR_NUMERIC)
@@ -59,8 +72,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan(BranchArgs a)
     const bool all = ns <= n_pick;
     Thresh T1, T2;
     T1.none = T2.none = true;
-    // the rest of the quota is chosen on the lower bound, or on its softmax race key (pick_rule 1)
-    const float *key2 = a.pick_rule == 1 ? a.pick_keys : a.lb;
+    const float *key2 = a.lb;  // the rest of the quota is chosen on the lower bound
     if (!all) {
         const uint8_t *keep = a.keep;
         T1 = radix_select(n, a.ub, a.id, [&](int i) { return mine(i) && keep[i] != 0; }, n1, hist, &sh_pk, &sh_pid,
@@ -68,37 +80,6 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan(BranchArgs a)
         const float *ub = a.ub;
         const uint64_t *ids = a.id;
         auto cand = [&](int i) { return mine(i) && keep[i] != 0 && !le_thresh(float_order(ub[i]), ids[i], T1); };
-        if (a.pick_rule == 1) {
-            // min-max scaling over the candidates' (non-NaN) lower bounds, then each candidate's race key
-            float mn = INFINITY, mx = -INFINITY;
-            for (int i = threadIdx.x; i < n; i += blockDim.x)
-                if (cand(i) && a.lb[i] == a.lb[i]) {
-                    mn = fminf(mn, a.lb[i]);
-                    mx = fmaxf(mx, a.lb[i]);
-                }
-            for (int o = 16; o > 0; o >>= 1) {
-                mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
-                mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-            }
-            __shared__ float rmn[kPlanThreads / 32], rmx[kPlanThreads / 32];
-            if (lane == 0) {
-                rmn[warp] = mn;
-                rmx[warp] = mx;
-            }
-            __syncthreads();
-            mn = INFINITY;
-            mx = -INFINITY;
-            for (int w = 0; w < kPlanThreads / 32; ++w) {
-                mn = fminf(mn, rmn[w]);
-                mx = fmaxf(mx, rmx[w]);
-            }
-            for (int i = threadIdx.x; i < n; i += blockDim.x)
-                if (cand(i)) {
-                    const float v = a.lb[i];
-                    a.pick_keys[i] = v == v ? pick_key(v, mn, mx, a.temperature, a.pick_seed, ids[i]) : v;
-                }
-            __syncthreads();
-        }
         T2 = radix_select(n, key2, a.id, cand, n_pick - n1, hist, &sh_pk, &sh_pid, &sh_rem, &sh_done);
     }
 
@@ -140,21 +121,353 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan(BranchArgs a)
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        if (gridDim.x == 1) {
-            a.d_counts[0] = 2 * base_p;
-            a.d_counts[1] = base_r;
-            a.d_counts[2] = 2 * base_p + base_r;
-            a.poff[0] = 0;
-            a.poff[1] = 2 * base_p;
-            if (a.pcounts) {
-                a.pcounts[0] = base_p;
-                a.pcounts[1] = base_r;
-            }
-        } else {
-            a.pcounts[2 * pb] = base_p;
-            a.pcounts[2 * pb + 1] = base_r;
-        }
+        a.pcounts[2 * pb] = base_p;
+        a.pcounts[2 * pb + 1] = base_r;
     }
+}
+
+// ---------------------------------------------------------------------------
+// One problem
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void plan_totals(const BranchArgs &a, int picked, int rest)
+{
+    a.d_counts[0] = 2 * picked;
+    a.d_counts[1] = rest;
+    a.d_counts[2] = 2 * picked + rest;
+    a.poff[0] = 0;
+    a.poff[1] = 2 * picked;
+    if (a.pcounts) {
+        a.pcounts[0] = picked;
+        a.pcounts[1] = rest;
+    }
+}
+
+// At most kSmallPlan rows, one per thread: a row is among the k smallest composite keys when fewer than k candidates
+// have a smaller one, so each selection is one count over the rows (48 rows: 28 us by radix passes -> 5 us).
+constexpr int kSmallPlan = 256;
+
+__global__ void __launch_bounds__(kSmallPlan) k_branch_plan_small(BranchArgs a)
+{
+    __shared__ uint32_t key[kSmallPlan];
+    __shared__ uint64_t ids[kSmallPlan];
+    __shared__ int wsum[2][kSmallPlan / 32];
+    __shared__ float wmn[kSmallPlan / 32], wmx[kSmallPlan / 32];
+    const int n = live_count(a.n, a.d_n);
+    const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+    const bool row = i < n;
+    int n_pick, n1;
+    plan_quota(a, 0, n_pick, n1);
+    const float lb = row ? a.lb[i] : 0.f, ub = row ? a.ub[i] : 0.f;
+    const uint64_t id = row ? a.id[i] : 0;
+    if (row && lb != lb) set_status(a.status, BAB_ERR_NUMERIC);  // a NaN bound is kept and latched
+    const bool kp = row && !((double)lb > a.inc_val[0]);
+    if (row) a.keep[i] = kp;
+    const int ns = __syncthreads_count(kp);
+    bool pk = kp;
+    if (ns > n_pick) {
+        // among the rows flagged `in`, whether this one is one of the k smallest by (order(v), id)
+        auto smallest = [&](bool in, float v, int k) {
+            key[i] = float_order(v);
+            ids[i] = in ? id : 0;
+            const unsigned in_warp = __ballot_sync(0xFFFFFFFFu, in);
+            if (lane == 0) wsum[0][warp] = (int)in_warp;
+            __syncthreads();
+            int less = 0;
+            const uint32_t mk = key[i];
+            if (in && k > 0)
+                for (int j = 0; j < n; ++j)
+                    less += ((wsum[0][j >> 5] >> (j & 31)) & 1) && (key[j] < mk || (key[j] == mk && ids[j] < id));
+            __syncthreads();
+            return in && k > 0 && less < k;
+        };
+        const bool by_ub = smallest(kp, ub, n1);
+        const bool cand = kp && !by_ub;
+        float v2 = lb;
+        if (a.pick_rule == 1) {
+            // min-max scaling over the candidates' (non-NaN) lower bounds, then each candidate's race key
+            float mn = cand && lb == lb ? lb : INFINITY, mx = cand && lb == lb ? lb : -INFINITY;
+            for (int o = 16; o > 0; o >>= 1) {
+                mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
+                mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+            }
+            if (lane == 0) {
+                wmn[warp] = mn;
+                wmx[warp] = mx;
+            }
+            __syncthreads();
+            for (int w = 0; w < kSmallPlan / 32; ++w) {
+                mn = fminf(mn, wmn[w]);
+                mx = fmaxf(mx, wmx[w]);
+            }
+            if (cand && lb == lb) v2 = pick_key(lb, mn, mx, a.temperature, a.pick_seed, id);
+            if (cand) a.pick_keys[i] = v2;
+        }
+        const bool by_lb = smallest(cand, v2, n_pick - n1);
+        pk = by_ub || by_lb;
+    }
+    const bool rs = kp && !pk;
+    const unsigned lt = (1u << lane) - 1u;
+    const unsigned bp = __ballot_sync(0xFFFFFFFFu, pk), br = __ballot_sync(0xFFFFFFFFu, rs);
+    __syncthreads();
+    if (lane == 0) {
+        wsum[0][warp] = __popc(bp);
+        wsum[1][warp] = __popc(br);
+    }
+    __syncthreads();
+    int op = 0, orr = 0, tp = 0, tr = 0;
+    for (int w = 0; w < kSmallPlan / 32; ++w) {
+        if (w < warp) {
+            op += wsum[0][w];
+            orr += wsum[1][w];
+        }
+        tp += wsum[0][w];
+        tr += wsum[1][w];
+    }
+    if (row) a.dest[i] = pk ? ((op + __popc(bp & lt)) | kPickFlag) : rs ? orr + __popc(br & lt) : -1;
+    if (i == 0) plan_totals(a, tp, tr);
+}
+
+// A cluster of 1 to 8 CTAs, each with a contiguous share of the rows: the histograms of a radix pass are summed over the
+// CTAs' shared memory (distributed shared memory), one cluster barrier a pass, and every CTA finds the same digit; the
+// ranks start from the other CTAs' counts.  A pass stops the selection as soon as its digit's rows are all needed.
+// What bounds it is the latency of a pass (a read of the share from L2 and the barrier), not bytes: 60000 rows in one
+// CTA took 473 us.
+constexpr int kPlanCTAs = 8;
+
+struct PlanShared {
+    unsigned hist[2][256];
+    unsigned wtot[8];
+    int part[2][2];
+    float mn, mx;
+    int wsum[2][kPlanThreads / 32];
+    float wmn[kPlanThreads / 32], wmx[kPlanThreads / 32];
+    int digit, rem, done;
+};
+
+__global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    __shared__ PlanShared sh;
+    const int n = live_count(a.n, a.d_n), share = (n + C - 1) / C;
+    const int i0 = min(n, rank * share), i1 = min(n, i0 + share);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double inc = a.inc_val[0];
+    int n_pick, n1;
+    plan_quota(a, 0, n_pick, n1);
+    // the sum of a value over the block's threads (every thread gets it), then over the cluster
+    auto block_sum = [&](int v) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        if (lane == 0) sh.wsum[0][warp] = v;
+        __syncthreads();
+        int t = sh.wsum[0][lane];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        __syncthreads();
+        return t;
+    };
+
+    // prune (strict, in FP64; a NaN bound is kept and latched as BAB_ERR_NUMERIC)
+    int cnt = 0;
+#pragma unroll 4
+    for (int i = i0 + tid; i < i1; i += kPlanThreads) {
+        const float lbi = a.lb[i];
+        if (lbi != lbi) set_status(a.status, BAB_ERR_NUMERIC);
+        const uint8_t k = !((double)lbi > inc);
+        a.keep[i] = k;
+        cnt += k;
+    }
+    cnt = block_sum(cnt);
+    if (tid == 0) sh.part[0][0] = cnt;
+    cluster.sync();
+    int ns = 0;
+    for (int q = 0; q < C; ++q) ns += *cluster.map_shared_rank(&sh.part[0][0], q);
+
+    const bool all = ns <= n_pick;
+    Thresh T1, T2;
+    T1.none = T2.none = true;
+    const float *key2 = a.pick_rule == 1 ? a.pick_keys : a.lb;
+    int parity = 0;
+    // the kth smallest (1-based) composite key among the share's rows accepted by filt, over the whole cluster
+    auto select = [&](const float *val, auto filt, int kth) {
+        Thresh T;
+        T.none = kth <= 0;
+        T.key = 0;
+        T.id = 0;
+        if (T.none) return T;
+        int rem = kth;
+        for (int pass = 0; pass < 12; ++pass, parity ^= 1) {
+            unsigned *hist = sh.hist[parity];
+            if (tid < 256) hist[tid] = 0;
+            __syncthreads();
+            for (int b = i0; b < i1; b += kPlanThreads) {
+                const int i = b + tid;
+                bool in = i < i1 && filt(i);
+                uint32_t dg = 0;
+                if (in) {
+                    const uint32_t key = float_order(val[i]);
+                    const uint64_t id = a.id[i];
+                    in = prefix_match(key, id, T.key, T.id, pass);
+                    dg = digit_of(key, id, pass);
+                }
+                // (the leading digits of most rows agree: one addition for the warp then)
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+                if (m == 0) continue;
+                const int first = __ffs(m) - 1;
+                const uint32_t d0 = __shfl_sync(0xFFFFFFFFu, dg, first);
+                if (__all_sync(0xFFFFFFFFu, !in || dg == d0)) {
+                    if (lane == first) atomicAdd(&hist[d0], (unsigned)__popc(m));
+                } else if (in) {
+                    atomicAdd(&hist[dg], 1u);
+                }
+            }
+            cluster.sync();  // every CTA's histogram complete
+            unsigned h = 0, inclusive = 0;
+            if (tid < 256) {
+                for (int q = 0; q < C; ++q) h += cluster.map_shared_rank(hist, q)[tid];
+                inclusive = h;
+                for (int o = 1; o < 32; o *= 2) {
+                    const unsigned v = __shfl_up_sync(0xFFFFFFFFu, inclusive, o);
+                    if (lane >= o) inclusive += v;
+                }
+                if (lane == 31) sh.wtot[warp] = inclusive;
+            }
+            if (tid == 0) sh.digit = -1;
+            __syncthreads();
+            if (tid < 256) {
+                for (int w = 0; w < warp; ++w) inclusive += sh.wtot[w];
+                const bool here = inclusive >= (unsigned)rem && inclusive - h < (unsigned)rem;
+                const bool none = tid == 255 && inclusive < (unsigned)rem;  // fewer candidates than asked for: all
+                if (here || none) {
+                    sh.digit = tid;
+                    sh.rem = rem - (int)(none ? inclusive : inclusive - h);
+                    sh.done = here && h == (unsigned)(rem - (int)(inclusive - h));
+                }
+            }
+            __syncthreads();
+            const uint32_t D = (uint32_t)sh.digit;
+            rem = sh.rem;
+            const bool done = sh.done != 0;
+            if (pass < 4) T.key |= D << (24 - 8 * pass);
+            else T.id |= (uint64_t)D << (56 - 8 * (pass - 4));
+            if (done) {
+                // every row with this prefix is needed
+                if (pass < 4) {
+                    T.key |= pass == 3 ? 0u : 0xFFFFFFFFu >> (8 * (pass + 1));
+                    T.id = ~0ull;
+                } else if (pass < 11) {
+                    T.id |= ~0ull >> (8 * (pass - 3));
+                }
+                parity ^= 1;
+                break;
+            }
+        }
+        return T;
+    };
+    if (!all) {
+        const uint8_t *keep = a.keep;
+        const float *ub = a.ub;
+        const uint64_t *ids = a.id;
+        T1 = select(ub, [&](int i) { return keep[i] != 0; }, n1);
+        auto cand = [&](int i) { return keep[i] != 0 && !le_thresh(float_order(ub[i]), ids[i], T1); };
+        if (a.pick_rule == 1) {
+            // min-max scaling over the candidates' (non-NaN) lower bounds, then each candidate's race key
+            float mn = INFINITY, mx = -INFINITY;
+            for (int i = i0 + tid; i < i1; i += kPlanThreads)
+                if (cand(i) && a.lb[i] == a.lb[i]) {
+                    mn = fminf(mn, a.lb[i]);
+                    mx = fmaxf(mx, a.lb[i]);
+                }
+            for (int o = 16; o > 0; o >>= 1) {
+                mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
+                mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+            }
+            if (lane == 0) {
+                sh.wmn[warp] = mn;
+                sh.wmx[warp] = mx;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                for (int w = 1; w < kPlanThreads / 32; ++w) {
+                    mn = fminf(mn, sh.wmn[w]);
+                    mx = fmaxf(mx, sh.wmx[w]);
+                }
+                sh.mn = mn;
+                sh.mx = mx;
+            }
+            cluster.sync();
+            for (int q = 0; q < C; ++q) {
+                mn = q == 0 ? *cluster.map_shared_rank(&sh.mn, q) : fminf(mn, *cluster.map_shared_rank(&sh.mn, q));
+                mx = q == 0 ? *cluster.map_shared_rank(&sh.mx, q) : fmaxf(mx, *cluster.map_shared_rank(&sh.mx, q));
+            }
+            for (int i = i0 + tid; i < i1; i += kPlanThreads)
+                if (cand(i)) {
+                    const float v = a.lb[i];
+                    a.pick_keys[i] = v == v ? pick_key(v, mn, mx, a.temperature, a.pick_seed, ids[i]) : v;
+                }
+            __syncthreads();
+        }
+        T2 = select(key2, cand, n_pick - n1);
+    }
+
+    // stable ranks of picked and unpicked survivors: the share's counts, the shares before it, then row by row
+    auto flags = [&](int i, bool &pk, bool &rs) {
+        const bool kp = i < i1 && a.keep[i] != 0;
+        pk = kp && (all || le_thresh(float_order(a.ub[i]), a.id[i], T1) || le_thresh(float_order(key2[i]), a.id[i], T2));
+        rs = kp && !pk;
+    };
+    int cp = 0, cr = 0;
+    for (int i = i0 + tid; i < i1; i += kPlanThreads) {
+        bool pk, rs;
+        flags(i, pk, rs);
+        cp += pk;
+        cr += rs;
+    }
+    cp = block_sum(cp);
+    cr = block_sum(cr);
+    if (tid == 0) {
+        sh.part[1][0] = cp;
+        sh.part[1][1] = cr;
+    }
+    cluster.sync();
+    int base_p = 0, base_r = 0, tp = 0, tr = 0;
+    for (int q = 0; q < C; ++q) {
+        const int *o = cluster.map_shared_rank(&sh.part[1][0], q);
+        if (q < rank) {
+            base_p += o[0];
+            base_r += o[1];
+        }
+        tp += o[0];
+        tr += o[1];
+    }
+    const unsigned lt = (1u << lane) - 1u;
+    for (int b = i0; b < i1; b += kPlanThreads) {
+        const int i = b + tid;
+        bool pk, rs;
+        flags(i, pk, rs);
+        const unsigned bp = __ballot_sync(0xFFFFFFFFu, pk), br = __ballot_sync(0xFFFFFFFFu, rs);
+        if (lane == 0) {
+            sh.wsum[0][warp] = __popc(bp);
+            sh.wsum[1][warp] = __popc(br);
+        }
+        __syncthreads();
+        // warp prefix of the warps' counts
+        int vp = sh.wsum[0][lane], vr = sh.wsum[1][lane], ip = vp, ir = vr;
+        for (int o = 1; o < 32; o *= 2) {
+            const int xp = __shfl_up_sync(0xFFFFFFFFu, ip, o), xr = __shfl_up_sync(0xFFFFFFFFu, ir, o);
+            if (lane >= o) {
+                ip += xp;
+                ir += xr;
+            }
+        }
+        const int op = __shfl_sync(0xFFFFFFFFu, ip - vp, warp), orr = __shfl_sync(0xFFFFFFFFu, ir - vr, warp);
+        if (i < i1) a.dest[i] = pk ? ((base_p + op + __popc(bp & lt)) | kPickFlag) : rs ? base_r + orr + __popc(br & lt) : -1;
+        base_p += __shfl_sync(0xFFFFFFFFu, ip, 31);
+        base_r += __shfl_sync(0xFFFFFFFFu, ir, 31);
+        __syncthreads();
+    }
+    if (rank == 0 && tid == 0) plan_totals(a, tp, tr);
+    cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
 // Several problems: output offsets of each problem's children and unpicked rows, and the totals.
@@ -180,30 +493,61 @@ __global__ void k_branch_offsets(BranchArgs a)
     a.d_counts[2] = (int)(2 * tp + tr);
 }
 
-__global__ void k_branch_write(BranchArgs a)
+// VEC coordinates per lane (4: every row is 16-byte aligned), LPR lanes per row.
+template <int VEC, int LPR>
+__global__ void __launch_bounds__(256) k_branch_write(BranchArgs a)
 {
     const int n = live_count(a.n, a.d_n);
-    const int lane = threadIdx.x & 31;
-    const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x % LPR;
+    const int row = blockIdx.x * (256 / LPR) + threadIdx.x / LPR;
+    const unsigned group = LPR == 32 ? 0xFFFFFFFFu : ((1u << (LPR % 32)) - 1u) << ((threadIdx.x & 31) / LPR * LPR);
     if (row >= n) return;
+    const int d = a.d;
+    const float *lo = a.lo + (size_t)row * d, *hi = a.hi + (size_t)row * d;
+    // one row's coordinates j .. j + VEC - 1
+    struct Part {
+        float v[VEC];
+    };
+    auto load = [](const float *p) {
+        Part q;
+        if (VEC == 4) {
+            const float4 t = *reinterpret_cast<const float4 *>(p);
+            q.v[0] = t.x;
+            q.v[1 % VEC] = t.y;
+            q.v[2 % VEC] = t.z;
+            q.v[3 % VEC] = t.w;
+        } else {
+            q.v[0] = *p;
+        }
+        return q;
+    };
+    auto store = [](float *p, const Part &q) {
+        if (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(q.v[0], q.v[1 % VEC], q.v[2 % VEC], q.v[3 % VEC]);
+        else *p = q.v[0];
+    };
+    const int j0 = lane * VEC;
+    Part l0{}, h0{};
+    if (j0 < d) {
+        // (before the row's destination is known: few rows are pruned)
+        l0 = load(lo + j0);
+        h0 = load(hi + j0);
+    }
     const int dst = a.dest[row];
     if (dst < 0) return;
-    const int d = a.d;
     const int pb = row_problem(a.batch, row);
     const int dp = a.batch.H ? a.k * problem_H(a.batch, pb, 0) : d;  // coordinates the problem uses
-    const float *lo = a.lo + (size_t)row * d, *hi = a.hi + (size_t)row * d;
     const uint64_t id = a.id[row];
     if (!(dst & kPickFlag)) {
         const size_t o = (size_t)a.poff[2 * pb + 1] + dst;
         if (o >= (size_t)a.cap_out) return;
         if (a.out_prob && lane == 0) a.out_prob[o] = pb;
         if (a.out_split_dim && lane == 0) a.out_split_dim[o] = a.split_dim ? a.split_dim[row] : -1;
-        for (int j = lane; j < d; j += 32) {
-            a.out_lo[o * d + j] = lo[j];
-            a.out_hi[o * d + j] = hi[j];
+        for (int j = j0; j < d; j += LPR * VEC) {
+            store(a.out_lo + o * d + j, j == j0 ? l0 : load(lo + j));
+            store(a.out_hi + o * d + j, j == j0 ? h0 : load(hi + j));
         }
         if (a.out_row_u)
-            for (int j = lane; j < d; j += 32) a.out_row_u[o * d + j] = a.row_u[(size_t)row * d + j];
+            for (int j = j0; j < d; j += LPR * VEC) store(a.out_row_u + o * d + j, load(a.row_u + (size_t)row * d + j));
         if (lane == 0) {
             a.out_id[o] = id;
             a.out_lb[o] = a.lb[row];
@@ -215,16 +559,21 @@ __global__ void k_branch_write(BranchArgs a)
     float wb = -1.f;
     int jb = 0x7FFFFFFF;
     const int given = a.split_dim ? a.split_dim[row] : -1;  // the sample-imbalance choice, when given
-    for (int j = lane; j < dp && !(given >= 0 && given < dp); j += 32) {
-        const float w = __fsub_rn(hi[j], lo[j]);
-        if (w > wb) {
-            wb = w;
-            jb = j;
+    if (!(given >= 0 && given < dp))
+        for (int j = j0; j < dp; j += LPR * VEC) {
+            const Part l = j == j0 ? l0 : load(lo + j), h = j == j0 ? h0 : load(hi + j);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const float w = __fsub_rn(h.v[e], l.v[e]);
+                if (j + e < dp && w > wb) {
+                    wb = w;
+                    jb = j + e;
+                }
+            }
         }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const float w2 = __shfl_xor_sync(0xFFFFFFFFu, wb, o);
-        const int j2 = __shfl_xor_sync(0xFFFFFFFFu, jb, o);
+    for (int o = LPR / 2; o > 0; o >>= 1) {
+        const float w2 = __shfl_xor_sync(group, wb, o);
+        const int j2 = __shfl_xor_sync(group, jb, o);
         if (w2 > wb || (w2 == wb && j2 < jb)) {
             wb = w2;
             jb = j2;
@@ -237,18 +586,22 @@ __global__ void k_branch_write(BranchArgs a)
     if (o0 + 1 >= (size_t)a.cap_out) return;
     if (a.out_prob && lane == 0) a.out_prob[o0] = a.out_prob[o0 + 1] = pb;
     if (a.out_split_dim && lane == 0) a.out_split_dim[o0] = a.out_split_dim[o0 + 1] = -1;
-    for (int j = lane; j < d; j += 32) {
-        const float l = lo[j], h = hi[j];
-        a.out_lo[o0 * d + j] = l;
-        a.out_hi[o0 * d + j] = (j == jb) ? mid : h;
-        a.out_lo[(o0 + 1) * d + j] = (j == jb) ? mid : l;
-        a.out_hi[(o0 + 1) * d + j] = h;
+    for (int j = j0; j < d; j += LPR * VEC) {
+        const Part l = j == j0 ? l0 : load(lo + j), h = j == j0 ? h0 : load(hi + j);
+        Part lm = l, hm = h;
+#pragma unroll
+        for (int e = 0; e < VEC; ++e)
+            if (j + e == jb) lm.v[e] = hm.v[e] = mid;
+        store(a.out_lo + o0 * d + j, l);
+        store(a.out_hi + o0 * d + j, hm);
+        store(a.out_lo + (o0 + 1) * d + j, lm);
+        store(a.out_hi + (o0 + 1) * d + j, h);
     }
     if (a.out_row_u)
-        for (int j = lane; j < d; j += 32) {
-            const float v = a.row_u[(size_t)row * d + j];
-            a.out_row_u[o0 * d + j] = v;
-            a.out_row_u[(o0 + 1) * d + j] = v;
+        for (int j = j0; j < d; j += LPR * VEC) {
+            const Part v = load(a.row_u + (size_t)row * d + j);
+            store(a.out_row_u + o0 * d + j, v);
+            store(a.out_row_u + (o0 + 1) * d + j, v);
         }
     if (lane == 0) {
         a.out_id[o0] = child_id(id, 0);
@@ -346,10 +699,40 @@ cudaError_t launch_split_dims(int d, const float *lo, const float *hi, const uin
 
 cudaError_t launch_prune_branch(const BranchArgs &a, cudaStream_t st)
 {
-    const int P = a.batch.P > 1 ? a.batch.P : 1;
-    k_branch_plan<<<P, kPlanThreads, 0, st>>>(a);
-    if (P > 1) k_branch_offsets<<<1, 32, 0, st>>>(a);
-    if (a.n > 0) k_branch_write<<<(a.n + 7) / 8, 256, 0, st>>>(a);
+    if (a.batch.P > 1) {
+        k_branch_plan<<<a.batch.P, kPlanThreads, 0, st>>>(a);
+        k_branch_offsets<<<1, 32, 0, st>>>(a);
+    } else if (a.n <= kSmallPlan) {
+        k_branch_plan_small<<<1, kSmallPlan, 0, st>>>(a);
+    } else {
+        // a CTA per 2048 rows (two a thread), at most kPlanCTAs
+        int C = 1;
+        while (C < kPlanCTAs && C * 2 * kPlanThreads < a.n) C *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)C);
+        cfg.blockDim = dim3(kPlanThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)C;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaError_t e = cudaLaunchKernelEx(&cfg, k_branch_plan_cl, a);
+        if (e != cudaSuccess) return e;
+    }
+    if (a.n > 0) {
+        // rows of whole, aligned 16-byte words: the fewest lanes (8, 16 or 32) that take a row in one pass; else a warp a
+        // row, a coordinate a lane
+        auto al = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
+        const bool vec = a.d % 4 == 0 && al(a.lo) && al(a.hi) && al(a.out_lo) && al(a.out_hi) && al(a.row_u) && al(a.out_row_u);
+        auto run = [&](auto kern, int lpr) { kern<<<(a.n + 256 / lpr - 1) / (256 / lpr), 256, 0, st>>>(a); };
+        if (!vec) run(k_branch_write<1, 32>, 32);
+        else if (a.d <= 32) run(k_branch_write<4, 8>, 8);
+        else if (a.d <= 64) run(k_branch_write<4, 16>, 16);
+        else run(k_branch_write<4, 32>, 32);
+    }
     return cudaGetLastError();
 }
 
