@@ -230,9 +230,10 @@ __global__ void __launch_bounds__(kSmallPlan) k_branch_plan_small(BranchArgs a)
 // A cluster of 1 to 8 CTAs, each with a contiguous share of the rows: the histograms of a radix pass are summed over the
 // CTAs' shared memory (distributed shared memory), one cluster barrier a pass, and every CTA finds the same digit; the
 // ranks start from the other CTAs' counts.  A pass stops the selection as soon as its digit's rows are all needed.
-// What bounds it is the latency of a pass (a read of the share from L2 and the barrier), not bytes: 60000 rows in one
-// CTA took 473 us.
+// What bounds it is the latency of a pass, not bytes: 60000 rows took one CTA 473 us, the cluster 84 us reading its share
+// again in every pass and 51 us with the rows in registers (at most kPlanItems a thread).
 constexpr int kPlanCTAs = 8;
+constexpr int kPlanItems = 8;  // rows a thread keeps in registers
 
 struct PlanShared {
     unsigned hist[2][256];
@@ -244,6 +245,9 @@ struct PlanShared {
     int digit, rem, done;
 };
 
+// ITEMS > 0: the share is at most ITEMS rows a thread, their keys and identifiers loaded once and kept in registers;
+// 0: any share, read again in every pass.
+template <int ITEMS>
 __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
 {
     namespace cg = cooperative_groups;
@@ -256,7 +260,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
     const double inc = a.inc_val[0];
     int n_pick, n1;
     plan_quota(a, 0, n_pick, n1);
-    // the sum of a value over the block's threads (every thread gets it), then over the cluster
+    // the sum of a value over the block's threads (every thread gets it)
     auto block_sum = [&](int v) {
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
         if (lane == 0) sh.wsum[0][warp] = v;
@@ -267,16 +271,69 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         return t;
     };
 
+    // A row's order-preserving keys of ub and of lb (or its race key), its identifier and whether it survives; row it of
+    // this thread is i0 + it * kPlanThreads + tid.
+    struct Row {
+        uint32_t ub, v2;
+        uint64_t id;
+        bool kept;
+    };
+    constexpr int R = ITEMS > 0 ? ITEMS : 1;
+    uint32_t r_ub[R], r_v2[R], r_kept = 0;
+    uint64_t r_id[R];
     // prune (strict, in FP64; a NaN bound is kept and latched as BAB_ERR_NUMERIC)
-    int cnt = 0;
-#pragma unroll 4
-    for (int i = i0 + tid; i < i1; i += kPlanThreads) {
-        const float lbi = a.lb[i];
+    auto prune = [&](int i, float lbi) {
         if (lbi != lbi) set_status(a.status, BAB_ERR_NUMERIC);
-        const uint8_t k = !((double)lbi > inc);
+        const bool k = !((double)lbi > inc);
         a.keep[i] = k;
-        cnt += k;
+        return k;
+    };
+    int cnt = 0;
+    if (ITEMS > 0) {
+        float v[R];
+#pragma unroll
+        for (int it = 0; it < R; ++it) {
+            const int i = i0 + it * kPlanThreads + tid;
+            v[it] = i < i1 ? a.lb[i] : 0.f;
+            r_ub[it] = i < i1 ? float_order(a.ub[i]) : 0u;
+            r_id[it] = i < i1 ? a.id[i] : 0ull;
+        }
+#pragma unroll
+        for (int it = 0; it < R; ++it) {
+            const int i = i0 + it * kPlanThreads + tid;
+            r_v2[it] = float_order(v[it]);
+            if (i < i1 && prune(i, v[it])) {
+                r_kept |= 1u << it;
+                ++cnt;
+            }
+        }
+    } else {
+        for (int i = i0 + tid; i < i1; i += kPlanThreads) cnt += prune(i, a.lb[i]);
     }
+    bool race = false;  // v2 is the race key from here on
+    // every row of the share in turn, all threads of the block together: f(row's index, its data); kept is false beyond
+    // the share
+    auto each = [&](auto f) {
+        if (ITEMS > 0) {
+#pragma unroll
+            for (int it = 0; it < R; ++it) {
+                if (it * kPlanThreads >= i1 - i0) break;  // (the same for the whole block)
+                Row r{r_ub[it], r_v2[it], r_id[it], ((r_kept >> it) & 1u) != 0};
+                f(i0 + it * kPlanThreads + tid, it, r);
+            }
+        } else {
+            for (int b = i0; b < i1; b += kPlanThreads) {
+                const int i = b + tid;
+                Row r{0u, 0u, 0ull, i < i1 && a.keep[i] != 0};
+                if (r.kept) {
+                    r.ub = float_order(a.ub[i]);
+                    r.v2 = float_order(race ? a.pick_keys[i] : a.lb[i]);
+                    r.id = a.id[i];
+                }
+                f(i, 0, r);
+            }
+        }
+    };
     cnt = block_sum(cnt);
     if (tid == 0) sh.part[0][0] = cnt;
     cluster.sync();
@@ -286,10 +343,9 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
     const bool all = ns <= n_pick;
     Thresh T1, T2;
     T1.none = T2.none = true;
-    const float *key2 = a.pick_rule == 1 ? a.pick_keys : a.lb;
     int parity = 0;
-    // the kth smallest (1-based) composite key among the share's rows accepted by filt, over the whole cluster
-    auto select = [&](const float *val, auto filt, int kth) {
+    // the kth smallest (1-based) composite key (key(row), id) among the rows accepted by filt, over the whole cluster
+    auto select = [&](auto key_of, auto filt, int kth) {
         Thresh T;
         T.none = kth <= 0;
         T.key = 0;
@@ -300,19 +356,13 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
             unsigned *hist = sh.hist[parity];
             if (tid < 256) hist[tid] = 0;
             __syncthreads();
-            for (int b = i0; b < i1; b += kPlanThreads) {
-                const int i = b + tid;
-                bool in = i < i1 && filt(i);
-                uint32_t dg = 0;
-                if (in) {
-                    const uint32_t key = float_order(val[i]);
-                    const uint64_t id = a.id[i];
-                    in = prefix_match(key, id, T.key, T.id, pass);
-                    dg = digit_of(key, id, pass);
-                }
+            each([&](int, int, const Row &r) {
+                const uint32_t key = key_of(r);
+                const bool in = filt(r) && prefix_match(key, r.id, T.key, T.id, pass);
+                const uint32_t dg = digit_of(key, r.id, pass);
                 // (the leading digits of most rows agree: one addition for the warp then)
                 const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
-                if (m == 0) continue;
+                if (m == 0) return;
                 const int first = __ffs(m) - 1;
                 const uint32_t d0 = __shfl_sync(0xFFFFFFFFu, dg, first);
                 if (__all_sync(0xFFFFFFFFu, !in || dg == d0)) {
@@ -320,11 +370,13 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
                 } else if (in) {
                     atomicAdd(&hist[dg], 1u);
                 }
-            }
+            });
             cluster.sync();  // every CTA's histogram complete
             unsigned h = 0, inclusive = 0;
             if (tid < 256) {
-                for (int q = 0; q < C; ++q) h += cluster.map_shared_rank(hist, q)[tid];
+#pragma unroll
+                for (int q = 0; q < kPlanCTAs; ++q)
+                    if (q < C) h += cluster.map_shared_rank(hist, q)[tid];
                 inclusive = h;
                 for (int o = 1; o < 32; o *= 2) {
                     const unsigned v = __shfl_up_sync(0xFFFFFFFFu, inclusive, o);
@@ -332,7 +384,6 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
                 }
                 if (lane == 31) sh.wtot[warp] = inclusive;
             }
-            if (tid == 0) sh.digit = -1;
             __syncthreads();
             if (tid < 256) {
                 for (int w = 0; w < warp; ++w) inclusive += sh.wtot[w];
@@ -365,19 +416,18 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         return T;
     };
     if (!all) {
-        const uint8_t *keep = a.keep;
-        const float *ub = a.ub;
-        const uint64_t *ids = a.id;
-        T1 = select(ub, [&](int i) { return keep[i] != 0; }, n1);
-        auto cand = [&](int i) { return keep[i] != 0 && !le_thresh(float_order(ub[i]), ids[i], T1); };
+        T1 = select([](const Row &r) { return r.ub; }, [](const Row &r) { return r.kept; }, n1);
+        auto cand = [&](const Row &r) { return r.kept && !le_thresh(r.ub, r.id, T1); };
         if (a.pick_rule == 1) {
             // min-max scaling over the candidates' (non-NaN) lower bounds, then each candidate's race key
             float mn = INFINITY, mx = -INFINITY;
-            for (int i = i0 + tid; i < i1; i += kPlanThreads)
-                if (cand(i) && a.lb[i] == a.lb[i]) {
-                    mn = fminf(mn, a.lb[i]);
-                    mx = fmaxf(mx, a.lb[i]);
+            each([&](int, int, const Row &r) {
+                const float v = float_unorder(r.v2);
+                if (cand(r) && v == v) {
+                    mn = fminf(mn, v);
+                    mx = fmaxf(mx, v);
                 }
+            });
             for (int o = 16; o > 0; o >>= 1) {
                 mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
                 mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
@@ -396,33 +446,33 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
                 sh.mx = mx;
             }
             cluster.sync();
+            mn = INFINITY;
+            mx = -INFINITY;
             for (int q = 0; q < C; ++q) {
-                mn = q == 0 ? *cluster.map_shared_rank(&sh.mn, q) : fminf(mn, *cluster.map_shared_rank(&sh.mn, q));
-                mx = q == 0 ? *cluster.map_shared_rank(&sh.mx, q) : fmaxf(mx, *cluster.map_shared_rank(&sh.mx, q));
+                mn = fminf(mn, *cluster.map_shared_rank(&sh.mn, q));
+                mx = fmaxf(mx, *cluster.map_shared_rank(&sh.mx, q));
             }
-            for (int i = i0 + tid; i < i1; i += kPlanThreads)
-                if (cand(i)) {
-                    const float v = a.lb[i];
-                    a.pick_keys[i] = v == v ? pick_key(v, mn, mx, a.temperature, a.pick_seed, ids[i]) : v;
-                }
+            each([&](int i, int it, const Row &r) {
+                if (!cand(r)) return;
+                float v = float_unorder(r.v2);
+                v = v == v ? pick_key(v, mn, mx, a.temperature, a.pick_seed, r.id) : v;
+                a.pick_keys[i] = v;
+                if (ITEMS > 0) r_v2[it] = float_order(v);
+            });
+            race = true;
             __syncthreads();
         }
-        T2 = select(key2, cand, n_pick - n1);
+        T2 = select([](const Row &r) { return r.v2; }, cand, n_pick - n1);
     }
 
     // stable ranks of picked and unpicked survivors: the share's counts, the shares before it, then row by row
-    auto flags = [&](int i, bool &pk, bool &rs) {
-        const bool kp = i < i1 && a.keep[i] != 0;
-        pk = kp && (all || le_thresh(float_order(a.ub[i]), a.id[i], T1) || le_thresh(float_order(key2[i]), a.id[i], T2));
-        rs = kp && !pk;
-    };
+    auto picked = [&](const Row &r) { return r.kept && (all || le_thresh(r.ub, r.id, T1) || le_thresh(r.v2, r.id, T2)); };
     int cp = 0, cr = 0;
-    for (int i = i0 + tid; i < i1; i += kPlanThreads) {
-        bool pk, rs;
-        flags(i, pk, rs);
+    each([&](int, int, const Row &r) {
+        const bool pk = picked(r);
         cp += pk;
-        cr += rs;
-    }
+        cr += r.kept && !pk;
+    });
     cp = block_sum(cp);
     cr = block_sum(cr);
     if (tid == 0) {
@@ -441,10 +491,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         tr += o[1];
     }
     const unsigned lt = (1u << lane) - 1u;
-    for (int b = i0; b < i1; b += kPlanThreads) {
-        const int i = b + tid;
-        bool pk, rs;
-        flags(i, pk, rs);
+    each([&](int i, int, const Row &r) {
+        const bool pk = picked(r), rs = r.kept && !pk;
         const unsigned bp = __ballot_sync(0xFFFFFFFFu, pk), br = __ballot_sync(0xFFFFFFFFu, rs);
         if (lane == 0) {
             sh.wsum[0][warp] = __popc(bp);
@@ -452,7 +500,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         }
         __syncthreads();
         // warp prefix of the warps' counts
-        int vp = sh.wsum[0][lane], vr = sh.wsum[1][lane], ip = vp, ir = vr;
+        const int vp = sh.wsum[0][lane], vr = sh.wsum[1][lane];
+        int ip = vp, ir = vr;
         for (int o = 1; o < 32; o *= 2) {
             const int xp = __shfl_up_sync(0xFFFFFFFFu, ip, o), xr = __shfl_up_sync(0xFFFFFFFFu, ir, o);
             if (lane >= o) {
@@ -465,7 +514,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         base_p += __shfl_sync(0xFFFFFFFFu, ip, 31);
         base_r += __shfl_sync(0xFFFFFFFFu, ir, 31);
         __syncthreads();
-    }
+    });
     if (rank == 0 && tid == 0) plan_totals(a, tp, tr);
     cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
@@ -719,7 +768,8 @@ cudaError_t launch_prune_branch(const BranchArgs &a, cudaStream_t st)
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, k_branch_plan_cl, a);
+        cudaError_t e = a.n <= C * kPlanItems * kPlanThreads ? cudaLaunchKernelEx(&cfg, k_branch_plan_cl<kPlanItems>, a)
+                                                             : cudaLaunchKernelEx(&cfg, k_branch_plan_cl<0>, a);
         if (e != cudaSuccess) return e;
     }
     if (a.n > 0) {

@@ -22,9 +22,11 @@ def _pool(n, d, seed, ties, nan):
     return lo, hi, ids[np.random.default_rng(seed).permutation(n)], lb, ub
 
 
-@pytest.mark.parametrize("n", [1, 33, 256, 257, 2048, 2049, 5000, 17000])
+@pytest.mark.parametrize("n", [1, 33, 256, 257, 2048, 2049, 5000, 17000, 66000])
 @pytest.mark.parametrize("d", [1, 10, 32, 40, 68, 132])
 def test_plan_and_write(oracle, gp, n, d):
+    if n > 60000 and d != 10:
+        pytest.skip("the share that is read again in every pass: once")
     g = gp(W.config_problem("tiny"))
     ties, nan = (0.6, 0.02) if n % 2 else (0.0, 0.0)
     lo, hi, ids, lb, ub = _pool(n, d, n + d, ties, nan)
@@ -38,7 +40,7 @@ def test_plan_and_write(oracle, gp, n, d):
             assert np.array_equal(r[key], np.asarray(o[key]), equal_nan=key in ("lb", "ub"))
 
 
-@pytest.mark.parametrize("n", [100, 3000, 9000])
+@pytest.mark.parametrize("n", [100, 3000, 9000, 70000])
 def test_softmax_pick(oracle, gp, n):
     from paper_2412_09584_gb300 import binding as B
     from gpu_util import DEV, T, ids_t
