@@ -750,33 +750,39 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
     Ab[1] = p; p += RBT * ld;
     float *lam = p; p += RBT * s4;
     float *mu = p; p += RBT * d4;
-    float *cst = p; p += RBT;
-    float *mg = p; p += RBT;
     float *Pu = p; p += 4 * RBT;  // obstacle cost: per row the pusher coefficient of the actions (2) and its |sum| (2)
     const int lane = tid & 31, warp = tid >> 5;
     const bool obst = a.cost.kind == 1;
     const bool has_alpha = v.alpha != nullptr;
     const int ts = a.t_stop;              // early stop: propagate back to x_ts only
     const bool with_margin = v.S != nullptr;
+    // A warp's rows (warp, warp + NTT / 32, ..): each lane sums its own constant terms (rounded down) and margin terms
+    // (rounded up) of a row over all steps and layers; the lanes are added once at the end.
+    constexpr int NW = NTT / 32, RW = (RBT + NW - 1) / NW;
+    float cl[RW], ml[RW];
+#pragma unroll
+    for (int i = 0; i < RW; ++i) cl[i] = ml[i] = 0.f;
 
     // early stop: the cost terms at steps 1 .. ts on their intervals, no coefficient of u before ts
     if (ts > 0) {
         for (int i = tid; i < RBT * d4; i += NTT) mu[i] = 0.f;
-        for (int r = warp; r < RBT; r += NTT / 32) {
-            float c = 0.f;
-            if (r < nrows)
-                for (int q = lane; q < ts * s; q += 32) {
-                    const int t = 1 + q / s, i = q % s;
-                    const float g = a.goal[i];
-                    const size_t xi = ((size_t)r * (H + 1) + t) * s + i;
-                    c = __fadd_rd(c, sq_min_rd(__fsub_rd(v.x_lo[xi], g), __fsub_ru(v.x_hi[xi], g)));
-                }
-            c = warp_sum_rd(c);
-            if (lane == 0) cst[r] = c;
+#pragma unroll
+        for (int ri = 0; ri < RW; ++ri) {
+            const int r = warp + ri * NW;
+            if (r >= nrows) break;
+            for (int q = lane; q < ts * s; q += 32) {
+                const int t = 1 + q / s, i = q % s;
+                const float g = a.goal[i];
+                const size_t xi = ((size_t)r * (H + 1) + t) * s + i;
+                cl[ri] = __fadd_rd(cl[ri], sq_min_rd(__fsub_rd(v.x_lo[xi], g), __fsub_ru(v.x_hi[xi], g)));
+            }
         }
     }
     // tangent of ||x_H - g||^2: coefficient 2m, constant -(2 m g + m^2)
-    for (int r = warp; r < RBT; r += NTT / 32) {
+#pragma unroll
+    for (int ri = 0; ri < RW; ++ri) {
+        const int r = warp + ri * NW;
+        if (r >= RBT) break;
         if (obst) {
             // the obstacle cost at step H: its linear lower bound on x_H, and the pusher penalties at H
             float aa = 0.f, c = 0.f;
@@ -789,12 +795,10 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 Pu[4 * r] = Pu[4 * r + 1] = Pu[4 * r + 2] = Pu[4 * r + 3] = 0.f;
                 if (r < nrows) c = __fadd_rd(c, pusher_lin(a.cost, H, k, v.lo + (size_t)r * d, v.hi + (size_t)r * d,
                                                            Pu + 4 * r, Pu + 4 * r + 2));
-                cst[r] = c;
-                mg[r] = 0.f;
+                cl[ri] = __fadd_rd(cl[ri], c);
             }
             continue;
         }
-        float c = 0.f;
         for (int i = lane; i < s; i += 32) {
             float aa = 0.f;
             if (r < nrows && H > ts) {
@@ -803,14 +807,9 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 const float Ls = __fsub_rd(v.x_lo[xi], g), Us = __fsub_ru(v.x_hi[xi], g);
                 const float m = 0.5f * (Ls + Us);
                 aa = 2.f * m;
-                c = __fadd_rd(c, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
+                cl[ri] = __fadd_rd(cl[ri], __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
             }
             lam[r * s4 + i] = aa;
-        }
-        c = warp_sum_rd(c);
-        if (lane == 0) {
-            cst[r] = ts > 0 ? __fadd_rd(cst[r], c) : c;
-            mg[r] = 0.f;
         }
     }
     group_barrier(grp, NTT);
@@ -820,71 +819,84 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
         {
             const int NpL = pad4(N.dims[L]);
             const float *bL = img + N.bwd_b[L];
-            for (int r = warp; r < RBT; r += NTT / 32) {
-                float c = 0.f, e = 0.f;
+#pragma unroll
+            for (int ri = 0; ri < RW; ++ri) {
+                const int r = warp + ri * NW;
+                if (r >= RBT) break;
+                float e = 0.f;
                 for (int q = lane; q < NpL; q += 32) {
                     const float A = q < s ? lam[r * s4 + q] : 0.f;
                     Ab[0][r * ld + q] = A;
                     if (q < s && r < nrows) {
-                        c = __fmaf_rd(A, bL[q], c);
+                        cl[ri] = __fmaf_rd(A, bL[q], cl[ri]);
                         if (with_margin) e = __fmaf_ru(fabsf(A), v.S[((size_t)r * H + t) * sw + sumh + q], e);
                     }
                 }
-                c = warp_sum_rd(c);
-                e = warp_sum_ru(e);
-                if (lane == 0) {
-                    cst[r] = __fadd_rd(cst[r], c);
-                    mg[r] = __fmaf_ru(N.gam[L], e, mg[r]);
-                }
+                ml[ri] = __fmaf_ru(N.gam[L], e, ml[ri]);
             }
             group_barrier(grp, NTT);
-            dense_rows_auto<RBT, NTT>(Ab[0], ld, img + N.bwd_w[L], nullptr, NpL, pad4(N.dims[L - 1]), Ab[1], ld, false, tid);
+            dense_rows_auto<RBT, NTT>(Ab[0], ld, img + N.bwd_w[L], nullptr, NpL, pad4(N.dims[L - 1]), Ab[1], ld, false,
+                                      tid);
             group_barrier(grp, NTT);
         }
         int cur = 1;
         for (int l = L - 1; l >= 1; --l) {
             const int dl = N.dims[l], Npl = pad4(dl);
             const float *bl = img + N.bwd_b[l];
-            for (int r = warp; r < RBT; r += NTT / 32) {
-                float c = 0.f, eg = 0.f, er = 0.f;
-                if (r < nrows) {
-                    const size_t base = ((size_t)r * H + t);
-                    for (int q = lane; q < dl; q += 32) {
-                        const size_t idx = base * sumh + N.hoff[l] + q;
-                        const float zl = v.pre_lo[idx], zu = v.pre_hi[idx];
+#pragma unroll
+            for (int ri = 0; ri < RW; ++ri) {
+                const int r = warp + ri * NW;
+                if (r >= RBT) break;
+                if (r >= nrows) {
+                    for (int q = lane; q < dl; q += 32) Ab[cur][r * ld + q] = 0.f;
+                    continue;
+                }
+                const size_t base = ((size_t)r * H + t), row = base * sumh + N.hoff[l], srow = base * sw + N.hoff[l];
+                float eg = 0.f, er = 0.f;
+                // four of the lane's neurons at a time: their intervals, margin helpers and slopes loaded together
+                for (int q0 = lane; q0 < dl; q0 += 128) {
+                    float zl[4], zu[4], sv[4], al[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int q = q0 + 32 * e;
+                        const bool in = q < dl;
+                        zl[e] = in ? v.pre_lo[row + q] : 0.f;
+                        zu[e] = in ? v.pre_hi[row + q] : 0.f;
+                        sv[e] = in && with_margin ? v.S[srow + q] : 0.f;
+                        al[e] = in && has_alpha ? v.alpha[row + q] : 0.f;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int q = q0 + 32 * e;
+                        if (q >= dl) break;
                         const float A = Ab[cur][r * ld + q];
-                        if (v.A_pre) v.A_pre[idx] = A;
+                        if (v.A_pre) v.A_pre[row + q] = A;
                         float D, ci;
-                        relax_select(zl, zu, A, has_alpha ? v.alpha[idx] : 0.f, has_alpha, D, ci);
+                        relax_select(zl[e], zu[e], A, al[e], has_alpha, D, ci);
                         const float Ap = A * D;
                         Ab[cur][r * ld + q] = Ap;
-                        c = __fmaf_rd(A, ci, c);
-                        c = __fmaf_rd(Ap, bl[q], c);
+                        cl[ri] = __fmaf_rd(A, ci, cl[ri]);
+                        cl[ri] = __fmaf_rd(Ap, bl[q], cl[ri]);
                         if (with_margin) {
-                            eg = __fmaf_ru(fabsf(Ap), v.S[base * sw + N.hoff[l] + q], eg);
-                            if (D != 0.f && D != 1.f) er = __fmaf_ru(fabsf(Ap), fmaxf(-zl, zu), er);
+                            eg = __fmaf_ru(fabsf(Ap), sv[e], eg);
+                            if (D != 0.f && D != 1.f) er = __fmaf_ru(fabsf(Ap), fmaxf(-zl[e], zu[e]), er);
                         }
                     }
-                } else {
-                    for (int q = lane; q < dl; q += 32) Ab[cur][r * ld + q] = 0.f;
                 }
-                c = warp_sum_rd(c);
-                eg = warp_sum_ru(eg);
-                er = warp_sum_ru(er);
-                if (lane == 0) {
-                    cst[r] = __fadd_rd(cst[r], c);
-                    mg[r] = __fadd_ru(mg[r], __fmaf_ru(N.gam[l], eg, __fmul_ru(kTwoU, er)));
-                }
+                ml[ri] = __fadd_ru(ml[ri], __fmaf_ru(N.gam[l], eg, __fmul_ru(kTwoU, er)));
             }
             group_barrier(grp, NTT);
-            dense_rows_auto<RBT, NTT>(Ab[cur], ld, img + N.bwd_w[l], nullptr, Npl, pad4(N.dims[l - 1]), Ab[cur ^ 1],
-                                      ld, false, tid);
+            dense_rows_auto<RBT, NTT>(Ab[cur], ld, img + N.bwd_w[l], nullptr, Npl, pad4(N.dims[l - 1]), Ab[cur ^ 1], ld,
+                                      false, tid);
             group_barrier(grp, NTT);
             cur ^= 1;
         }
         // A is on [x_t | u_t]: mu_t = A_u; lam <- lam + A_x (+ tangent of ||x_t - g||^2 for t >= 1)
-        for (int r = warp; r < RBT; r += NTT / 32) {
-            float c = 0.f, e = 0.f;
+#pragma unroll
+        for (int ri = 0; ri < RW; ++ri) {
+            const int r = warp + ri * NW;
+            if (r >= RBT) break;
+            float e = 0.f;
             if (obst) {
                 // mu_t = A_u + the pusher coefficient of the later steps; its rounding (H additions) in the margin
                 const float *lo_r = v.lo + (size_t)r * d, *hi_r = v.hi + (size_t)r * d;
@@ -897,7 +909,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                         e = __fmaf_ru(__fmul_ru(__fmul_ru((float)(H + 2), kTwoU), __fadd_ru(fabsf(Au), Pa)), um, e);
                     }
                 }
-                float aa = 0.f;
+                float aa = 0.f, c = 0.f;
                 if (t > ts && t >= 1 && r < nrows) {
                     const size_t xi = ((size_t)r * (H + 1) + t) * s;
                     c = obstacle_state_lin(a.cost, t, s, v.x_lo + xi, v.x_hi + xi, a.goal, lane, aa);
@@ -911,13 +923,13 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                     const float mag = __fadd_ru(__fadd_ru(fabsf(lo_), fabsf(Ax)), fabsf(aa));
                     if (with_margin) e = __fmaf_ru(__fmul_ru(kTwoU, mag), B, e);
                 }
-                e = warp_sum_ru(e);
                 if (lane == 0) {
                     if (t >= 1 && r < nrows)
                         c = __fadd_rd(c, pusher_lin(a.cost, t, k, lo_r, hi_r, Pu + 4 * r, Pu + 4 * r + 2));
-                    cst[r] = __fadd_rd(cst[r], c);
-                    mg[r] = __fadd_ru(mg[r], e);
+                    cl[ri] = __fadd_rd(cl[ri], c);
                 }
+                ml[ri] = __fadd_ru(ml[ri], e);
+                __syncwarp();
                 continue;
             }
             for (int j = lane; j < k; j += 32) mu[r * d4 + t * k + j] = Ab[cur][r * ld + s + j];
@@ -935,7 +947,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                         const float Ls = __fsub_rd(xl, g), Us = __fsub_ru(xu, g);
                         const float m = 0.5f * (Ls + Us);
                         aa = 2.f * m;
-                        c = __fadd_rd(c, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
+                        cl[ri] = __fadd_rd(cl[ri], __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
                     }
                 }
                 const float ln = (lo_ + Ax) + aa;
@@ -943,19 +955,17 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 const float mag = __fadd_ru(__fadd_ru(fabsf(lo_), fabsf(Ax)), fabsf(aa));
                 if (with_margin) e = __fmaf_ru(__fmul_ru(kTwoU, mag), B, e);
             }
-            c = warp_sum_rd(c);
-            e = warp_sum_ru(e);
-            if (lane == 0) {
-                cst[r] = __fadd_rd(cst[r], c);
-                mg[r] = __fadd_ru(mg[r], e);
-            }
+            ml[ri] = __fadd_ru(ml[ri], e);
         }
         group_barrier(grp, NTT);
     }
 
     // lam . x0, then Theorem 2 in box form: sum_j min_{u in [lo, hi]} mu_j u + rho u^2
-    for (int r = warp; r < nrows; r += NTT / 32) {
-        float c = 0.f, val = 0.f, e = 0.f;
+#pragma unroll
+    for (int ri = 0; ri < RW; ++ri) {
+        const int r = warp + ri * NW;
+        if (r >= nrows) break;
+        float c = cl[ri], val = 0.f, e = ml[ri];
         if (ts == 0) {
             for (int i = lane; i < s; i += 32) c = __fmaf_rd(lam[r * s4 + i], a.x0[i], c);
         } else {
@@ -966,7 +976,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 c = __fadd_rd(c, fminf(__fmul_rd(li, v.x_lo[xi]), __fmul_rd(li, v.x_hi[xi])));
             }
         }
-        c = __fadd_rd(cst[r], warp_sum_rd(c));
+        c = warp_sum_rd(c);
         for (int j = lane; j < d; j += 32) {
             const float m_ = mu[r * d4 + j];
             const float lo = v.lo[(size_t)r * d + j], hi = v.hi[(size_t)r * d + j];
@@ -996,10 +1006,9 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
         e = warp_sum_ru(e);
         if (lane == 0) {
             const float raw = __fadd_rd(c, val);
-            const float marg = __fadd_ru(mg[r], e);
-            const float lbv = __fsub_rd(raw, marg);
+            const float lbv = __fsub_rd(raw, e);
             v.lb[r] = lbv;
-            if (v.margin) v.margin[r] = marg;
+            if (v.margin) v.margin[r] = e;
             if (v.lin_const) v.lin_const[r] = c;
             if (v.lb_best) v.lb_best[r] = fmaxf(v.lb_best[r], lbv);
         }
@@ -1044,19 +1053,34 @@ __device__ void fwd_rows(const BoundArgs &a, const float *img, float *p, const R
             cur ^= 1;
             if (l < L) {
                 const int dl = N.dims[l];
-                for (int i = tid; i < RBT * dl; i += NTT) {
-                    const int r = i / dl, q = i % dl;
-                    if (r >= nrows) continue;
-                    const size_t idx = ((size_t)r * H + t) * sumh + N.hoff[l] + q;
-                    const float z = Z[cur][r * ld + q];
-                    const float zl = v.pre_lo[idx], zu = v.pre_hi[idx], A = v.A_pre[idx];
-                    float D, c;
-                    relax_select(zl, zu, A, has_alpha ? v.alpha[idx] : 0.f, has_alpha, D, c);
-                    const bool unstable = zl < 0.f && zu > 0.f;
-                    const float g = (unstable && A >= 0.f) ? A * z : 0.f;
-                    if (adam) adam_update(v.alpha[idx], v.adam_m[idx], v.adam_v[idx], g, *adam);
-                    else v.grad[idx] = g;
-                    Z[cur][r * ld + q] = fmaf(D, z, c);
+                // four neurons at a time, their loads together
+                for (int i0 = tid; i0 < nrows * dl; i0 += 4 * NTT) {
+                    float zl[4], zu[4], A[4], al[4];
+                    size_t idx[4];
+                    int at[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int i = i0 + e * NTT, r = i / dl, q = i - r * dl;
+                        idx[e] = ((size_t)r * H + t) * sumh + N.hoff[l] + q;
+                        at[e] = i < nrows * dl ? r * ld + q : -1;
+                        const bool in = at[e] >= 0;
+                        zl[e] = in ? v.pre_lo[idx[e]] : 0.f;
+                        zu[e] = in ? v.pre_hi[idx[e]] : 0.f;
+                        A[e] = in ? v.A_pre[idx[e]] : 0.f;
+                        al[e] = in && has_alpha ? v.alpha[idx[e]] : 0.f;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (at[e] < 0) break;
+                        const float z = Z[cur][at[e]];
+                        float D, c;
+                        relax_select(zl[e], zu[e], A[e], al[e], has_alpha, D, c);
+                        const bool unstable = zl[e] < 0.f && zu[e] > 0.f;
+                        const float g = (unstable && A[e] >= 0.f) ? A[e] * z : 0.f;
+                        if (adam) adam_update(v.alpha[idx[e]], v.adam_m[idx[e]], v.adam_v[idx[e]], g, *adam);
+                        else v.grad[idx[e]] = g;
+                        Z[cur][at[e]] = fmaf(D, z, c);
+                    }
                 }
                 group_barrier(grp, NTT);
             }
