@@ -1671,7 +1671,8 @@ int bab_bound_batch(bab_ctx *c, const float *x0, const float *goal, const int *h
     const size_t nh = (size_t)n * max_horizon * N.sumh, nx = (size_t)n * (max_horizon + 1) * N.s;
     const size_t ns = (size_t)n * max_horizon * (N.sumh + N.s);
     const size_t floats = 2 * nh + 2 * nx + ns + (alpha_steps > 0 ? 4 * nh : 0);
-    rc = ensure_scratch(c, floats * sizeof(float) + 16 * 256);
+    const size_t queue = batch_queue_ints(n, c->n_problems);
+    rc = ensure_scratch(c, floats * sizeof(float) + queue * sizeof(int) + 17 * 256);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     BoundArgs a = make_bound_args(c, x0, goal, max_horizon, 0.f, lo, hi, n, d_n);
@@ -1694,6 +1695,7 @@ int bab_bound_batch(bab_ctx *c, const float *x0, const float *goal, const int *h
         a.A_pre = cv.take<float>(nh);
     }
     a.lb_best = lb;
+    if (queue) a.queue = cv.take<int>(queue);
     e = launch_alpha_warp(a, alpha_steps, lr, al, m, v, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "batched bound kernel");
     return BAB_OK;

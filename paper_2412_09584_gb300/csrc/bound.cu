@@ -756,8 +756,10 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
     const bool has_alpha = v.alpha != nullptr;
     const int ts = a.t_stop;              // early stop: propagate back to x_ts only
     const bool with_margin = v.S != nullptr;
-    // A warp's rows (warp, warp + NTT / 32, ..): each lane sums its own constant terms (rounded down) and margin terms
-    // (rounded up) of a row over all steps and layers; the lanes are added once at the end.
+    // A warp's rows (warp, warp + NTT / 32, ..): a row's constant (rounded down; the same on every lane), summed over the
+    // lanes in every layer, and each lane's own margin terms (rounded up, all nonnegative), added over the lanes once at
+    // the end.  (The constant's terms have both signs: kept per lane too, 32 larger sums rounded in every layer, it came
+    // out up to 1.2 times further from the exact one.)
     constexpr int NW = NTT / 32, RW = (RBT + NW - 1) / NW;
     float cl[RW], ml[RW];
 #pragma unroll
@@ -770,12 +772,14 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
         for (int ri = 0; ri < RW; ++ri) {
             const int r = warp + ri * NW;
             if (r >= nrows) break;
+            float c = 0.f;
             for (int q = lane; q < ts * s; q += 32) {
                 const int t = 1 + q / s, i = q % s;
                 const float g = a.goal[i];
                 const size_t xi = ((size_t)r * (H + 1) + t) * s + i;
-                cl[ri] = __fadd_rd(cl[ri], sq_min_rd(__fsub_rd(v.x_lo[xi], g), __fsub_ru(v.x_hi[xi], g)));
+                c = __fadd_rd(c, sq_min_rd(__fsub_rd(v.x_lo[xi], g), __fsub_ru(v.x_hi[xi], g)));
             }
+            cl[ri] = warp_sum_rd(c);
         }
     }
     // tangent of ||x_H - g||^2: coefficient 2m, constant -(2 m g + m^2)
@@ -795,10 +799,11 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 Pu[4 * r] = Pu[4 * r + 1] = Pu[4 * r + 2] = Pu[4 * r + 3] = 0.f;
                 if (r < nrows) c = __fadd_rd(c, pusher_lin(a.cost, H, k, v.lo + (size_t)r * d, v.hi + (size_t)r * d,
                                                            Pu + 4 * r, Pu + 4 * r + 2));
-                cl[ri] = __fadd_rd(cl[ri], c);
             }
+            cl[ri] = __shfl_sync(0xFFFFFFFFu, c, 0);
             continue;
         }
+        float c = 0.f;
         for (int i = lane; i < s; i += 32) {
             float aa = 0.f;
             if (r < nrows && H > ts) {
@@ -807,10 +812,12 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 const float Ls = __fsub_rd(v.x_lo[xi], g), Us = __fsub_ru(v.x_hi[xi], g);
                 const float m = 0.5f * (Ls + Us);
                 aa = 2.f * m;
-                cl[ri] = __fadd_rd(cl[ri], __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
+                c = __fadd_rd(c, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
             }
             lam[r * s4 + i] = aa;
         }
+        c = warp_sum_rd(c);
+        cl[ri] = ts > 0 ? __fadd_rd(cl[ri], c) : c;
     }
     group_barrier(grp, NTT);
 
@@ -823,15 +830,16 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
             for (int ri = 0; ri < RW; ++ri) {
                 const int r = warp + ri * NW;
                 if (r >= RBT) break;
-                float e = 0.f;
+                float c = 0.f, e = 0.f;
                 for (int q = lane; q < NpL; q += 32) {
                     const float A = q < s ? lam[r * s4 + q] : 0.f;
                     Ab[0][r * ld + q] = A;
                     if (q < s && r < nrows) {
-                        cl[ri] = __fmaf_rd(A, bL[q], cl[ri]);
+                        c = __fmaf_rd(A, bL[q], c);
                         if (with_margin) e = __fmaf_ru(fabsf(A), v.S[((size_t)r * H + t) * sw + sumh + q], e);
                     }
                 }
+                cl[ri] = __fadd_rd(cl[ri], warp_sum_rd(c));
                 ml[ri] = __fmaf_ru(N.gam[L], e, ml[ri]);
             }
             group_barrier(grp, NTT);
@@ -852,7 +860,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                     continue;
                 }
                 const size_t base = ((size_t)r * H + t), row = base * sumh + N.hoff[l], srow = base * sw + N.hoff[l];
-                float eg = 0.f, er = 0.f;
+                float c = 0.f, eg = 0.f, er = 0.f;
                 // four of the lane's neurons at a time: their intervals, margin helpers and slopes loaded together
                 for (int q0 = lane; q0 < dl; q0 += 128) {
                     float zl[4], zu[4], sv[4], al[4];
@@ -875,14 +883,15 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                         relax_select(zl[e], zu[e], A, al[e], has_alpha, D, ci);
                         const float Ap = A * D;
                         Ab[cur][r * ld + q] = Ap;
-                        cl[ri] = __fmaf_rd(A, ci, cl[ri]);
-                        cl[ri] = __fmaf_rd(Ap, bl[q], cl[ri]);
+                        c = __fmaf_rd(A, ci, c);
+                        c = __fmaf_rd(Ap, bl[q], c);
                         if (with_margin) {
                             eg = __fmaf_ru(fabsf(Ap), sv[e], eg);
                             if (D != 0.f && D != 1.f) er = __fmaf_ru(fabsf(Ap), fmaxf(-zl[e], zu[e]), er);
                         }
                     }
                 }
+                cl[ri] = __fadd_rd(cl[ri], warp_sum_rd(c));
                 ml[ri] = __fadd_ru(ml[ri], __fmaf_ru(N.gam[l], eg, __fmul_ru(kTwoU, er)));
             }
             group_barrier(grp, NTT);
@@ -923,16 +932,15 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                     const float mag = __fadd_ru(__fadd_ru(fabsf(lo_), fabsf(Ax)), fabsf(aa));
                     if (with_margin) e = __fmaf_ru(__fmul_ru(kTwoU, mag), B, e);
                 }
-                if (lane == 0) {
-                    if (t >= 1 && r < nrows)
-                        c = __fadd_rd(c, pusher_lin(a.cost, t, k, lo_r, hi_r, Pu + 4 * r, Pu + 4 * r + 2));
-                    cl[ri] = __fadd_rd(cl[ri], c);
-                }
+                if (lane == 0 && t >= 1 && r < nrows)
+                    c = __fadd_rd(c, pusher_lin(a.cost, t, k, lo_r, hi_r, Pu + 4 * r, Pu + 4 * r + 2));
+                cl[ri] = __fadd_rd(cl[ri], __shfl_sync(0xFFFFFFFFu, c, 0));
                 ml[ri] = __fadd_ru(ml[ri], e);
                 __syncwarp();
                 continue;
             }
             for (int j = lane; j < k; j += 32) mu[r * d4 + t * k + j] = Ab[cur][r * ld + s + j];
+            float c = 0.f;
             for (int i = lane; i < s; i += 32) {
                 const float Ax = Ab[cur][r * ld + i];
                 const float lo_ = lam[r * s4 + i];
@@ -947,7 +955,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                         const float Ls = __fsub_rd(xl, g), Us = __fsub_ru(xu, g);
                         const float m = 0.5f * (Ls + Us);
                         aa = 2.f * m;
-                        cl[ri] = __fadd_rd(cl[ri], __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
+                        c = __fadd_rd(c, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
                     }
                 }
                 const float ln = (lo_ + Ax) + aa;
@@ -955,6 +963,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 const float mag = __fadd_ru(__fadd_ru(fabsf(lo_), fabsf(Ax)), fabsf(aa));
                 if (with_margin) e = __fmaf_ru(__fmul_ru(kTwoU, mag), B, e);
             }
+            cl[ri] = __fadd_rd(cl[ri], warp_sum_rd(c));
             ml[ri] = __fadd_ru(ml[ri], e);
         }
         group_barrier(grp, NTT);
@@ -965,7 +974,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
     for (int ri = 0; ri < RW; ++ri) {
         const int r = warp + ri * NW;
         if (r >= nrows) break;
-        float c = cl[ri], val = 0.f, e = ml[ri];
+        float c = 0.f, val = 0.f, e = ml[ri];
         if (ts == 0) {
             for (int i = lane; i < s; i += 32) c = __fmaf_rd(lam[r * s4 + i], a.x0[i], c);
         } else {
@@ -976,7 +985,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 c = __fadd_rd(c, fminf(__fmul_rd(li, v.x_lo[xi]), __fmul_rd(li, v.x_hi[xi])));
             }
         }
-        c = warp_sum_rd(c);
+        c = __fadd_rd(cl[ri], warp_sum_rd(c));
         for (int j = lane; j < d; j += 32) {
             const float m_ = mu[r * d4 + j];
             const float lo = v.lo[(size_t)r * d + j], hi = v.hi[(size_t)r * d + j];

@@ -127,6 +127,80 @@ __host__ __device__ inline RowsLayout rows_layout(const NetDesc &N)
 
 }  // namespace
 
+// The queue of a batch's alpha-CROWN: rounds of up to kWarps rows of one problem each, the problems of the longest
+// horizons first, so that the CTAs that take rounds from it finish together (with horizons of 10 to 80 and rounds dealt
+// out in row order, the CTAs that met long horizons twice set the time: 64 problems, 8889 rows, 20 steps 25.2 -> 13.6
+// ms).  queue: [0] the next round, [1] the number of rounds, then per round its first place in the permutation of rows
+// and its rows, then the permutation.  One CTA.
+constexpr int kQueueHead = 2, kQueueProblems = 2048;
+
+__host__ __device__ inline int batch_rounds_most(int n, int P) { return n / kWarps + P + 1; }
+
+__global__ void __launch_bounds__(1024) k_batch_rounds(BoundArgs a)
+{
+    extern __shared__ int bsm[];
+    const int P = a.batch.P, n = live_count(a.n, a.d_n, a.row0), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int *count = bsm, *order = bsm + P, *row_at = bsm + 2 * P;
+    __shared__ int wr[32], wq[32];
+    int *rounds = a.queue + kQueueHead, *perm = rounds + 2 * batch_rounds_most(a.n, P);
+    for (int p = tid; p < P; p += 1024) count[p] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += 1024) atomicAdd(&count[row_problem(a.batch, i)], 1);
+    // the problems by horizon, longest first
+    for (int p = tid; p < P; p += 1024) {
+        const int h = problem_H(a.batch, p, a.H);
+        int rank = 0;
+        for (int q = 0; q < P; ++q) {
+            const int g = problem_H(a.batch, q, a.H);
+            rank += g > h || (g == h && q < p);
+        }
+        order[rank] = p;
+    }
+    __syncthreads();
+    // first row and first round of every problem: each thread's problems, then the threads before it
+    const int per = (P + 1023) / 1024, p0 = min(P, tid * per), p1 = min(P, p0 + per);
+    int rows = 0, rnds = 0;
+    for (int e = p0; e < p1; ++e) {
+        rows += count[order[e]];
+        rnds += (count[order[e]] + kWarps - 1) / kWarps;
+    }
+    int ir = rows, iq = rnds;
+    for (int o = 1; o < 32; o *= 2) {
+        const int x = __shfl_up_sync(0xFFFFFFFFu, ir, o), y = __shfl_up_sync(0xFFFFFFFFu, iq, o);
+        if (lane >= o) {
+            ir += x;
+            iq += y;
+        }
+    }
+    if (lane == 31) {
+        wr[warp] = ir;
+        wq[warp] = iq;
+    }
+    __syncthreads();
+    int row = ir - rows, rnd = iq - rnds;
+    for (int w = 0; w < warp; ++w) {
+        row += wr[w];
+        rnd += wq[w];
+    }
+    for (int e = p0; e < p1; ++e) {
+        const int p = order[e], c = count[p];
+        row_at[p] = row;
+        for (int f = 0; f < c; f += kWarps, ++rnd) {
+            rounds[2 * rnd] = row + f;
+            rounds[2 * rnd + 1] = min(kWarps, c - f);
+        }
+        row += c;
+    }
+    if (tid == 1023) {
+        a.queue[0] = 0;
+        a.queue[1] = rnd;
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += 1024) perm[atomicAdd(&row_at[row_problem(a.batch, i)], 1)] = i;
+}
+
+size_t batch_queue_ints(int n, int P) { return P > 1 && P <= kQueueProblems ? kQueueHead + 2 * (size_t)batch_rounds_most(n, P) + n : 0; }
+
 // What bounds it: issue slots (about 1400 instructions a box and step) and the latency of the per-box arrays in L2; each
 // product is a third of them.  Adam's divisions of zeros (stable neurons, those whose coefficient never took the lower
 // line) went through their slow path and are skipped, the chord's slope goes to the adjoint in place of the coefficient.
@@ -136,7 +210,8 @@ __host__ __device__ inline RowsLayout rows_layout(const NetDesc &N)
 // from global memory with shuffle broadcasts (dense_warp).  Both sum in the same order.
 // OBST: the pushing-with-obstacles cost (a separate instance, so that the squared-distance kernel carries none of
 // its code or registers).
-template <int P, bool ROWS, bool OBST>
+// QUEUE: a batch's rounds come from its queue.
+template <int P, bool ROWS, bool OBST, bool QUEUE>
 __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
     k_alpha_warp(BoundArgs a, int steps, float lr, float *alpha_g, float *m_g, float *v_g, const AdamTable tab)
 {
@@ -159,9 +234,23 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
     const bool opt = steps > 0;           // steps == 0: one bound with the adaptive slopes, no adjoint
     constexpr bool obst = OBST;           // the pushing-with-obstacles cost (one problem, s <= 32)
     int loaded = -1;                      // the problem whose rows are in shared memory
-    for (int base = blockIdx.x * kWarps; base < nlive; base += gridDim.x * kWarps) {
-        // a round of kWarps boxes; the rows of its first box's problem serve every box of that problem
-        const int pr = row_problem(a.batch, base);
+    __shared__ int round_sh;
+    const int *rounds = QUEUE ? a.queue + kQueueHead : nullptr;
+    const int *perm = QUEUE ? rounds + 2 * batch_rounds_most(a.n, a.batch.P) : nullptr;
+    const int nrounds = QUEUE ? a.queue[1] : (nlive + kWarps - 1) / kWarps;
+    for (int round = blockIdx.x;; round += gridDim.x) {
+        // a round of up to kWarps boxes: of one problem, from the queue (longest horizons first); without a queue the
+        // next kWarps rows, and the rows of the first one's problem serve every box of that problem
+        if (QUEUE) {
+            __syncthreads();
+            if (threadIdx.x == 0) round_sh = atomicAdd(a.queue, 1);
+            __syncthreads();
+            round = round_sh;
+        }
+        if (round >= nrounds) break;
+        const int base = QUEUE ? rounds[2 * round] : round * kWarps;
+        const int count = QUEUE ? rounds[2 * round + 1] : min(kWarps, nlive - base);
+        const int pr = row_problem(a.batch, QUEUE ? perm[base] : base);
         if (ROWS && pr != loaded) {
             __syncthreads();
             const float *F = a.fwd + (size_t)pr * N.img_floats, *Bw = a.bwd + (size_t)pr * N.img_floats;
@@ -180,11 +269,11 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
             __syncthreads();
             loaded = pr;
         }
-        const int box = base + wib;
-        if (box >= nlive) continue;
+        if (wib >= count) continue;
+        const int box = QUEUE ? perm[base + wib] : base + wib;
         // the box's problem: weights, start, goal, horizon and rho
         const int pb = row_problem(a.batch, box);
-        const bool use_rows = ROWS && pb == loaded;
+        const bool use_rows = ROWS && (QUEUE || pb == loaded);
         const float *fwd = a.fwd + (size_t)pb * N.img_floats, *bwd = a.bwd + (size_t)pb * N.img_floats;
         // forward product of layer l: out[q] = b[q] + sum_c W[q][c] in[c]
         auto dense_f = [&](const float (&in)[P], int l, float (&out)[P]) {
@@ -233,10 +322,10 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
         float lb_best = -INFINITY;
         for (int step = 1; step <= (opt ? steps : 1); ++step) {
             // ------------------------------ bound (Theorems 1-2) ------------------------------
-            // Each lane sums its own constant terms (rounded down) and margin terms (rounded up) over all steps and
-            // layers, as crown_rows does; the lanes are added once at the end.
+            // The constant (rounded down) is summed over the lanes in every layer, the margin's terms (rounded up) stay on
+            // their lanes until the end, as in crown_rows.
             float A[P], lam[P], tmp[P];
-            float cst = 0.f, mg = 0.f;
+            float cst, mg = 0.f;
             // the pushing-with-obstacles cost: the pusher penalties' coefficient of every earlier action (2) and
             // the sum of its magnitudes (2), accumulated backward from step H (the same values on every lane)
             float Pu[4] = {0.f, 0.f, 0.f, 0.f};
@@ -247,9 +336,9 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                 float c = obstacle_state_lin(a.cost, H, s, xlo + (size_t)H * s, xhi + (size_t)H * s, goal, lane, aa);
 #pragma unroll
                 for (int q = 0; q < P; ++q) lam[q] = (q == 0 && lane < s) ? aa : 0.f;
-                c = __fadd_rd(c, pusher_lin(a.cost, H, k, blo, bhi, Pu, Pu + 2));
-                if (lane == 0) cst = __fadd_rd(cst, c);
+                cst = __fadd_rd(c, pusher_lin(a.cost, H, k, blo, bhi, Pu, Pu + 2));
             } else {
+                float c = 0.f;
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     const int i = lane + 32 * q;
@@ -259,26 +348,28 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                         const float Ls = __fsub_rd(xlo[(size_t)H * s + i], g), Us = __fsub_ru(xhi[(size_t)H * s + i], g);
                         const float m = 0.5f * (Ls + Us);
                         aa = 2.f * m;
-                        cst = __fadd_rd(cst, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
+                        c = __fadd_rd(c, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
                     }
                     lam[q] = aa;
                 }
+                cst = warp_sum_rd(c);
             }
             for (int t = H - 1; t >= 0; --t) {
                 {
                     const int NpL = pad4(N.dims[L]);
                     const float *bL = bwd + N.bwd_b[L];
-                    float e = 0.f;
+                    float c = 0.f, e = 0.f;
 #pragma unroll
                     for (int q = 0; q < P; ++q) {
                         const int i = lane + 32 * q;
                         const float Av = i < s ? lam[q] : 0.f;
                         A[q] = Av;
                         if (i < s) {
-                            cst = __fmaf_rd(Av, bL[i], cst);
+                            c = __fmaf_rd(Av, bL[i], c);
                             e = __fmaf_ru(fabsf(Av), S[(size_t)t * sw + sumh + i], e);
                         }
                     }
+                    cst = __fadd_rd(cst, warp_sum_rd(c));
                     mg = __fmaf_ru(N.gam[L], e, mg);
                     dense_b(A, L, tmp);
 #pragma unroll
@@ -287,7 +378,7 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                 for (int l = L - 1; l >= 1; --l) {
                     const int dl = N.dims[l];
                     const float *bl = bwd + N.bwd_b[l];
-                    float eg = 0.f, er = 0.f;
+                    float c = 0.f, eg = 0.f, er = 0.f;
 #pragma unroll
                     for (int q = 0; q < P; ++q) {
                         const int j = lane + 32 * q;
@@ -302,12 +393,13 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                             if (opt) Ap[idx] = (Av < 0.f && zl < 0.f && zu > 0.f) ? -D : Av;
                             const float Apj = Av * D;
                             A[q] = Apj;
-                            cst = __fmaf_rd(Av, ci, cst);
-                            cst = __fmaf_rd(Apj, bl[j], cst);
+                            c = __fmaf_rd(Av, ci, c);
+                            c = __fmaf_rd(Apj, bl[j], c);
                             eg = __fmaf_ru(fabsf(Apj), S[(size_t)t * sw + N.hoff[l] + j], eg);
                             if (D != 0.f && D != 1.f) er = __fmaf_ru(fabsf(Apj), fmaxf(-zl, zu), er);
                         }
                     }
+                    cst = __fadd_rd(cst, warp_sum_rd(c));
                     mg = __fadd_ru(mg, __fmaf_ru(N.gam[l], eg, __fmul_ru(kTwoU, er)));
                     dense_b(A, l, tmp);
 #pragma unroll
@@ -344,12 +436,12 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                         e = __fmaf_ru(__fmul_ru(kTwoU, mag), B, e);
                     }
                     if (t >= 1) c = __fadd_rd(c, pusher_lin(a.cost, t, k, blo, bhi, Pu, Pu + 2));
-                    if (lane == 0) cst = __fadd_rd(cst, c);
+                    cst = __fadd_rd(cst, c);
                     mg = __fadd_ru(mg, e);
                     continue;
                 }
                 // A is on [x_t | u_t]: mu_t = A_u; lam <- lam + A_x (+ tangent of ||x_t - g||^2 for t >= 1)
-                float e = 0.f;
+                float c = 0.f, e = 0.f;
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     const int i = lane + 32 * q;
@@ -363,7 +455,7 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                             const float Ls = __fsub_rd(xl, g), Us = __fsub_ru(xu, g);
                             const float m = 0.5f * (Ls + Us);
                             aa = 2.f * m;
-                            cst = __fadd_rd(cst, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
+                            c = __fadd_rd(c, __fmaf_rd(-aa, g, -__fmul_ru(m, m)));
                             B = fmaxf(fabsf(xl), fabsf(xu));
                         } else {
                             B = fabsf(x0[i]);
@@ -373,19 +465,20 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1))
                         e = __fmaf_ru(__fmul_ru(kTwoU, mag), B, e);
                     }
                 }
+                cst = __fadd_rd(cst, warp_sum_rd(c));
                 mg = __fadd_ru(mg, e);
             }
             __syncwarp();
             // lam . x0, then Theorem 2 in box form
             float lbv;
             {
-                float c = cst, val = 0.f, e = mg;
+                float c = 0.f, val = 0.f, e = mg;
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     const int i = lane + 32 * q;
                     if (i < s) c = __fmaf_rd(lam[q], x0[i], c);
                 }
-                c = warp_sum_rd(c);
+                c = __fadd_rd(cst, warp_sum_rd(c));
                 for (int j = lane; j < dp; j += 32) {
                     const float m_ = mu[j];
                     const float lo = blo[j], hi = bhi[j];
@@ -499,16 +592,18 @@ static cudaError_t launch_warp_variant(const BoundArgs &a, int steps, float lr, 
     const size_t smem = rows ? with_rows : per_warp;
     if (smem + 1024 > (size_t)max_optin) return cudaErrorInvalidConfiguration;
     const bool ob = a.cost.kind == 1;
-    auto kern = rows ? (ob ? k_alpha_warp<P, true, true> : k_alpha_warp<P, true, false>)
-                     : (ob ? k_alpha_warp<P, false, true> : k_alpha_warp<P, false, false>);
+    auto kern = a.queue ? (rows ? k_alpha_warp<P, true, false, true> : k_alpha_warp<P, false, false, true>)
+                : rows  ? (ob ? k_alpha_warp<P, true, true, false> : k_alpha_warp<P, true, false, false>)
+                        : (ob ? k_alpha_warp<P, false, true, false> : k_alpha_warp<P, false, false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kWarps * 32, smem);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
-    const int need = (a.n + kWarps - 1) / kWarps;
+    const int need = a.queue ? batch_rounds_most(a.n, a.batch.P) : (a.n + kWarps - 1) / kWarps;
     const int grid = need < nsm * occ ? need : nsm * occ;
+    if (a.queue) k_batch_rounds<<<1, 1024, 3 * (size_t)a.batch.P * sizeof(int), st>>>(a);
     AdamTable tab;
     fill_adam_table(tab);
     kern<<<grid, kWarps * 32, smem, st>>>(a, steps, lr, alpha, m, v, tab);

@@ -116,6 +116,7 @@ struct BoundArgs {
     // alpha
     float *grad_alpha;       // [n][H][sumh]
     int *status;
+    int *queue;              // batched alpha-CROWN: batch_queue_ints of scratch (nullable)
     // tensor-core CROWN
     const uint8_t *tcb_img;  // backward image (W_l^T, BF16 hi then lo)
     const float *tc_bias;    // biases padded to multiples of 16 (offsets tc_boff)
@@ -418,6 +419,8 @@ cudaError_t launch_ibp_warp(const BoundArgs &a, cudaStream_t st);
 // (lin_coef); GL, GU [n][Hmax][sumh] and GX [n][Hmax+1][s] are scratch
 cudaError_t launch_box_grad_warp(const BoundArgs &a, float *GL, float *GU, float *GX, float *glo, float *ghi,
                                  cudaStream_t st);
+// ints of scratch for the queue of a batch of n rows over P problems (0: none is used)
+size_t batch_queue_ints(int n, int P);
 // the whole alpha optimisation with one warp per box; alpha (written), m, v: [n][Hmax][sumh] device arrays;
 // steps == 0: one bound with the adaptive slopes (alpha, m, v unused)
 cudaError_t launch_alpha_warp(const BoundArgs &a, int steps, float lr, float *alpha, float *m, float *v,
