@@ -129,7 +129,7 @@ __host__ __device__ inline RowsLayout rows_layout(const NetDesc &N)
 
 // The queue of a batch's alpha-CROWN: rounds of up to kWarps rows of one problem each, the problems of the longest
 // horizons first, so that the CTAs that take rounds from it finish together (with horizons of 10 to 80 and rounds dealt
-// out in row order, the CTAs that met long horizons twice set the time: 64 problems, 8889 rows, 20 steps 25.2 -> 13.6
+// out in row order, the CTAs that met long horizons twice set the time: 64 problems, 8889 rows, 20 steps 25.2 -> 14.2
 // ms).  queue: [0] the next round, [1] the number of rounds, then per round its first place in the permutation of rows
 // and its rows, then the permutation.  One CTA.
 constexpr int kQueueHead = 2, kQueueProblems = 2048;
