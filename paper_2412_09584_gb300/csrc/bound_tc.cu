@@ -127,7 +127,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpi + 1) + (STREAM ? 1 : 0)) * 32, 
     __shared__ uint64_t bar_full[kMaxStages], bar_empty[kMaxStages];
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_index(), lane = threadIdx.x & 31;
     const int mma_warp = NSLOT * kEpi;
     const int L = N.L, s = N.s, k = N.k, H = a.H, d = a.d, sumh = N.sumh, sw = N.sumh + N.s;
     volatile int *abort = &abort_flag;
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpi + 1) + (STREAM ? 1 : 0)) * 32, 
             }
         }
         if (STG) cp_wait<0>();  // no copy may land after the shared memory is released
-    } else if (warp < mma_warp + NSLOT && lane == 0) {
+    } else if (warp < mma_warp + NSLOT && tc::elect_one()) {
         // ---------------------- MMA issuer of slot (warp - mma_warp) ----------------------
         const int sl = warp - mma_warp;
         const int gi = blockIdx.x * NSLOT + sl;
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpi + 1) + (STREAM ? 1 : 0)) * 32, 
             tc::mma_commit(&bar_fin);
             tc::mbar_wait(&bar_fin, 0, &never, kWaitNs);
         }
-    } else if (STREAM && warp == mma_warp + NSLOT && lane == 0) {
+    } else if (STREAM && warp == mma_warp + NSLOT && tc::elect_one()) {
         // ------------- producer: the backward image's atoms in the issuer's order (l = L .. 1) -------------
         const long long cnt = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / G + 1 : 0;
         uint32_t it = 0;
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__((4 * WQ * MB + 1 + (TF || MB == 2 ? 1 : 0)) * 
     __shared__ uint64_t bar_full[STRM ? kRingMaxStages : 1], bar_empty[STRM ? kRingMaxStages : 1];
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_index(), lane = threadIdx.x & 31;
     const int L = N.L, s = N.s, k = N.k, H = a.H, d = a.d, sumh = N.sumh, sw = N.sumh + N.s;
     volatile int *abort = &abort_flag;
 
@@ -1038,7 +1038,7 @@ __global__ void __launch_bounds__((4 * WQ * MB + 1 + (TF || MB == 2 ? 1 : 0)) * 
             }
         }
         cp_wait<0>();  // no copy may land after the shared memory is released
-    } else if (warp == NE && lane == 0) {
+    } else if (warp == NE && tc::elect_one()) {
         // ---------------------- MMA issuer ----------------------
         const long long cnt = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
         long long left = cnt * H * L;
@@ -1119,7 +1119,7 @@ __global__ void __launch_bounds__((4 * WQ * MB + 1 + (TF || MB == 2 ? 1 : 0)) * 
             tc::mma_commit(&bar_fin);
             tc::mbar_wait(&bar_fin, 0, &never, kWaitNs);
         }
-    } else if (STRM && warp == NE + 1 && lane == 0) {
+    } else if (STRM && warp == NE + 1 && tc::elect_one()) {
         // ---------- producer: the image's K blocks in the issuer's order (t = H-1 .. 0, l = L .. 1) ----------
         // BF16: block kb of layer l's hi rows at tcb_hi[l] + kb rows, its lo rows at tcb_lo[l] + kb rows; TF32: the
         // two halves of block kb back to back at tf_off[l] + 2 kb rows (rows = the layer's tcb_N[l] x 128 bytes)

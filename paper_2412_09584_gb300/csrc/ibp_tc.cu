@@ -128,7 +128,7 @@ template <bool TF> __global__ void __launch_bounds__((kEpiW + 2) * 32, 1) k_ibp_
     __shared__ uint64_t bar_a, bar_d, bar_fin, bar_full[kStages], bar_empty[kStages];
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_index(), lane = threadIdx.x & 31;
     const int L = N.L, s = N.s, k = N.k, H = a.H, d = a.d, sumh = N.sumh, sw = N.sumh + N.s;
     volatile int *abort = &abort_flag;
 
@@ -256,7 +256,7 @@ template <bool TF> __global__ void __launch_bounds__((kEpiW + 2) * 32, 1) k_ibp_
             }
             if (!ok) break;
         }
-    } else if (warp == kEpiW && lane == 0) {
+    } else if (warp == kEpiW && tc::elect_one()) {
         // ---------------------- MMA issuer ----------------------
         const int cnt = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
         const uint32_t idesc = TF ? tc::idesc_tf32_f32(128, kNB) : tc::idesc_bf16_f32(128, kNB);
@@ -312,7 +312,7 @@ template <bool TF> __global__ void __launch_bounds__((kEpiW + 2) * 32, 1) k_ibp_
             tc::mma_commit(&bar_fin);
             tc::mbar_wait(&bar_fin, 0, &never, kWaitNs);
         }
-    } else if (warp == kEpiW + 1 && lane == 0) {
+    } else if (warp == kEpiW + 1 && tc::elect_one()) {
         // ------------- producer: the interval image's stages in the issuer's order -------------
         const int cnt = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
         uint32_t it = 0;

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpiWarps + 1) + (STREAM ? NSLOT : 0
     __shared__ uint64_t bar_full[NSLOT * kMaxStages], bar_empty[NSLOT * kMaxStages];
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_index(), lane = threadIdx.x & 31;
     const int mma_warp = NSLOT * kEpiWarps;
     const int L = N.L, s = N.s, k = N.k;
     volatile int *abort = &abort_flag;
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpiWarps + 1) + (STREAM ? NSLOT : 0
                 }
             }
         }
-    } else if (warp < mma_warp + NSLOT && lane == 0) {
+    } else if (warp < mma_warp + NSLOT && tc::elect_one()) {
         // ---------------------- MMA issuer of slot (warp - mma_warp) ----------------------
         const int sl = warp - mma_warp;
         const long long gi = (long long)blockIdx.x * NSLOT + sl;
@@ -574,7 +574,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpiWarps + 1) + (STREAM ? NSLOT : 0
             tc::mma_commit(&bar_fin);
             tc::mbar_wait(&bar_fin, 0, &never, kWaitLimitNs);
         }
-    } else if (STREAM && warp >= mma_warp + NSLOT && lane == 0) {
+    } else if (STREAM && warp >= mma_warp + NSLOT && tc::elect_one()) {
         // ------------------- producer of slot ps: the weight atoms in that issuer's order -------------------
         const int ps = warp - mma_warp - NSLOT;
         uint64_t *full = bar_full + ps * kMaxStages, *empty = bar_empty + ps * kMaxStages;
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(NSLOT * (kEpiWarps + 1) * 32, 1) k_rollout_tcf
     __shared__ uint64_t bar_w, bar_a[NSLOT], bar_d[NSLOT], bar_tok[NSLOT], bar_fin;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_index(), lane = threadIdx.x & 31;
     const int mma_warp = NSLOT * kEpiWarps;
     const int L = N.L, s = N.s, k = N.k;
     volatile int *abort = &abort_flag;
@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(NSLOT * (kEpiWarps + 1) * 32, 1) k_rollout_tcf
                 }
             }
         }
-    } else if (warp < mma_warp + NSLOT && lane == 0) {
+    } else if (warp < mma_warp + NSLOT && tc::elect_one()) {
         // ---------------------- MMA issuer of slot (warp - mma_warp) ----------------------
         // per tile: layer 1 of step 0 (phase 0), then per step layers 2 .. L-1 and the fused product
         const int sl = warp - mma_warp;

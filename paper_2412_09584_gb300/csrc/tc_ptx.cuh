@@ -29,6 +29,23 @@ __device__ __forceinline__ uint64_t globaltimer()
     return t;
 }
 
+// ---- warp roles -----------------------------------------------------------
+// The warp's index as a value the compiler knows to be the same in all lanes, and one lane of a whole warp.
+// Code under elect_one() is compiled for a single thread; under lane == 0 every tcgen05.mma cost its issuer about
+// 120 cycles, twice what a 128 x 128 x 16 product takes to execute, and the issuers were what bounded the kernels.
+// The roles that issue MMAs or bulk copies are entered by elect_one(): k_rollout_tcf 4096 x 1024 x H = 20 with its
+// re-score 8.23 -> 6.78 ms, k_rollout_tc (BF16, four 256-wide layers) 2.86 -> 2.49 ms with its
+// re-scores, in the 3-term split 4.27 -> 3.39 ms; the manipulation net's lower bounds with BF16-split interval bounds
+// 15.3 -> 12.9 ms.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0); }
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n .reg .b32 r;\n elect.sync r|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(p));
+    return p != 0;
+}
+
 // ---- mbarrier -------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {
