@@ -371,19 +371,19 @@ __device__ __noinline__ bool ibp_dense_any(int tid, int nt, bool first, const fl
 
 // Weights beyond shared memory: the layer's forward image goes through a ring of kIbpStages stages of kIbpSpan
 // inputs each, copied asynchronously while the stage before is multiplied; every thread owns the same TR x TN
-// outputs throughout (kIbpStreamRows / TR x Np / TN of them, at most kIbpNT).
+// outputs throughout (rb / TR x Np / TN of them, at most kIbpNT).
 constexpr int kIbpSpan = 32, kIbpStages = 2, kIbpStreamRows = 32;
 
 template <int TR, int TN, bool FIRST>
 __device__ __forceinline__ bool ibp_dense_stream(const float *__restrict__ alo, const float *__restrict__ ahi,
                                                  const uint32_t *__restrict__ mask, int ld,
                                                  float *__restrict__ ring, const float *__restrict__ Wt,
-                                                 const float *__restrict__ bias, int Kp, int Np,
+                                                 const float *__restrict__ bias, int Kp, int Np, int rb,
                                                  float *__restrict__ zlo, float *__restrict__ zhi, const IbpSink &o)
 {
     const int ngc = Np / TN;
     const int rg = threadIdx.x / ngc, c0 = (threadIdx.x - rg * ngc) * TN, r0 = rg * TR;
-    const bool mine = rg < kIbpStreamRows / TR;
+    const bool mine = rg < rb / TR;
     const int nspan = (Kp + kIbpSpan - 1) / kIbpSpan;
     auto fetch = [&](int q) {
         if (q < nspan) {
@@ -452,14 +452,16 @@ __device__ __forceinline__ int group_or(int g, int nt, int v)
 
 // Interval bounds of a tile of boxes.  The weights sit in shared memory and the CTA's warps form kIbpGroups groups of
 // rb boxes each that share them and run on their own (buffers, barriers): while one group waits at a layer's end or
-// walks the narrow output layer, the others multiply.  STREAM: the image does not fit; one group of rb =
-// kIbpStreamRows boxes.  tiles: two bits per layer, the tile of ibp_tile.  safe: some weight may not be finite.
+// walks the narrow output layer, the others multiply.  STREAM: the image does not fit; one group of rb boxes,
+// ROWS of them if not 0.  tiles: two bits per layer, the tile of ibp_tile.  safe: some weight may not be finite.
+// from: the grid's first box (0 with ROWS).
 // What bounds it: issue slots and the latencies of a layer's ends (a step of the pushing network is four layers); the
 // FMAs of the upper ends alone take 3.2 (4 x 4 outputs a thread) to 4.2 cycles (2 x 4) per weight and row.  Measured,
-// all arrays written: pushing 3001 boxes 1079 -> 586 us; object manipulation, 16384 boxes, 51.4 -> 20.6 ms.
-template <bool STREAM>
-__global__ void __launch_bounds__(kIbpNT, 1) k_ibp(BoundArgs a, int rb, int tiles, int vec_h, int vec_s, int safe)
+// all arrays written: pushing 3001 boxes 1079 -> 586 us; object manipulation, 16384 boxes, 51.4 -> 18.5 ms.
+template <bool STREAM, int ROWS = 0>
+__global__ void __launch_bounds__(kIbpNT, 1) k_ibp(BoundArgs a, int rb, int tiles, int vec_h, int vec_s, int safe, int from)
 {
+    const int first = ROWS ? 0 : from;
     constexpr int G = STREAM ? 1 : kIbpGroups, TG = kIbpNT / G;
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
@@ -467,10 +469,10 @@ __global__ void __launch_bounds__(kIbpNT, 1) k_ibp(BoundArgs a, int rb, int tile
     const int s = N.s, k = N.k, L = N.L, d = a.d, H = a.H, sumh = N.sumh;
     const int ld = ibp_ld(N.maxw_p), s4 = pad4(s);
     const int nlive = live_count(a.n, a.d_n, a.row0);
-    if ((int)blockIdx.x * G * rb >= nlive) return;
+    if (first + (int)blockIdx.x * G * rb >= nlive) return;
     // a group's first warps do its narrow layers: spread the groups' over the schedulers (warp id modulo 4)
     const int grp = threadIdx.x / TG, tid = (threadIdx.x + 32 * grp) % TG;
-    const int box0 = ((int)blockIdx.x * G + grp) * rb;
+    const int box0 = first + ((int)blockIdx.x * G + grp) * rb;
     const float *img = a.fwd;
     float *p = sm, *ring = nullptr;
     if (STREAM) {
@@ -649,16 +651,34 @@ __global__ void __launch_bounds__(kIbpNT, 1) k_ibp(BoundArgs a, int rb, int tile
             } else if (!STREAM && l > 1 && rb * Np <= 2 * TG && Np < 64) {
                 bad = ibp_dense_narrow(tid, TG, in_l, in_h, ld, rb, Wt, bias, Kp, Np, zl, zh, o);
             } else if (STREAM) {
-                // the largest tile whose items still cover the threads: 32 rows of 256, 128 or 32 columns
-                if (l == 1) {
-                    if (Np > 128) bad = ibp_dense_stream<4, 4, true>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
-                    else if (Np > 32) bad = ibp_dense_stream<2, 4, true>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
-                    else bad = ibp_dense_stream<1, 2, true>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                // the largest tile whose items still cover the threads: 32 rows of 256, 128 or 32 columns, and half the
+                // rows a thread for each halving of the rows
+#define IBP_STREAM(TR, TN, F) ibp_dense_stream<TR, TN, F>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, ROWS ? ROWS : rb, zl, zh, o)
+                if (ROWS) {
+                    if (l == 1) {
+                        if (Np > 128) bad = IBP_STREAM(4, 4, true);
+                        else if (Np > 32) bad = IBP_STREAM(2, 4, true);
+                        else bad = IBP_STREAM(1, 2, true);
+                    } else {
+                        if (Np > 128) bad = IBP_STREAM(4, 4, false);
+                        else if (Np > 32) bad = IBP_STREAM(2, 4, false);
+                        else bad = IBP_STREAM(1, 2, false);
+                    }
                 } else {
-                    if (Np > 128) bad = ibp_dense_stream<4, 4, false>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
-                    else if (Np > 32) bad = ibp_dense_stream<2, 4, false>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
-                    else bad = ibp_dense_stream<1, 2, false>(in_l, in_h, mk, ld, ring, Wt, bias, Kp, Np, zl, zh, o);
+                    const int tr = Np > 128 ? (rb > 16 ? 4 : rb > 8 ? 2 : 1) : Np > 32 ? (rb > 16 ? 2 : 1) : 0;
+                    if (l == 1) {
+                        if (tr == 4) bad = IBP_STREAM(4, 4, true);
+                        else if (tr == 2) bad = IBP_STREAM(2, 4, true);
+                        else if (tr == 1) bad = IBP_STREAM(1, 4, true);
+                        else bad = IBP_STREAM(1, 2, true);
+                    } else {
+                        if (tr == 4) bad = IBP_STREAM(4, 4, false);
+                        else if (tr == 2) bad = IBP_STREAM(2, 4, false);
+                        else if (tr == 1) bad = IBP_STREAM(1, 4, false);
+                        else bad = IBP_STREAM(1, 2, false);
+                    }
                 }
+#undef IBP_STREAM
             } else {
                 switch ((l == 1 ? 4 : 0) + ((tiles >> (2 * l)) & 3)) {
                     case 0: bad = ibp_dense<4, 4, false>(tid, in_l, in_h, mk, ld, rb, Wt, bias, Kp, Np, zl, zh, o); break;
@@ -1361,14 +1381,28 @@ cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st)
         const size_t smem = (img + kIbpGroups * ibp_rest_floats(N, rb)) * 4;
         cudaError_t e = cudaFuncSetAttribute(k_ibp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_ibp<false><<<(a.n + per - 1) / per, kIbpNT, smem, st>>>(a, rb, tiles, vec_h, vec_s, a.unchecked);
+        k_ibp<false><<<(a.n + per - 1) / per, kIbpNT, smem, st>>>(a, rb, tiles, vec_h, vec_s, a.unchecked, 0);
     } else {
-        const int rb = kIbpStreamRows;
-        const size_t smem = ((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, rb)) * 4;
-        if (smem > (size_t)budget) return cudaErrorInvalidConfiguration;
-        cudaError_t e = cudaFuncSetAttribute(k_ibp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // Whole waves of full tiles, then one wave of tiles with as few rows as hold the rest: a tile of the object-
+        // manipulation network (H = 40) takes 5.1 ms with 32 rows, 4.9 with 24, 3.3 with 12 or 16, 2.5 with 8, 1.9
+        // with 4.  32 rows throughout -> this: 16 boxes 6.3 -> 1.9 ms, 1200 6.3 -> 2.5, 6000 11.3 -> 7.6, 16384
+        // 20.1 -> 18.5, whole waves as before.
+        const int waves = a.n / (kIbpStreamRows * num_sms), full = waves * kIbpStreamRows * num_sms, left = a.n - full;
+        auto run = [&](auto kern, int rb, int first, int boxes) {
+            const size_t smem = ((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, rb)) * 4;
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            kern<<<(boxes + rb - 1) / rb, kIbpNT, smem, st>>>(a, rb, 0, vec_h, vec_s, a.unchecked, first);
+            return cudaGetLastError();
+        };
+        if (((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, kIbpStreamRows)) * 4 > (size_t)budget)
+            return cudaErrorInvalidConfiguration;
+        const int tail = ((left + num_sms - 1) / num_sms + 3) & ~3;
+        cudaError_t e = cudaSuccess;
+        if (waves > 0) e = run(k_ibp<true, kIbpStreamRows>, kIbpStreamRows, 0, full);
+        if (e == cudaSuccess && left > 0)
+            e = run(k_ibp<true>, tail, full, left);
         if (e != cudaSuccess) return e;
-        k_ibp<true><<<(a.n + rb - 1) / rb, kIbpNT, smem, st>>>(a, rb, 0, vec_h, vec_s, a.unchecked);
     }
     return cudaGetLastError();
 }
@@ -1412,7 +1446,7 @@ cudaError_t launch_crown(const BoundArgs &a, int num_sms, cudaStream_t st) { ret
 cudaError_t preload_ibp_crown()
 {
     cudaFuncAttributes fa;
-    const void *kerns[] = {(const void *)k_ibp<true>, (const void *)k_ibp<false>,
+    const void *kerns[] = {(const void *)k_ibp<true>, (const void *)k_ibp<true, kIbpStreamRows>, (const void *)k_ibp<false>,
                            (const void *)k_rows<1, true, false>, (const void *)k_rows<1, false, false>,
                            (const void *)k_rows<2, true, false>, (const void *)k_rows<2, false, false>,
                            (const void *)k_rows<4, true, false>, (const void *)k_rows<4, false, false>,
