@@ -1238,52 +1238,71 @@ __global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a,
     cluster.sync();  // no CTA leaves while another may still write its shared memory
 }
 
-// BF16 mode, one problem, every box re-scored: the same FP32 re-score as k_rescore_fp32 for a tile of RR boxes
-// at once (one row per box: its chosen sample), the layers as register-blocked FP32 products over the tile with
-// the network image in shared memory (WSMEM) or read through L1, so that each weight read serves RR boxes.
-constexpr int kRescoreRows = 28;  // 4096 boxes make 147 CTAs: one wave on 152 SMs
-// 512 threads: a 128-wide layer of the tile is 448 register tiles of 2 rows x 4 columns, one per thread (256
-// threads took two each, 0.49 ms for 4096 boxes)
-constexpr int kRescoreThreads = 512;
-static_assert(kRescoreRows <= kRescoreThreads, "one thread per row keeps that row's pusher position");
-template <bool WSMEM, bool OBST>
+// BF16 mode, one problem, every box re-scored: the same FP32 re-score as k_rescore_fp32 (one row per box: its chosen
+// sample), the layers as register-blocked FP32 products.  With the network image in shared memory (G > 1) a CTA's warps
+// form G groups of RR boxes that share it and run on their own, behind their own barriers; else one group reads the
+// image through L1, so that each weight read serves RR boxes.
+// What bounds it: shared-memory reads of the weights (about 5 thousand cycles for a 128-wide layer of 4 x 8 boxes, 4 x 4
+// outputs a thread); with few boxes the chain of layers.  28 boxes on one group of 512 threads throughout -> this:
+// pushing network, H = 20: 64 to 1200 boxes 285 -> 187 us, 2400 285 -> 212, 4096 286 -> 268, 9000 849 -> 532; 256-wide
+// layers, H = 40: 500 boxes 5.0 -> 2.3 ms, 2400 5.1 -> 2.7, 9000 14.6 -> 10.7.
+constexpr int kRescoreThreads = 512, kRescoreGroups = 4, kRescoreTile = 28;
+
+// Shared-memory floats of one group of rr boxes.
+__host__ __device__ inline size_t rescore_floats(const NetDesc &N, int rr)
+{
+    return (2 * (size_t)rr * N.maxw_p + (size_t)rr * (pad4(N.s) + pad4(N.k)) + rr + 3) & ~size_t(3);
+}
+
+template <int RR, int G, bool OBST>
 __global__ void __launch_bounds__(kRescoreThreads) k_rescore_rows(RolloutArgs a)
 {
-    constexpr int RR = kRescoreRows, NT = kRescoreThreads;
+    constexpr int NT = kRescoreThreads / G;
+    static_assert(RR <= NT, "one thread per row keeps that row's pusher position");
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
     const NetDesc &N = a.net;
     const int s = N.s, k = N.k, L = N.L, d = a.d, ld = N.maxw_p, s4 = pad4(s), Kp1 = pad4(s + k);
+    const int nlive = live_count(a.n, a.d_n);
+    if ((int)blockIdx.x * G * RR >= nlive) return;  // the whole tile is beyond the live rows (so below, nlive >= 1)
     const float *img = a.fwd;
     float *p = sm;
-    if (WSMEM) {
-        for (int i = threadIdx.x; i < N.img_floats / 4; i += NT) smem4[i] = reinterpret_cast<const float4 *>(a.fwd)[i];
+    if (G > 1) {
+        for (int i = threadIdx.x; i < N.img_floats / 4; i += kRescoreThreads)
+            smem4[i] = reinterpret_cast<const float4 *>(a.fwd)[i];
         img = sm;
         p += N.img_floats;
+        __syncthreads();
     }
+    // a group's first warps do its narrow layers: spread the groups' over the schedulers (warp id modulo 4)
+    const int grp = G > 1 ? threadIdx.x / NT : 0, tid = G > 1 ? (threadIdx.x + 32 * grp) % NT : threadIdx.x;
+    auto barrier = [&]() {
+        if (G > 1) group_barrier(grp, NT);
+        else __syncthreads();
+    };
+    const int row0 = ((int)blockIdx.x * G + grp) * RR;
+    if (row0 >= nlive) return;
+    p += grp * rescore_floats(N, RR);
     float *act0 = p; p += RR * ld;
     float *act1 = p; p += RR * ld;
     float *xs = p; p += RR * s4;
     float *us = p; p += RR * pad4(k);
-    float *fsum = p; p += RR;
-    __shared__ uint64_t hbs[RR];
-    __shared__ uint32_t ms[RR];
-    __shared__ int take[RR];
-    const int nlive = live_count(a.n, a.d_n);
-    const int row0 = blockIdx.x * RR;
-    if (row0 >= nlive) return;  // the whole tile is beyond the live rows (so below, nlive >= 1)
-    for (int r = threadIdx.x; r < RR; r += NT) {
+    float *fsum = p;
+    __shared__ uint64_t hbs_[G][RR];
+    __shared__ uint32_t ms_[G][RR];
+    uint64_t *hbs = hbs_[grp];
+    uint32_t *ms = ms_[grp];
+    for (int r = tid; r < RR; r += NT) {
         const int box = row0 + r < nlive ? row0 + r : nlive - 1;  // idle rows recompute a valid box, unused
-        take[r] = row0 + r < nlive;
         hbs[r] = box_hash(a.seed, a.id[box]);
         ms[r] = (uint32_t)(a.keys[box] & 0xFFFFFFFFull);
         fsum[r] = 0.f;
     }
-    for (int i = threadIdx.x; i < RR * s; i += NT) xs[(i / s) * s4 + i % s] = a.x0[i % s];
-    float px = OBST ? a.cost.p0x : 0.f, py = OBST ? a.cost.p0y : 0.f;  // pusher position of row threadIdx.x
-    __syncthreads();
+    for (int i = tid; i < RR * s; i += NT) xs[(i / s) * s4 + i % s] = a.x0[i % s];
+    float px = OBST ? a.cost.p0x : 0.f, py = OBST ? a.cost.p0y : 0.f;  // pusher position of row tid
+    barrier();
     for (int t = 0; t < a.H; ++t) {
-        for (int i = threadIdx.x; i < RR * Kp1; i += NT) {
+        for (int i = tid; i < RR * Kp1; i += NT) {
             const int r = i / Kp1, c = i % Kp1;
             const int box = row0 + r < nlive ? row0 + r : nlive - 1;
             float v = 0.f;
@@ -1296,18 +1315,22 @@ __global__ void __launch_bounds__(kRescoreThreads) k_rescore_rows(RolloutArgs a)
             }
             act0[r * ld + c] = v;
         }
-        __syncthreads();
+        barrier();
         float *in = act0, *out = act1;
         for (int l = 1; l <= L; ++l) {
-            dense_rows_auto<RR, NT>(in, ld, img + N.fwd_w[l], img + N.fwd_b[l], pad4(N.dims[l - 1]), pad4(N.dims[l]),
-                                    out, ld, l < L);
-            __syncthreads();
+            const int Kp = pad4(N.dims[l - 1]), Np = pad4(N.dims[l]);
+            const float *W = img + N.fwd_w[l], *b = img + N.fwd_b[l];
+            if (G > 1 && RR == 8 && Np >= 64)
+                dense_rows<RR, NT, (RR == 8 ? 4 : 1), 4>(in, ld, W, b, Kp, Np, out, ld, l < L, tid);
+            else
+                dense_rows_auto<RR, NT>(in, ld, W, b, Kp, Np, out, ld, l < L, tid);
+            barrier();
             float *tmp = in;
             in = out;
             out = tmp;
         }
         // the step's action cost (inputs in index order), then the state cost, as k_rescore_fp32 sums them
-        for (int r = threadIdx.x; r < RR; r += NT) {
+        for (int r = tid; r < RR; r += NT) {
             float f = fsum[r];
             for (int j = 0; j < k; ++j) {
                 const float u = us[r * pad4(k) + j];
@@ -1327,10 +1350,10 @@ __global__ void __launch_bounds__(kRescoreThreads) k_rescore_rows(RolloutArgs a)
             }
             fsum[r] = f + c;
         }
-        __syncthreads();
+        barrier();
     }
-    for (int r = threadIdx.x; r < RR; r += NT)
-        if (take[r]) a.ub[row0 + r] = fsum[r];
+    for (int r = tid; r < RR; r += NT)
+        if (row0 + r < nlive) a.ub[row0 + r] = fsum[r];
 }
 
 static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
@@ -1371,20 +1394,37 @@ static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
         else k_rescore_fp32<false><<<grid, 256, 0, st>>>(a);
         return cudaGetLastError();
     }
-    int dev, budget = 0;
+    int dev, budget = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&budget, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const size_t rest =
-        ((size_t)2 * kRescoreRows * N.maxw_p + (size_t)kRescoreRows * (pad4(N.s) + pad4(N.k)) + kRescoreRows) * 4;
-    const size_t img = (size_t)N.img_floats * 4;
-    const bool wsmem = img + rest + 1024 <= (size_t)budget;
-    const size_t smem = (wsmem ? img : 0) + rest;
-    auto kern = a.cost.kind == 1 ? (wsmem ? k_rescore_rows<true, true> : k_rescore_rows<false, true>)
-                                 : (wsmem ? k_rescore_rows<true, false> : k_rescore_rows<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(a.n + kRescoreRows - 1) / kRescoreRows, kRescoreThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    auto run = [&](auto plain, auto obst, int rows, size_t floats) {
+        auto kern = a.cost.kind == 1 ? obst : plain;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * floats));
+        if (e != cudaSuccess) return e;
+        kern<<<(a.n + rows - 1) / rows, kRescoreThreads, 4 * floats, st>>>(a);
+        return cudaGetLastError();
+    };
+    // The image in shared memory beside the groups: as few boxes per group as make one wave (2, 4; 8 beyond), or as
+    // fit; no room for the image: one group, as few boxes as make one wave (4, 8, 16), beyond that 16 or kRescoreTile,
+    // whose waves take less time (a tile of 28 1.85 times one of 16 on 256-wide layers).
+    constexpr int G = kRescoreGroups, T = kRescoreTile;
+    const size_t img = (size_t)N.img_floats, room = ((size_t)budget - 1024) / 4;
+    int rr = 2;
+    while (rr < 8 && (long long)sms * G * rr < a.n) rr *= 2;
+    while (rr > 2 && img + G * rescore_floats(N, rr) > room) rr /= 2;
+    const size_t floats = img + G * rescore_floats(N, rr);
+    if (floats <= room) {
+        if (rr == 2) return run(k_rescore_rows<2, G, false>, k_rescore_rows<2, G, true>, 2 * G, floats);
+        if (rr == 4) return run(k_rescore_rows<4, G, false>, k_rescore_rows<4, G, true>, 4 * G, floats);
+        return run(k_rescore_rows<8, G, false>, k_rescore_rows<8, G, true>, 8 * G, floats);
+    }
+    auto waves = [&](int rows) { return ((a.n + rows - 1) / rows + sms - 1) / sms; };
+    rr = waves(4) == 1 ? 4 : waves(8) == 1 ? 8 : 100 * waves(16) <= 185 * waves(T) ? 16 : T;
+    if (rr == 4) return run(k_rescore_rows<4, 1, false>, k_rescore_rows<4, 1, true>, rr, rescore_floats(N, rr));
+    if (rr == 8) return run(k_rescore_rows<8, 1, false>, k_rescore_rows<8, 1, true>, rr, rescore_floats(N, rr));
+    if (rr == 16) return run(k_rescore_rows<16, 1, false>, k_rescore_rows<16, 1, true>, rr, rescore_floats(N, rr));
+    return run(k_rescore_rows<T, 1, false>, k_rescore_rows<T, 1, true>, rr, rescore_floats(N, rr));
 }
 
 template <int NSLOT, int SPLIT, int SX, bool STREAM, bool CEM, bool OBST>
