@@ -161,7 +161,7 @@ def rollout_roofline(precision, p, nb, M, H, roll_ms):
     achieved = 2.0 * nb * M * H * macs / (roll_ms / 1e3) / 1e12
     if precision == "fp32":
         pk = fp32_peak_measured()
-        roof = {"kernel": "k_rollout_fp32 (bab_rollout)", "bound": "alu", "peak": pk["tflops"],
+        roof = {"kernel": "k_rollout_rows (bab_rollout)", "bound": "alu", "peak": pk["tflops"],
                 "peak_note": "of measured FP32 FMA rate (bab_probe_fp32_peak on this GPU, best of scalar "
                              f"{pk['scalar']:.1f} and paired {pk['paired']:.1f} TFLOP/s)"}
     else:
@@ -922,7 +922,7 @@ def batched_bab(dev, iters=50, n_pick=64, samples=None, alpha_steps=None, P=None
             "launch_rows_per_iteration": nb,
             "subdomain_bounds_per_s": children / (ms / 1e3),
             "rollout_steps_per_s": children * samples * float(np.mean(Hs)) / (ms / 1e3),
-            "launches_per_iteration": 3 + 4 + 2 + 1, "timed_region": "CUDA-graph replays, one launch per kernel, "
+            "launches_per_iteration": 3 + 4 + 3 + 1, "timed_region": "CUDA-graph replays, one launch per kernel, "
                                                                     "after a device copy of the iteration's quotas",
             "live_rows_end": n, "live_rows_per_problem_end": {"min": int(live.min()), "median": float(np.median(live)),
                                                                "max": int(live.max())},

@@ -6,21 +6,22 @@
 //                row k of every layer, S_k = sum_j |W_kj| max|a_j| over the
 //                layer's input box (used to bound the rounding error of the
 //                backward products).
-//   k_crown      Theorem 1 backward propagation of the tangent-linearised cost
+//   k_rows       CROWN: Theorem 1 backward propagation of the tangent-linearised cost
 //                through all H steps, then Theorem 2 in box form.  Constant
 //                terms are accumulated with downward rounding (so they are
 //                lower bounds by construction); the rounding error of the
 //                coefficient vectors (the products A W_l, the relaxation
 //                products, the state-coefficient updates) is bounded a
 //                posteriori and subtracted as `margin`.
-//   k_alpha_fwd  forward pass of the relaxed network from x_0 and the
-//                concretizing point u*, giving dLB/dalpha = A_j z~_j.
+//                Its other form (FWD) is the adjoint, the forward pass of the relaxed
+//                network from x_0 and the concretizing point u*, giving
+//                dLB/dalpha = A_j z~_j.
 //   k_adam       projected Adam ascent on alpha.
 //
-// In k_crown and k_alpha_fwd a CTA owns RB boxes (rows); the network image lives
-// in shared memory when it fits (otherwise it is read through L2); the rows move
-// through the layers as register-blocked FP32 products (dense_rows), and each
-// per-row reduction is one warp with shuffles.  k_ibp has its own tiles.
+// In k_rows a CTA's warps form groups of a few boxes (rows) each that share the
+// network image, in shared memory when it fits (otherwise it is read through L2);
+// the rows move through the layers as register-blocked FP32 products (dense_rows),
+// and each per-row reduction is one warp with shuffles.  k_ibp has its own tiles.
 #include <cmath>
 
 #include "bab_internal.cuh"
@@ -28,7 +29,7 @@
 
 namespace bab {
 
-constexpr int RB = 28;  // boxes per CTA: 4096 boxes make 147 CTAs, one wave on 152 SMs (32 left 24 SMs idle)
+constexpr int RB = 28;  // boxes whose working set must fit in shared memory for k_rows to take a network
 constexpr int NT = 512;
 constexpr float kTwoU = 1.1920930376163597e-07f;  // 2^-23 (1 + 2^-20): twice the unit roundoff, rounded up
 
@@ -704,7 +705,7 @@ __global__ void __launch_bounds__(kIbpNT, 1) k_ibp(BoundArgs a, int rb, int tile
 // ---------------------------------------------------------------------------
 // CROWN and its adjoint over a tile of rows.  The per-box arrays are reached
 // through a RowsView whose pointers start at the tile's first box, so the same
-// code runs on the global arrays (k_crown, k_alpha_fwd) and on copies held in
+// code runs on the global arrays (k_rows) and on copies held in
 // shared memory for a whole alpha optimisation (k_alpha_fused).
 // ---------------------------------------------------------------------------
 struct RowsView {
@@ -1158,7 +1159,7 @@ __global__ void __launch_bounds__(NT, 1) k_rows(BoundArgs a, int stride)
 // helpers, slopes, Adam moments, coefficients before relaxation, u*) stay in
 // shared memory for all `steps` (bound, adjoint + Adam) rounds; only the best
 // bound (and the final slopes, when asked for) go back to global memory.  The
-// arithmetic is that of k_crown, k_alpha_fwd and k_adam, step for step.
+// arithmetic is that of k_rows and k_adam, step for step.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline size_t fused_box_floats(const NetDesc &N, int H, int d)
 {

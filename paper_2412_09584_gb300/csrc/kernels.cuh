@@ -101,7 +101,7 @@ struct BoundArgs {
     int row0;                // the launch's first row within the caller's arrays (chunked calls; d_n counts from 0)
     int H, d;
     float rho;
-    // interval bounds (written by k_ibp, read by k_crown / k_alpha_fwd)
+    // interval bounds (written by k_ibp, read by k_rows)
     float *pre_lo, *pre_hi;  // [n][H][sumh]
     float *x_lo, *x_hi;      // [n][H+1][s]
     float *S;                // [n][H][sumh + s] (nullable): per row of each layer, an upper bound of sum_j |W_kj| max|a_j|
