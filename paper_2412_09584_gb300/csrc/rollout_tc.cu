@@ -365,7 +365,9 @@ __global__ void __launch_bounds__((NSLOT * (kEpiWarps + 1) + (STREAM ? NSLOT : 0
                         // 16 columns per TMEM round trip: two loads per wait spill at the 96-register cap with the
                         // bias additions or the hi/lo split, and measured slower for BF16 with the bias in the MMA
                         // (11.1 against 10.5 ms); four epilogue warps per tile with two 64-column waits per layer
-                        // measured slower too: the conversions then run on half as many warps
+                        // measured slower too: the conversions then run on half as many warps; so did 32 or 64 columns
+                        // where one tile has the registers (streamed BF16, 65536 rollouts with re-scores: 2.61 against
+                        // 2.48 ms)
                         constexpr int kCols = 16;
                         for (int c0 = c_beg; c0 < c_end; c0 += kCols) {
                             uint32_t v[kCols / 16][16];
@@ -471,7 +473,7 @@ __global__ void __launch_bounds__((NSLOT * (kEpiWarps + 1) + (STREAM ? NSLOT : 0
             const uint32_t idesc = tc::idesc_bf16_f32(128, Nl);
             if (!STREAM) {
                 // operands stepped with 32-bit adds on precomputed descriptor words, four K steps (one 64-wide
-                // K-atom) unrolled: the issuing thread's own instructions, not the tensor core, set the MMA rate
+                // K-atom) unrolled, so that the issuing thread keeps up with the tensor core (62 cycles an MMA)
                 const int nks = Kl / 16;
                 const uint32_t atom = (uint32_t)Nl * 8u;  // one K-atom of the image in 16-byte units
                 uint32_t qh = tc::desc_sw128_lo(tc::smem_u32(wimg + N.tc_hi[l]));
@@ -929,7 +931,8 @@ __global__ void __launch_bounds__(NSLOT * (kEpiWarps + 1) * 32, 1) k_rollout_tcf
             const uint32_t a0 = ph == 0 ? acol + rowc : acol;  // layer 1 of step 0 reads the input row
             const uint32_t idesc = tc::idesc_bf16_f32(128, Nl);
             // the other slot may start once half of this product is issued (a quarter, three quarters or all of it
-            // measured 8.47, 8.43 and 8.45 ms against 8.30 for 4096 x 1024 x H = 20 rollouts with the re-score)
+            // measured 8.47, 8.43 and 8.45 ms against 8.30 for 4096 x 1024 x H = 20 rollouts with the re-score; with
+            // the elected issuers three quarters measured 6.81 against 6.78)
             const int nks = Kl / 16, kpass = (nks + 1) / 2;
             const uint32_t atom = (uint32_t)Nl * 8u;
             uint32_t q = tc::desc_sw128_lo(tc::smem_u32(wimg + boff));
