@@ -1084,27 +1084,51 @@ __global__ void __launch_bounds__(256) k_rescore_fp32(RolloutArgs a)
 }
 
 // BF16 mode, one problem, top-k re-score of a large network: the boxes of the top-k list, nbox (at most kRescoreBoxes)
-// per thread-block cluster at a time, a warp each in every CTA.  Each of the cluster's CTAs keeps its share of every layer's
+// per thread-block cluster at a time, a warp each in every CTA.  Each of the cluster's CTAs keeps its share of the layers'
 // columns of W_l^T (at most 32) in shared memory for all steps and boxes, computes those outputs one per lane (the same
 // sums, in the same order, as k_rescore_fp32 and k_rescore_rows: from the bias over the inputs in order) and writes them
 // into every CTA's shared memory (distributed shared memory); a cluster barrier closes each layer.  The outputs alternate
 // between two buffers without restarting at a step, so a CTA one layer ahead writes the buffer that nobody reads.  The
 // list and its count are the same for every CTA, so all of them reach the same barriers.
+// The columns of a layer that is not in `resident` (rescore_cl_layers: those beyond shared memory) are copied into one
+// buffer that these layers share, at every step, before the layer's product.
 // What bounds it: the chain of 200 layers (40 steps of the object-manipulation network), each a dependent FMA chain of
 // up to 256 inputs and a cluster barrier.  64 boxes: 1710 us with every layer's columns staged from L2 at every step
 // and one box per cluster -> 401 us.
 constexpr int kRescoreCTAs = 8, kRescoreBoxes = 8, kRescoreClThreads = 32 * kRescoreBoxes;
 
-// Floats of shared memory for a CTA's columns of every layer, [inputs][columns] and their biases each.
-__host__ __device__ inline size_t rescore_cl_floats(const NetDesc &N)
+// Floats of shared memory for a CTA's columns of layer l, [inputs][columns], and their biases.
+__host__ __device__ inline size_t rescore_cl_floats(const NetDesc &N, int l)
 {
-    size_t f = 0;
-    for (int l = 1; l <= N.L; ++l) f += (size_t)(N.dims[l - 1] + 1) * ((N.dims[l] + kRescoreCTAs - 1) / kRescoreCTAs);
-    return f;
+    return (size_t)(N.dims[l - 1] + 1) * ((N.dims[l] + kRescoreCTAs - 1) / kRescoreCTAs);
+}
+
+// The layers (bit l) whose columns stay in `room` floats of shared memory, and the floats they take: all of them, or
+// the first ones that fit beside a buffer for the widest layer.
+static uint32_t rescore_cl_layers(const NetDesc &N, size_t room, size_t &floats)
+{
+    size_t all = 0, most = 0;
+    uint32_t resident = 0;
+    for (int l = 1; l <= N.L; ++l) {
+        const size_t f = rescore_cl_floats(N, l);
+        all += f;
+        most = f > most ? f : most;
+        resident |= 1u << l;
+    }
+    floats = all;
+    if (all <= room) return resident;
+    resident = 0;
+    floats = most;  // the buffer
+    for (int l = 1; l <= N.L; ++l)
+        if (floats + rescore_cl_floats(N, l) <= room) {
+            floats += rescore_cl_floats(N, l);
+            resident |= 1u << l;
+        }
+    return resident;
 }
 
 template <bool OBST>
-__global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a, int nbox)
+__global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a, int nbox, uint32_t resident)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -1119,23 +1143,26 @@ __global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a,
     const int lane = threadIdx.x & 31, slot = threadIdx.x >> 5;
     const int count = (int)a.topk_t[3];
     if (cl * nbox >= count) return;  // the same in every CTA of the cluster
-    {
-        float *w = wsl;
-        for (int l = 1; l <= N.L; ++l) {
-            const int no = N.dims[l], ni = N.dims[l - 1], Np = pad4(no);
-            const int chunk = (no + kRescoreCTAs - 1) / kRescoreCTAs, q0 = rank * chunk;
-            const float *Wt = a.fwd + N.fwd_w[l];
+    // this CTA's columns of layer l and their biases
+    auto fill = [&](int l, float *w) {
+        const int no = N.dims[l], ni = N.dims[l - 1], Np = pad4(no);
+        const int chunk = (no + kRescoreCTAs - 1) / kRescoreCTAs, q0 = rank * chunk;
+        const float *Wt = a.fwd + N.fwd_w[l];
 #pragma unroll 8
-            for (int i = threadIdx.x; i < ni * chunk; i += kRescoreClThreads) {
-                const int c = i / chunk, j = i - c * chunk;
-                w[i] = q0 + j < no ? __ldg(Wt + (size_t)c * Np + q0 + j) : 0.f;
-            }
-            w += ni * chunk;
-            for (int j = threadIdx.x; j < chunk; j += kRescoreClThreads) w[j] = q0 + j < no ? a.fwd[N.fwd_b[l] + q0 + j] : 0.f;
-            w += chunk;
+        for (int i = threadIdx.x; i < ni * chunk; i += kRescoreClThreads) {
+            const int c = i / chunk, j = i - c * chunk;
+            w[i] = q0 + j < no ? __ldg(Wt + (size_t)c * Np + q0 + j) : 0.f;
         }
-    }
-    // (the warps beyond the boxes' have helped stage the weights; they go on to the barriers only)
+        for (int j = threadIdx.x; j < chunk; j += kRescoreClThreads)
+            w[ni * chunk + j] = q0 + j < no ? a.fwd[N.fwd_b[l] + q0 + j] : 0.f;
+    };
+    float *stage = wsl;  // behind the resident layers
+    for (int l = 1; l <= N.L; ++l)
+        if ((resident >> l) & 1u) {
+            fill(l, stage);
+            stage += rescore_cl_floats(N, l);
+        }
+    // (the warps beyond the boxes' help stage the weights and reach the barriers)
     const bool works = slot < nbox;
     const int sl = works ? slot : 0;
     float *xin = reinterpret_cast<float *>(xin4[sl]), *xs = xs_[sl], *es = es_[sl];
@@ -1159,10 +1186,18 @@ __global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a,
         cluster.sync();  // the weights staged; the cluster's CTAs running, the last boxes' buffers free
         int cur = 0;
         for (int t = 0; t < a.H; ++t) {
-            const float *w = wsl;
+            const float *next = wsl;
             for (int l = 1; l <= N.L; ++l) {
                 const int no = N.dims[l], ni = N.dims[l - 1];
                 const int chunk = (no + kRescoreCTAs - 1) / kRescoreCTAs, q = rank * chunk + lane;  // chunk <= 32
+                const float *w = stage;
+                if ((resident >> l) & 1u) {
+                    w = next;
+                    next += (ni + 1) * chunk;
+                } else {
+                    fill(l, stage);  // (the buffer's last layer was read before that layer's cluster barrier)
+                    __syncthreads();
+                }
                 const float4 *in = l == 1 ? xin4[sl] : act4[sl][cur ^ 1];
                 if (works && lane < chunk && q < no) {
                     float acc = w[ni * chunk + lane];
@@ -1205,7 +1240,6 @@ __global__ void __launch_bounds__(kRescoreClThreads) k_rescore_cl(RolloutArgs a,
 #pragma unroll
                     for (int r2 = 0; r2 < kRescoreCTAs; ++r2) cluster.map_shared_rank(out, r2)[q] = v;
                 }
-                w += (ni + 1) * chunk;
                 cluster.sync();  // every CTA's copy of the layer output complete
                 cur ^= 1;
             }
@@ -1364,12 +1398,20 @@ static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
     const NetDesc &N = a.net;
     long long macs = 0;
     for (int l = 1; l <= N.L; ++l) macs += (long long)N.dims[l] * N.dims[l - 1];
-    const size_t cl_smem = rescore_cl_floats(N) * sizeof(float);
-    if (a.batch.P <= 1 && a.topk > 0 && macs * a.H > 2000000 && cl_smem <= 200 * 1024) {
+    if (a.batch.P <= 1 && a.topk > 0 && macs * a.H > 2000000) {
         // a large network's top k: a cluster of kRescoreCTAs per nbox listed boxes, as many as make one wave of clusters
         // (this GPU holds 15 at one CTA per SM), at most a warp each
         auto kern = a.cost.kind == 1 ? k_rescore_cl<true> : k_rescore_cl<false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem);
+        int dev, budget = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&budget, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+        if (e != cudaSuccess) return e;
+        size_t floats;
+        const uint32_t resident = rescore_cl_layers(N, ((size_t)budget - fa.sharedSizeBytes) / sizeof(float), floats);
+        const size_t cl_smem = floats * sizeof(float);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         const int nbox = a.topk > 15 * kRescoreBoxes ? kRescoreBoxes : (a.topk + 14) / 15;
@@ -1385,7 +1427,7 @@ static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, kern, a, nbox);
+        return cudaLaunchKernelEx(&cfg, kern, a, nbox, resident);
     }
     if (a.batch.P > 1 || a.topk > 0) {
         // each box reads its own problem's image; with a top-k selection all but k boxes return at once
