@@ -1387,20 +1387,23 @@ cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st)
         // Whole waves of full tiles, then one wave of tiles with as few rows as hold the rest: a tile of the object-
         // manipulation network (H = 40) takes 5.1 ms with 32 rows, 4.9 with 24, 3.3 with 12 or 16, 2.5 with 8, 1.9
         // with 4.  32 rows throughout -> this: 16 boxes 6.3 -> 1.9 ms, 1200 6.3 -> 2.5, 6000 11.3 -> 7.6, 16384
-        // 20.1 -> 18.5, whole waves as before.
-        const int waves = a.n / (kIbpStreamRows * num_sms), full = waves * kIbpStreamRows * num_sms, left = a.n - full;
+        // 20.1 -> 18.5, whole waves as before.  A full tile has kIbpStreamRows rows, or the most that fit beside the
+        // ring (28 or 24 of the widest layers from 113 states on).
+        auto bytes = [&](int rb) { return ((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, rb)) * 4; };
+        int rows = kIbpStreamRows;
+        while (rows > 4 && bytes(rows) > (size_t)budget) rows -= 4;
+        if (bytes(rows) > (size_t)budget) return cudaErrorInvalidConfiguration;
+        const int wave = rows * num_sms, full = a.n / wave * wave, left = a.n - full;
         auto run = [&](auto kern, int rb, int first, int boxes) {
-            const size_t smem = ((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, rb)) * 4;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(rb));
             if (e != cudaSuccess) return e;
-            kern<<<(boxes + rb - 1) / rb, kIbpNT, smem, st>>>(a, rb, 0, vec_h, vec_s, a.unchecked, first);
+            kern<<<(boxes + rb - 1) / rb, kIbpNT, bytes(rb), st>>>(a, rb, 0, vec_h, vec_s, a.unchecked, first);
             return cudaGetLastError();
         };
-        if (((size_t)kIbpStages * kIbpSpan * kMaxWidth + ibp_rest_floats(N, kIbpStreamRows)) * 4 > (size_t)budget)
-            return cudaErrorInvalidConfiguration;
         const int tail = ((left + num_sms - 1) / num_sms + 3) & ~3;
         cudaError_t e = cudaSuccess;
-        if (waves > 0) e = run(k_ibp<true, kIbpStreamRows>, kIbpStreamRows, 0, full);
+        if (full > 0)
+            e = rows == kIbpStreamRows ? run(k_ibp<true, kIbpStreamRows>, rows, 0, full) : run(k_ibp<true>, rows, 0, full);
         if (e == cudaSuccess && left > 0)
             e = run(k_ibp<true>, tail, full, left);
         if (e != cudaSuccess) return e;
