@@ -1368,6 +1368,7 @@ static void ibp_vec(const BoundArgs &a, int &vec_h, int &vec_s)
 cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st)
 {
     if (a.n <= 0) return cudaSuccess;
+    if (ibp_warp_takes(a)) return launch_ibp_warp(a, st);
     const NetDesc &N = a.net;
     const int budget = max_optin_smem();
     if (num_sms <= 0) num_sms = sm_count();
@@ -1459,7 +1460,7 @@ cudaError_t preload_ibp_crown()
         cudaError_t e = cudaFuncGetAttributes(&fa, k);
         if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    return preload_ibp_warp();
 }
 
 cudaError_t launch_alpha_fwd(const BoundArgs &a, int num_sms, cudaStream_t st) { return launch_rows<true>(a, num_sms, st); }

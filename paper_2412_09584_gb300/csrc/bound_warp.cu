@@ -611,29 +611,85 @@ static cudaError_t launch_warp_variant(const BoundArgs &a, int steps, float lr, 
 }
 
 
+// The directed sums of one layer's outputs lane + 32 q (q < Q; those beyond Np are not meaningful) over the inputs in
+// order from the bias: lower and upper ends, and the sum S is formed from.  zlo, zhi: the warp's inputs in shared memory
+// (Kp of them, a multiple of 4).
+template <int P, int Q, bool FIRST>
+__device__ __forceinline__ void ibp_warp_sums(const float *__restrict__ zlo, const float *__restrict__ zhi, int Kp,
+                                              const float *__restrict__ W, const float *__restrict__ bias, int Np,
+                                              float (&lo)[P], float (&hi)[P], float (&sum)[P])
+{
+    const int lane = threadIdx.x & 31;
+    const float *Wk[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int j = min(lane + 32 * q, Np - 1);
+        Wk[q] = W + j;
+        lo[q] = hi[q] = bias[j];
+        sum[q] = 0.f;
+    }
+#pragma unroll 2
+    for (int k = 0; k < Kp; k += 4) {
+        const float4 l4 = *reinterpret_cast<const float4 *>(zlo + k), h4 = *reinterpret_cast<const float4 *>(zhi + k);
+        float w[4][Q];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                w[u][q] = *Wk[q];
+                Wk[q] += Np;
+            }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float il = u == 0 ? l4.x : u == 1 ? l4.y : u == 2 ? l4.z : l4.w;
+            const float ih = u == 0 ? h4.x : u == 1 ? h4.y : u == 2 ? h4.z : h4.w;
+            const float am = FIRST ? fmaxf(fabsf(il), fabsf(ih)) : il;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const bool pos = w[u][q] >= 0.f;
+                lo[q] = __fmaf_rd(w[u][q], pos ? il : ih, lo[q]);
+                hi[q] = __fmaf_ru(w[u][q], pos ? ih : il, hi[q]);
+                sum[q] = __fmaf_ru(fabsf(w[u][q]), am, sum[q]);
+            }
+        }
+    }
+}
+
+// CTAs of kWarps warps an SM holds.
+constexpr int ibp_warp_ctas(int P) { return P <= 2 ? 4 : P <= 4 ? 2 : 1; }
+
 // Interval bound propagation (outward-rounded FP32) through the H-step unrolled
 // network, one warp per box: lane q holds the interval of inputs and outputs
 // q, q + 32, ...; per output the three directed-rounding sums (lower, upper,
 // and the one S = sum_j |W_kj| max|a_j| is formed from) run over the inputs in
 // order from the bias, as in k_ibp, so the bounds are bit-identical to it.  Writes the pre-activation
-// bounds, the state intervals, S and (nullable) the interval bound of the cost.
-template <int P, bool WSMEM>
-__global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_ibp_warp(BoundArgs a)
+// bounds, the state intervals, S (nullable) and (nullable) the interval bound of the cost.
+// What bounds it: issue slots (per input a compare, two selects and three FMAs an output slot), and with few boxes the
+// latency of the layers.  The inputs are read from shared memory, four to a load, and the weights loaded four inputs
+// ahead: broadcasting them by shuffles, one input at a time, took 1.4 times as long (two 32-wide layers, 12 steps,
+// 16384 boxes 335 -> 240 us; two 64-wide ones 797 -> 536).
+// OBST: the pushing-with-obstacles cost (one problem, s <= 32, k = 2).
+template <int P, bool WSMEM, bool OBST>
+__global__ void __launch_bounds__(kWarps * 32, ibp_warp_ctas(P)) k_ibp_warp(BoundArgs a)
 {
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
     const NetDesc &N = a.net;
     const int s = N.s, k = N.k, L = N.L, Hm = a.batch.Hmax, d = a.d, sumh = N.sumh, sw = sumh + s;
     const float *fwd = a.fwd;
+    float *zlo = sm;
     if (WSMEM) {
         for (int i = threadIdx.x; i < N.img_floats / 4; i += blockDim.x)
             smem4[i] = reinterpret_cast<const float4 *>(a.fwd)[i];
         fwd = sm;
+        zlo += N.img_floats;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    zlo += (size_t)wib * 2 * N.maxw_p;  // the box's input intervals of a layer
+    float *zhi = zlo + N.maxw_p;
     const int nlive = live_count(a.n, a.d_n, a.row0);
-    for (int box = blockIdx.x * kWarps + wib; box < nlive; box += gridDim.x * kWarps) {
+    for (int box = blockIdx.x * nw + wib; box < nlive; box += gridDim.x * nw) {
         const int pb = row_problem(a.batch, box);
         if (!WSMEM) fwd = a.fwd + (size_t)pb * N.img_floats;
         const float *x0 = a.x0 + (size_t)pb * s, *goal = a.goal + (size_t)pb * s;
@@ -641,7 +697,7 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_
         const float rho = problem_rho(a.batch, pb, a.rho);
         const float *blo = a.lo + (size_t)box * d, *bhi = a.hi + (size_t)box * d;
         float *pl = a.pre_lo + (size_t)box * Hm * sumh, *ph = a.pre_hi + (size_t)box * Hm * sumh;
-        float *S = a.S + (size_t)box * Hm * sw;
+        float *S = a.S ? a.S + (size_t)box * Hm * sw : nullptr;
         float *xlo = a.x_lo + (size_t)box * (Hm + 1) * s, *xhi = a.x_hi + (size_t)box * (Hm + 1) * s;
         float xl[P], xu[P];
 #pragma unroll
@@ -654,6 +710,8 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_
             }
         }
         float lbacc = 0.f;
+        // the pusher's position box (obstacle cost)
+        float pxl = a.cost.p0x, pxh = pxl, pyl = a.cost.p0y, pyh = pyl;
         for (int t = 0; t < H; ++t) {
             float zl[P], zu[P];
 #pragma unroll
@@ -671,54 +729,38 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_
             for (int l = 1; l <= L; ++l) {
                 const int Kp = pad4(N.dims[l - 1]), Np = pad4(N.dims[l]), dl = N.dims[l];
                 const float *W = fwd + N.fwd_w[l], *bias = fwd + N.fwd_b[l];
-                float al_[P], ah_[P], as_[P];
 #pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    const int j = lane + 32 * q;
-                    const float bj = j < Np ? bias[j] : 0.f;
-                    al_[q] = ah_[q] = bj;
-                    as_[q] = 0.f;
-                }
-                const float *Wk = W + lane;
-#pragma unroll
-                for (int pk = 0; pk < P; ++pk) {
-                    if (32 * pk >= Kp) break;
-                    const int kn = min(32, Kp - 32 * pk);
-                    for (int kl = 0; kl < kn; ++kl) {
-                        const float il = __shfl_sync(0xFFFFFFFFu, zl[pk], kl);
-                        const float ih = __shfl_sync(0xFFFFFFFFu, zu[pk], kl);
-                        const float am = l == 1 ? fmaxf(fabsf(il), fabsf(ih)) : il;
-#pragma unroll
-                        for (int q = 0; q < P; ++q) {
-                            if (lane + 32 * q < Np) {
-                                const float w = Wk[32 * q];
-                                const bool pos = w >= 0.f;
-                                al_[q] = __fmaf_rd(w, pos ? il : ih, al_[q]);
-                                ah_[q] = __fmaf_ru(w, pos ? ih : il, ah_[q]);
-                                as_[q] = __fmaf_ru(fabsf(w), am, as_[q]);
-                            }
-                        }
-                        Wk += Np;
+                for (int q = 0; q < P; ++q)
+                    if (lane + 32 * q < Kp) {
+                        zlo[lane + 32 * q] = zl[q];
+                        zhi[lane + 32 * q] = zu[q];
                     }
+                __syncwarp();
+                float al_[P], ah_[P], as_[P];
+                // (only the slots the layer has outputs for)
+                if (l == 1) {
+                    if (P > 1 && Np <= 32) ibp_warp_sums<P, 1, true>(zlo, zhi, Kp, W, bias, Np, al_, ah_, as_);
+                    else ibp_warp_sums<P, P, true>(zlo, zhi, Kp, W, bias, Np, al_, ah_, as_);
+                } else {
+                    if (P > 1 && Np <= 32) ibp_warp_sums<P, 1, false>(zlo, zhi, Kp, W, bias, Np, al_, ah_, as_);
+                    else ibp_warp_sums<P, P, false>(zlo, zhi, Kp, W, bias, Np, al_, ah_, as_);
                 }
+                __syncwarp();
                 const int soff = (l < L) ? N.hoff[l] : sumh;
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     const int j = lane + 32 * q;
+                    if (32 * q >= Np) break;
                     if (j < dl) {
-                        S[(size_t)t * sw + soff + j] = l == 1 ? as_[q] : ibp_s(al_[q], ah_[q], bias[j], as_[q]);
+                        if (S) S[(size_t)t * sw + soff + j] = l == 1 ? as_[q] : ibp_s(al_[q], ah_[q], bias[j], as_[q]);
                         if (l < L) {
                             pl[(size_t)t * sumh + N.hoff[l] + j] = al_[q];
                             ph[(size_t)t * sumh + N.hoff[l] + j] = ah_[q];
                         }
                     }
-                    if (l < L && j < dl) {
-                        zl[q] = fmaxf(al_[q], 0.f);
-                        zu[q] = fmaxf(ah_[q], 0.f);
-                    } else {
-                        zl[q] = al_[q];
-                        zu[q] = ah_[q];
-                    }
+                    const bool relu = l < L && j < dl;
+                    zl[q] = relu ? fmaxf(al_[q], 0.f) : al_[q];
+                    zu[q] = relu ? fmaxf(ah_[q], 0.f) : ah_[q];
                 }
             }
             // x_{t+1} in [x_t] + [z_L]; interval bound of ||x_{t+1} - g||^2
@@ -733,10 +775,38 @@ __global__ void __launch_bounds__(kWarps * 32, P <= 2 ? 4 : (P <= 4 ? 2 : 1)) k_
                     xlo[(size_t)(t + 1) * s + i] = nl;
                     xhi[(size_t)(t + 1) * s + i] = nh;
                     const float g = goal[i];
-                    v = __fadd_rd(v, sq_min_rd(__fsub_rd(nl, g), __fsub_ru(nh, g)));
+                    if (OBST) {
+                        // distance from g to the interval, rounded down, squared rounded down
+                        const float e = fmaxf(fmaxf(__fsub_rd(nl, g), __fsub_rd(g, nh)), 0.f);
+                        v = __fmaf_rd(e, e, v);
+                        zlo[i] = nl;
+                        zhi[i] = nh;
+                    } else {
+                        v = __fadd_rd(v, sq_min_rd(__fsub_rd(nl, g), __fsub_ru(nh, g)));
+                    }
                 }
             }
             v = warp_sum_rd(v);
+            if (OBST) {
+                // w_{t+1} times the distance from g to the box, then the penalties at their minima (rounded down); the
+                // pusher is where u_t has taken it
+                pxl = __fadd_rd(pxl, blo[t * k]);
+                pyl = __fadd_rd(pyl, blo[t * k + 1]);
+                pxh = __fadd_ru(pxh, bhi[t * k]);
+                pyh = __fadd_ru(pyh, bhi[t * k + 1]);
+                __syncwarp();
+                float pen = 0.f;
+                const int nq = s / 2 + 1;
+                for (int q = lane; q < a.cost.n_obs * nq; q += 32) {
+                    const int o = q / nq, kp = q % nq - 1;
+                    pen = __fadd_rd(pen, kp < 0 ? penalty_min_rd(a.cost, o, pxl, pxh, pyl, pyh)
+                                                : penalty_min_rd(a.cost, o, zlo[2 * kp], zhi[2 * kp], zlo[2 * kp + 1],
+                                                                 zhi[2 * kp + 1]));
+                }
+                pen = warp_sum_rd(pen);
+                v = __fadd_rd(__fmul_rd(a.cost.w[t], __fsqrt_rd(v)), pen);
+                __syncwarp();
+            }
             lbacc = __fadd_rd(lbacc, v);
         }
         if (a.lb_ibp && lane == 0) a.lb_ibp[box] = lbacc;
@@ -750,19 +820,26 @@ static cudaError_t launch_ibp_variant(const BoundArgs &a, cudaStream_t st)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const size_t img = (size_t)a.net.img_floats * sizeof(float);
-    const bool wsmem = a.batch.P <= 1 && img + 1024 <= (size_t)max_optin;
-    const size_t smem = wsmem ? img : 0;
-    auto kern = wsmem ? k_ibp_warp<P, true> : k_ibp_warp<P, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t img = (size_t)a.net.img_floats * sizeof(float), row = 2 * (size_t)a.net.maxw_p * sizeof(float);
+    const bool wsmem = a.batch.P <= 1 && img + kWarps * row + 1024 <= (size_t)max_optin;
+    auto smem = [&](int warps) { return (wsmem ? img : 0) + warps * row; };
+    // CTAs of kWarps warps, or of half as many where all boxes then run at once on fewer warps of the busiest SM (4096
+    // boxes: 28 against 32)
+    auto slots = [&](int warps) {
+        const long long room = (max_optin + 1024LL) / (long long)(smem(warps) + 1024), most = ibp_warp_ctas(P) * (kWarps / warps);
+        return (room < most ? room : most) * nsm;
+    };
+    auto busiest = [&](int warps) { return ((a.n + warps - 1) / warps + nsm - 1) / nsm * warps; };
+    constexpr int half = kWarps / 2;
+    const int warps = (long long)a.n <= slots(half) * half && busiest(half) < busiest(kWarps) ? half : kWarps;
+    const long long need = (a.n + warps - 1) / warps, most = slots(warps) > 0 ? slots(warps) : nsm;
+    auto kern = wsmem ? k_ibp_warp<P, true, false> : k_ibp_warp<P, false, false>;
+    if constexpr (P <= 2)
+        if (a.cost.kind == 1) kern = k_ibp_warp<P, true, true>;
+    if (a.cost.kind == 1 && (P > 2 || !wsmem)) return cudaErrorInvalidConfiguration;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(warps));
     if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kWarps * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    const int need = (a.n + kWarps - 1) / kWarps;
-    const int grid = need < nsm * occ ? need : nsm * occ;
-    kern<<<grid, kWarps * 32, smem, st>>>(a);
+    kern<<<(int)(need < most ? need : most), warps * 32, smem(warps), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -773,6 +850,23 @@ static int lanes_needed(const NetDesc &N)
     // every layer's width and the input row [x | u] must fit the lanes' slots
     const int need = pad4(maxw) > pad4(N.s + N.k) ? pad4(maxw) : pad4(N.s + N.k);
     return need <= 32 ? 1 : need <= 64 ? 2 : need <= 128 ? 4 : need <= 256 ? 8 : 0;
+}
+
+// Whether one problem's interval bounds go to k_ibp_warp: no layer wider than 64 (the network then fits in shared
+// memory).  Against k_ibp (boxes x steps of two hidden layers): 32 wide, 300 x 12 66 -> 31 us, 4096 x 12 100 -> 72,
+// 16384 x 12 383 -> 240; 64 wide, 300 x 12 101 -> 54, 16384 x 12 695 -> 536.  96 wide, k_ibp's tiles are the faster
+// ones: 4096 x 20 420 against 1000 us.
+bool ibp_warp_takes(const BoundArgs &a)
+{
+    const int lanes = lanes_needed(a.net);
+    return lanes >= 1 && lanes <= 2;
+}
+
+cudaError_t preload_ibp_warp()
+{
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, k_ibp_warp<1, true, false>);
+    return e == cudaSuccess ? cudaFuncGetAttributes(&fa, k_ibp_warp<2, true, false>) : e;
 }
 
 cudaError_t launch_ibp_warp(const BoundArgs &a, cudaStream_t st)

@@ -413,7 +413,9 @@ cudaError_t launch_alpha_fwd(const BoundArgs &a, int num_sms, cudaStream_t st);
 cudaError_t launch_alpha_init(const BoundArgs &a, cudaStream_t st);
 // the whole alpha optimisation of a tile of boxes in one CTA (needs the interval bounds of launch_ibp)
 cudaError_t launch_alpha_fused(const BoundArgs &a, int steps, float lr, float *alpha_out, int variant, cudaStream_t st);
-// interval bounds with one warp per box (any problem of the batch)
+// interval bounds with one warp per box (any problem of the batch; the obstacle cost where ibp_warp_takes the network)
+bool ibp_warp_takes(const BoundArgs &a);
+cudaError_t preload_ibp_warp();
 cudaError_t launch_ibp_warp(const BoundArgs &a, cudaStream_t st);
 // d(bound)/d(box faces), one warp per box, after interval bounds and a CROWN pass that stored A_pre, u*, mu
 // (lin_coef); GL, GU [n][Hmax][sumh] and GX [n][Hmax+1][s] are scratch

@@ -187,6 +187,7 @@ extern "C" int bab_bound_crown_static(int n_layers, const int *dims, const float
     a.d_n = nullptr;
     a.unchecked = 1;  // the caller's device parameters have not been seen
     a.H = horizon;
+    a.batch.Hmax = horizon;
     a.d = N.k * horizon;
     a.rho = rho;
     a.lb = lb;
