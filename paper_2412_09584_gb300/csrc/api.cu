@@ -1671,7 +1671,7 @@ int bab_bound_batch(bab_ctx *c, const float *x0, const float *goal, const int *h
     const size_t nh = (size_t)n * max_horizon * N.sumh, nx = (size_t)n * (max_horizon + 1) * N.s;
     const size_t ns = (size_t)n * max_horizon * (N.sumh + N.s);
     const size_t floats = 2 * nh + 2 * nx + ns + (alpha_steps > 0 ? 4 * nh : 0);
-    const size_t queue = batch_queue_ints(n, c->n_problems);
+    const size_t queue = batch_queue_ints(n, c->n_problems, alpha_steps, max_horizon);
     rc = ensure_scratch(c, floats * sizeof(float) + queue * sizeof(int) + 17 * 256);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;

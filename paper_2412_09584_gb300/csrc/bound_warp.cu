@@ -131,8 +131,9 @@ __host__ __device__ inline RowsLayout rows_layout(const NetDesc &N)
 // horizons first, so that the CTAs that take rounds from it finish together (with horizons of 10 to 80 and rounds dealt
 // out in row order, the CTAs that met long horizons twice set the time: 64 problems, 8889 rows, 20 steps 25.2 -> 14.2
 // ms).  queue: [0] the next round, [1] the number of rounds, then per round its first place in the permutation of rows
-// and its rows, then the permutation.  One CTA.
-constexpr int kQueueHead = 2, kQueueProblems = 2048;
+// and its rows, then the permutation.  One CTA; the problems are sorted by buckets of horizons (by comparing all
+// pairs, 512 problems took 12 us longer).
+constexpr int kQueueHead = 2, kQueueProblems = 2048, kQueueBuckets = 256;
 
 __host__ __device__ inline int batch_rounds_most(int n, int P) { return n / kWarps + P + 1; }
 
@@ -141,21 +142,37 @@ __global__ void __launch_bounds__(1024) k_batch_rounds(BoundArgs a)
     extern __shared__ int bsm[];
     const int P = a.batch.P, n = live_count(a.n, a.d_n, a.row0), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int *count = bsm, *order = bsm + P, *row_at = bsm + 2 * P;
-    __shared__ int wr[32], wq[32];
+    __shared__ int wr[32], wq[32], place[kQueueBuckets];
     int *rounds = a.queue + kQueueHead, *perm = rounds + 2 * batch_rounds_most(a.n, P);
     for (int p = tid; p < P; p += 1024) count[p] = 0;
+    for (int b = tid; b < kQueueBuckets; b += 1024) place[b] = 0;
     __syncthreads();
     for (int i = tid; i < n; i += 1024) atomicAdd(&count[row_problem(a.batch, i)], 1);
-    // the problems by horizon, longest first
-    for (int p = tid; p < P; p += 1024) {
-        const int h = problem_H(a.batch, p, a.H);
-        int rank = 0;
-        for (int q = 0; q < P; ++q) {
-            const int g = problem_H(a.batch, q, a.H);
-            rank += g > h || (g == h && q < p);
+    // the problems by horizon, longest first (the order of those within a 256th of the longest does not matter)
+    auto bucket = [&](int p) {
+        const long long h = problem_H(a.batch, p, a.H);
+        return kQueueBuckets - 1 - (int)(a.batch.Hmax < kQueueBuckets ? h : h * (kQueueBuckets - 1) / a.batch.Hmax);
+    };
+    for (int p = tid; p < P; p += 1024) atomicAdd(&place[bucket(p)], 1);
+    __syncthreads();
+    if (tid < kQueueBuckets) {
+        const int c = place[tid];
+        int in = c;
+        for (int o = 1; o < 32; o *= 2) {
+            const int x = __shfl_up_sync(0xFFFFFFFFu, in, o);
+            if (lane >= o) in += x;
         }
-        order[rank] = p;
+        if (lane == 31) wr[warp] = in;
+        place[tid] = in - c;
     }
+    __syncthreads();
+    if (tid < kQueueBuckets) {
+        int before = 0;
+        for (int w = 0; w < warp; ++w) before += wr[w];
+        place[tid] += before;
+    }
+    __syncthreads();
+    for (int p = tid; p < P; p += 1024) order[atomicAdd(&place[bucket(p)], 1)] = p;
     __syncthreads();
     // first row and first round of every problem: each thread's problems, then the threads before it
     const int per = (P + 1023) / 1024, p0 = min(P, tid * per), p1 = min(P, p0 + per);
@@ -199,7 +216,18 @@ __global__ void __launch_bounds__(1024) k_batch_rounds(BoundArgs a)
     for (int i = tid; i < n; i += 1024) perm[atomicAdd(&row_at[row_problem(a.batch, i)], 1)] = i;
 }
 
-size_t batch_queue_ints(int n, int P) { return P > 1 && P <= kQueueProblems ? kQueueHead + 2 * (size_t)batch_rounds_most(n, P) + n : 0; }
+// The queue is used where the call does enough to pay for it (passes over the network: two an alpha step, one without
+// any, times the longest horizon), or where most problems have few rows, so that a round in row order would hold rows of
+// several problems, all but one of them with weights read through L1.  Measured, queue against row order: horizons of 5
+// without alpha steps, 8 to 64 rows a problem 47 against 39 us (64 wide, 64 problems), one row a problem 76 against 121;
+// horizons of 3 to 30 without alpha steps within 0.92 and 1.9 of each other, 32768 rows 1.12 to 1.13 times as fast.
+size_t batch_queue_ints(int n, int P, int alpha_steps, int max_horizon)
+{
+    if (P < 2 || P > kQueueProblems) return 0;
+    const long long passes = alpha_steps > 0 ? 2LL * alpha_steps : 1;
+    if (passes * max_horizon < 16 && n >= 4LL * P) return 0;
+    return kQueueHead + 2 * (size_t)batch_rounds_most(n, P) + n;
+}
 
 // What bounds it: issue slots (about 1400 instructions a box and step) and the latency of the per-box arrays in L2; each
 // product is a third of them.  Adam's divisions of zeros (stable neurons, those whose coefficient never took the lower
@@ -603,7 +631,11 @@ static cudaError_t launch_warp_variant(const BoundArgs &a, int steps, float lr, 
     if (occ < 1) return cudaErrorInvalidConfiguration;
     const int need = a.queue ? batch_rounds_most(a.n, a.batch.P) : (a.n + kWarps - 1) / kWarps;
     const int grid = need < nsm * occ ? need : nsm * occ;
-    if (a.queue) k_batch_rounds<<<1, 1024, 3 * (size_t)a.batch.P * sizeof(int), st>>>(a);
+    if (a.queue) {
+        k_batch_rounds<<<1, 1024, 3 * (size_t)a.batch.P * sizeof(int), st>>>(a);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     AdamTable tab;
     fill_adam_table(tab);
     kern<<<grid, kWarps * 32, smem, st>>>(a, steps, lr, alpha, m, v, tab);

@@ -422,7 +422,7 @@ cudaError_t launch_ibp_warp(const BoundArgs &a, cudaStream_t st);
 cudaError_t launch_box_grad_warp(const BoundArgs &a, float *GL, float *GU, float *GX, float *glo, float *ghi,
                                  cudaStream_t st);
 // ints of scratch for the queue of a batch of n rows over P problems (0: none is used)
-size_t batch_queue_ints(int n, int P);
+size_t batch_queue_ints(int n, int P, int alpha_steps, int max_horizon);
 // the whole alpha optimisation with one warp per box; alpha (written), m, v: [n][Hmax][sumh] device arrays;
 // steps == 0: one bound with the adaptive slopes (alpha, m, v unused)
 cudaError_t launch_alpha_warp(const BoundArgs &a, int steps, float lr, float *alpha, float *m, float *v,
