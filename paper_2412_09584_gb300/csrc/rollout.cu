@@ -238,6 +238,14 @@ __host__ __device__ inline int incumbent_lanes(int chunk, int ni)
     return best;
 }
 
+// The same where the weights are read through L2: two at least, so that a warp's load touches fewer rows (128 problems of
+// the pushing network, one CTA each, 20 steps: one lane 1301 us, two 1164).
+__host__ __device__ inline int incumbent_lanes_l2(int chunk, int ni)
+{
+    const int ks = incumbent_lanes(chunk, ni);
+    return ks == 1 && 2 * chunk <= kIncThreads ? 2 : ks;
+}
+
 // doubles of shared memory a CTA of a cluster of ncta needs: its rows of every layer's weights (ni + lanes apart, so
 // that the outputs of a warp read different banks) and their biases
 __host__ __device__ inline size_t incumbent_doubles(const NetDesc &N, int ncta)
@@ -275,8 +283,10 @@ __global__ void __launch_bounds__(kIncThreads) k_incumbent_fp64(RolloutArgs a)
     __shared__ double f_sh;
     __shared__ int row_sh, ks_sh[kMaxLayers + 1];
     const int lane = threadIdx.x & 31;
-    if (threadIdx.x >= 1 && (int)threadIdx.x <= N.L)
-        ks_sh[threadIdx.x] = incumbent_lanes((N.dims[threadIdx.x] + ncta - 1) / ncta, N.dims[threadIdx.x - 1]);
+    if (threadIdx.x >= 1 && (int)threadIdx.x <= N.L) {
+        const int chunk = (N.dims[threadIdx.x] + ncta - 1) / ncta;
+        ks_sh[threadIdx.x] = WSMEM ? incumbent_lanes(chunk, N.dims[threadIdx.x - 1]) : incumbent_lanes_l2(chunk, N.dims[threadIdx.x - 1]);
+    }
     unsigned long long best = ~0ull;
 #pragma unroll 8
     for (int i = threadIdx.x; i < nlive; i += kIncThreads)
@@ -577,12 +587,17 @@ void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
 {
     if (a.n <= 0) return;
     // One CTA where a step is at most 4096 multiply-adds (2048 clocks of one SM's FP64 rate, about the layers' cluster
-    // barriers) or many problems are evaluated side by side and each is small; else a cluster of kIncCTAs, or of 8 where
-    // the GPU does not place 16.
+    // barriers); else a cluster of kIncCTAs, or of 8 where the GPU does not place 16.  Several problems run side by side,
+    // and their clusters share the SMs: a cluster each for up to 64 problems (32 with one step) of more than 512 P
+    // multiply-adds a step.
+    // Measured, cluster against one CTA, 20 steps: pushing network 2 problems 774 to 1279 us, 64 1038 to 1298, 128 1394
+    // to 1301; 160 and 128 wide, 32 problems 643 to 711, 64 795 to 711; two 64-wide layers, 8 problems 318 to 316, 16 332
+    // to 316; two 256-wide layers, 64 problems 2126 to 2515, 128 2585 to 2543.
     const NetDesc &N = a.net;
     long long macs = 0;
     for (int l = 1; l <= N.L; ++l) macs += (long long)N.dims[l] * N.dims[l - 1];
-    int ncta = macs > (a.batch.P > 1 ? 65536 : 4096) ? kIncCTAs : 1;
+    const bool several = a.batch.P > 1;
+    int ncta = macs > 4096 && (!several || (a.batch.P <= (a.H > 1 ? 64 : 32) && macs > 512LL * a.batch.P)) ? kIncCTAs : 1;
     // whether this GPU places a 16-CTA cluster (non-portable size) with the most shared memory the kernel takes:
     // decided at the first launch, which runs eagerly before any graph capture, and kept (one device per process)
     constexpr size_t kMaxSmem = 200 * 1024;
@@ -597,8 +612,10 @@ void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
         return ok && incumbent_placed<true>(kIncCTAs, kMaxSmem) && incumbent_placed<false>(kIncCTAs, 0);
     }();
     if (ncta > 8 && !big_ok) ncta = 8;
+    // One CTA: the weights of a single step (of several problems: of one or two) are not worth their copy (512 problems
+    // of two 64-wide layers: one step 88 us with, 77 without; five steps 238 and 239).
     const size_t smem = incumbent_doubles(N, ncta) * sizeof(double);
-    if (smem <= kMaxSmem) incumbent_run<true>(a, ncta, smem, st);
+    if (smem <= kMaxSmem && (ncta > 1 || a.H > (several ? 2 : 1))) incumbent_run<true>(a, ncta, smem, st);
     else incumbent_run<false>(a, ncta, 0, st);
 }
 
