@@ -993,10 +993,7 @@ int bab_rollout_cem(bab_ctx *c, const float *x0, const float *goal, int H, float
                                        : launch_rollout_tc(a, 3, c->tune_rollout_tc, c->num_sms, st);
         if (e == cudaSuccess) e = launch_cem_step(g, st);
     }
-    if (e == cudaSuccess && inc_val) {
-        launch_incumbent(a, st);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess && inc_val) e = launch_incumbent(a, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "cross-entropy search kernels");
     return BAB_OK;
 }
@@ -1109,8 +1106,7 @@ int bab_update_incumbent(bab_ctx *c, const float *x0, const float *goal, int H, 
     a.inc_val = inc_val;
     a.inc_u = inc_u;
     a.status = c->d_status;
-    launch_incumbent(a, (cudaStream_t)stream);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_incumbent(a, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "incumbent kernel");
     return BAB_OK;
 }

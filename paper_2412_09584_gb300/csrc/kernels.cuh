@@ -394,7 +394,7 @@ void launch_rollout_finalize(const RolloutArgs &a, cudaStream_t st);
 // search-integrated bounds around an FP32 rollout (a.emp_* set): key init before, float conversion after
 void launch_emp_init(const RolloutArgs &a, cudaStream_t st);
 void launch_emp_finish(const RolloutArgs &a, cudaStream_t st);
-void launch_incumbent(const RolloutArgs &a, cudaStream_t st);
+cudaError_t launch_incumbent(const RolloutArgs &a, cudaStream_t st);
 cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st);
 // interval bounds on tensor cores (split products with a computed margin; squared-distance cost, widths <= 256)
 cudaError_t launch_ibp_tc(const BoundArgs &a, int num_sms, cudaStream_t st);

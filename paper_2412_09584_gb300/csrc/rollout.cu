@@ -10,6 +10,8 @@
 // tile, adds the residual, and reduces the per-row cost with warp shuffles.
 // A tile's best (f, m) is folded into its box with a 64-bit atomicMin on
 // (order(f) << 32 | m), which keeps the lowest m among equal values.
+#include <atomic>
+
 #include <cooperative_groups.h>
 
 #include "bab_internal.cuh"
@@ -485,7 +487,7 @@ cudaError_t launch_rollout_fp32(const RolloutArgs &a, int variant, int num_sms, 
     if (e != cudaSuccess) return e;
     if (a.cem_mu) return cudaGetLastError();  // the cross-entropy search keeps its own best (launch_cem_step)
     launch_rollout_finalize(a, st);
-    if (a.inc_val) launch_incumbent(a, st);
+    if (a.inc_val && (e = launch_incumbent(a, st)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -545,47 +547,74 @@ void launch_rollout_finalize(const RolloutArgs &a, cudaStream_t st)
     if (a.n > 0) k_rollout_finalize<<<a.n, 128, 0, st>>>(a);
 }
 
+// The most shared memory the incumbent kernel takes.
+constexpr size_t kIncMaxSmem = 200 * 1024;
+
+// The kernel's attributes on the current device (the same for every launch, so that threads do not undo each other's) and
+// a launch of `blocks` CTAs in clusters of ncta.
+template <bool WSMEM>
+static cudaError_t incumbent_config(int ncta, int blocks, size_t smem, cudaStream_t st, cudaLaunchConfig_t &cfg,
+                                    cudaLaunchAttribute &attr)
+{
+    cudaError_t e = cudaSuccess;
+    if (WSMEM)
+        e = cudaFuncSetAttribute(k_incumbent_fp64<WSMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIncMaxSmem);
+    if (e == cudaSuccess && ncta > 8)
+        e = cudaFuncSetAttribute(k_incumbent_fp64<WSMEM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kIncThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)ncta;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return e;
+}
+
 template <bool WSMEM>
 static bool incumbent_placed(int ncta, size_t smem)
 {
-    cudaLaunchConfig_t q = {};
-    q.gridDim = dim3((unsigned)ncta);
-    q.blockDim = dim3(kIncThreads);
-    q.dynamicSmemBytes = smem;
-    cudaLaunchAttribute qa[1];
-    qa[0].id = cudaLaunchAttributeClusterDimension;
-    qa[0].val.clusterDim.x = (unsigned)ncta;
-    qa[0].val.clusterDim.y = 1;
-    qa[0].val.clusterDim.z = 1;
-    q.attrs = qa;
-    q.numAttrs = 1;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
     int nclusters = 0;
-    const bool ok = cudaOccupancyMaxActiveClusters(&nclusters, k_incumbent_fp64<WSMEM>, &q) == cudaSuccess && nclusters >= 1;
-    cudaGetLastError();
+    const bool ok = incumbent_config<WSMEM>(ncta, ncta, smem, nullptr, cfg, attr) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&nclusters, k_incumbent_fp64<WSMEM>, &cfg) == cudaSuccess && nclusters >= 1;
+    if (!ok) cudaGetLastError();
     return ok;
 }
 
 template <bool WSMEM>
-static void incumbent_run(const RolloutArgs &a, int ncta, size_t smem, cudaStream_t st)
+static cudaError_t incumbent_run(const RolloutArgs &a, int ncta, size_t smem, cudaStream_t st)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(ncta * (a.batch.P > 1 ? a.batch.P : 1)));
-    cfg.blockDim = dim3(kIncThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)ncta;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_incumbent_fp64<WSMEM>, a);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    const cudaError_t e = incumbent_config<WSMEM>(ncta, ncta * (a.batch.P > 1 ? a.batch.P : 1), smem, st, cfg, attr);
+    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, k_incumbent_fp64<WSMEM>, a);
 }
 
-void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
+// Whether the current device places a 16-CTA cluster (non-portable size) with the most shared memory the kernel takes:
+// asked at a device's first launch, which runs eagerly before any graph capture.
+static bool incumbent_wide()
 {
-    if (a.n <= 0) return;
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];  // 0: not asked, 1: no, 2: yes
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return false;
+    int k = known[dev].load();
+    if (k == 0) {
+        k = incumbent_placed<true>(kIncCTAs, kIncMaxSmem) && incumbent_placed<false>(kIncCTAs, 0) ? 2 : 1;
+        known[dev].store(k);
+    }
+    return k == 2;
+}
+
+cudaError_t launch_incumbent(const RolloutArgs &a, cudaStream_t st)
+{
+    if (a.n <= 0) return cudaSuccess;
     // One CTA where a step is at most 4096 multiply-adds (2048 clocks of one SM's FP64 rate, about the layers' cluster
     // barriers); else a cluster of kIncCTAs, or of 8 where the GPU does not place 16.  Several problems run side by side,
     // and their clusters share the SMs: a cluster each for up to 64 problems (32 with one step) of more than 512 P
@@ -598,25 +627,12 @@ void launch_incumbent(const RolloutArgs &a, cudaStream_t st)
     for (int l = 1; l <= N.L; ++l) macs += (long long)N.dims[l] * N.dims[l - 1];
     const bool several = a.batch.P > 1;
     int ncta = macs > 4096 && (!several || (a.batch.P <= (a.H > 1 ? 64 : 32) && macs > 512LL * a.batch.P)) ? kIncCTAs : 1;
-    // whether this GPU places a 16-CTA cluster (non-portable size) with the most shared memory the kernel takes:
-    // decided at the first launch, which runs eagerly before any graph capture, and kept (one device per process)
-    constexpr size_t kMaxSmem = 200 * 1024;
-    static const bool big_ok = [] {
-        bool ok = true;
-        for (int w = 0; w < 2; ++w) {
-            auto kern = w ? k_incumbent_fp64<true> : k_incumbent_fp64<false>;
-            ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-            if (w) ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) == cudaSuccess;
-        }
-        cudaGetLastError();
-        return ok && incumbent_placed<true>(kIncCTAs, kMaxSmem) && incumbent_placed<false>(kIncCTAs, 0);
-    }();
-    if (ncta > 8 && !big_ok) ncta = 8;
+    if (ncta > 8 && !incumbent_wide()) ncta = 8;
     // One CTA: the weights of a single step (of several problems: of one or two) are not worth their copy (512 problems
     // of two 64-wide layers: one step 88 us with, 77 without; five steps 238 and 239).
     const size_t smem = incumbent_doubles(N, ncta) * sizeof(double);
-    if (smem <= kMaxSmem && (ncta > 1 || a.H > (several ? 2 : 1))) incumbent_run<true>(a, ncta, smem, st);
-    else incumbent_run<false>(a, ncta, 0, st);
+    if (smem <= kIncMaxSmem && (ncta > 1 || a.H > (several ? 2 : 1))) return incumbent_run<true>(a, ncta, smem, st);
+    return incumbent_run<false>(a, ncta, 0, st);
 }
 
 }  // namespace bab

@@ -1409,9 +1409,11 @@ static cudaError_t launch_rescore(const RolloutArgs &a, cudaStream_t st)
         cudaError_t e = cudaFuncGetAttributes(&fa, kern);
         if (e != cudaSuccess) return e;
         size_t floats;
-        const uint32_t resident = rescore_cl_layers(N, ((size_t)budget - fa.sharedSizeBytes) / sizeof(float), floats);
+        const size_t room = (size_t)budget - fa.sharedSizeBytes;
+        const uint32_t resident = rescore_cl_layers(N, room / sizeof(float), floats);
         const size_t cl_smem = floats * sizeof(float);
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem);
+        // (the same for every network, so that threads with different ones do not undo each other's)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         const int nbox = a.topk > 15 * kRescoreBoxes ? kRescoreBoxes : (a.topk + 14) / 15;
@@ -1580,7 +1582,7 @@ cudaError_t launch_rollout_tc(RolloutArgs a, int split, int nslot_pref, int num_
         if (a.topk > 0) k_topk_select<<<1, 1024, 0, st>>>(a);
         e = launch_rescore(a, st);
         if (e != cudaSuccess) return e;
-        if (a.inc_val) launch_incumbent(a, st);
+        if (a.inc_val && (e = launch_incumbent(a, st)) != cudaSuccess) return e;
         return cudaGetLastError();
     }
     if (nslot_pref == 3 || nslot_pref == 4) nslot_pref -= 2;
@@ -1652,7 +1654,7 @@ cudaError_t launch_rollout_tc(RolloutArgs a, int split, int nslot_pref, int num_
         e = launch_rescore(a, st);
         if (e != cudaSuccess) return e;
     }
-    if (a.inc_val) launch_incumbent(a, st);
+    if (a.inc_val && (e = launch_incumbent(a, st)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
