@@ -143,7 +143,9 @@ __device__ __forceinline__ void plan_totals(const BranchArgs &a, int picked, int
 }
 
 // At most kSmallPlan rows, one per thread: a row is among the k smallest composite keys when fewer than k candidates
-// have a smaller one, so each selection is one count over the rows (48 rows: 28 us by radix passes -> 5 us).
+// have a smaller one, so each selection is one count over the rows, without a branch (the others carry the largest key).
+// 48 rows: 28 us by radix passes -> 5 us; the whole call at 256 rows: 29 to 37 us by radix passes, 39 to 46 with a branch
+// a row, 17 without (the host's launches).
 constexpr int kSmallPlan = 256;
 
 __global__ void __launch_bounds__(kSmallPlan) k_branch_plan_small(BranchArgs a)
@@ -167,18 +169,17 @@ __global__ void __launch_bounds__(kSmallPlan) k_branch_plan_small(BranchArgs a)
     if (ns > n_pick) {
         // among the rows flagged `in`, whether this one is one of the k smallest by (order(v), id)
         auto smallest = [&](bool in, float v, int k) {
-            key[i] = float_order(v);
-            ids[i] = in ? id : 0;
-            const unsigned in_warp = __ballot_sync(0xFFFFFFFFu, in);
-            if (lane == 0) wsum[0][warp] = (int)in_warp;
+            const uint32_t mk = float_order(v);
+            key[i] = in ? mk : 0xFFFFFFFFu;
+            ids[i] = in ? id : ~0ull;
             __syncthreads();
             int less = 0;
-            const uint32_t mk = key[i];
-            if (in && k > 0)
-                for (int j = 0; j < n; ++j)
-                    less += ((wsum[0][j >> 5] >> (j & 31)) & 1) && (key[j] < mk || (key[j] == mk && ids[j] < id));
+            if (k > 0) {
+#pragma unroll 8
+                for (int j = 0; j < n; ++j) less += (key[j] < mk) | ((key[j] == mk) & (ids[j] < id));
+            }
             __syncthreads();
-            return in && k > 0 && less < k;
+            return in && less < k;
         };
         const bool by_ub = smallest(kp, ub, n1);
         const bool cand = kp && !by_ub;
@@ -260,6 +261,12 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
     const double inc = a.inc_val[0];
     int n_pick, n1;
     plan_quota(a, 0, n_pick, n1);
+    // (a lone CTA needs neither the cluster's barriers nor its view of the shared memory: ties among 600 rows 43 -> 36 us)
+    auto sync = [&]() {
+        if (C > 1) cluster.sync();
+        else __syncthreads();
+    };
+    auto of = [&](auto *p, int q) { return C > 1 ? cluster.map_shared_rank(p, q) : p; };
     // the sum of a value over the block's threads (every thread gets it)
     auto block_sum = [&](int v) {
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
@@ -336,9 +343,9 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
     };
     cnt = block_sum(cnt);
     if (tid == 0) sh.part[0][0] = cnt;
-    cluster.sync();
+    sync();
     int ns = 0;
-    for (int q = 0; q < C; ++q) ns += *cluster.map_shared_rank(&sh.part[0][0], q);
+    for (int q = 0; q < C; ++q) ns += *of(&sh.part[0][0], q);
 
     const bool all = ns <= n_pick;
     Thresh T1, T2;
@@ -371,12 +378,12 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
                     atomicAdd(&hist[dg], 1u);
                 }
             });
-            cluster.sync();  // every CTA's histogram complete
+            sync();  // every CTA's histogram complete
             unsigned h = 0, inclusive = 0;
             if (tid < 256) {
 #pragma unroll
                 for (int q = 0; q < kPlanCTAs; ++q)
-                    if (q < C) h += cluster.map_shared_rank(hist, q)[tid];
+                    if (q < C) h += of(hist, q)[tid];
                 inclusive = h;
                 for (int o = 1; o < 32; o *= 2) {
                     const unsigned v = __shfl_up_sync(0xFFFFFFFFu, inclusive, o);
@@ -445,12 +452,12 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
                 sh.mn = mn;
                 sh.mx = mx;
             }
-            cluster.sync();
+            sync();
             mn = INFINITY;
             mx = -INFINITY;
             for (int q = 0; q < C; ++q) {
-                mn = fminf(mn, *cluster.map_shared_rank(&sh.mn, q));
-                mx = fmaxf(mx, *cluster.map_shared_rank(&sh.mx, q));
+                mn = fminf(mn, *of(&sh.mn, q));
+                mx = fmaxf(mx, *of(&sh.mx, q));
             }
             each([&](int i, int it, const Row &r) {
                 if (!cand(r)) return;
@@ -479,10 +486,10 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         sh.part[1][0] = cp;
         sh.part[1][1] = cr;
     }
-    cluster.sync();
+    sync();
     int base_p = 0, base_r = 0, tp = 0, tr = 0;
     for (int q = 0; q < C; ++q) {
-        const int *o = cluster.map_shared_rank(&sh.part[1][0], q);
+        const int *o = of(&sh.part[1][0], q);
         if (q < rank) {
             base_p += o[0];
             base_r += o[1];
@@ -516,7 +523,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_branch_plan_cl(BranchArgs a)
         __syncthreads();
     });
     if (rank == 0 && tid == 0) plan_totals(a, tp, tr);
-    cluster.sync();  // no CTA leaves while another may still read its shared memory
+    sync();  // no CTA leaves while another may still read its shared memory
 }
 
 // Several problems: output offsets of each problem's children and unpicked rows, and the totals.
