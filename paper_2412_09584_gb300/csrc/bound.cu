@@ -755,6 +755,19 @@ __host__ __device__ inline size_t fwd_rows_floats(const NetDesc &N, int rb)
     return 2 * (size_t)rb * N.maxw_p + (size_t)rb * pad4(N.s);
 }
 
+// A layer's product over RBT rows by NTT threads: dense_rows_auto's tiles, but 4 x 4 outputs a thread where 4 x 8 would
+// leave half of the threads idle (coefficients of 9728 boxes, H = 5: two 256-wide layers 947 -> 651 us, four of them, the
+// image read through L2, 2348 -> 1470).
+template <int RBT, int NTT>
+__device__ __forceinline__ void rows_product(const float *in, int ldi, const float *B, const float *bias, int Kp, int Np,
+                                             float *out, int ldo, int tid)
+{
+    if (RBT == 8 && NTT == 128 && Np > 128)
+        dense_rows<RBT, NTT, (RBT == 8 ? 4 : 1), 4>(in, ldi, B, bias, Kp, Np, out, ldo, false, tid);
+    else
+        dense_rows_auto<RBT, NTT>(in, ldi, B, bias, Kp, Np, out, ldo, false, tid);
+}
+
 // Theorem 1 backward propagation of the tangent-linearised cost through all H
 // steps, then Theorem 2 in box form, for rows 0 .. nrows-1 of the view (rows
 // nrows .. RBT-1 are padding), by NTT consecutive threads of the CTA (group grp
@@ -864,8 +877,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 ml[ri] = __fmaf_ru(N.gam[L], e, ml[ri]);
             }
             group_barrier(grp, NTT);
-            dense_rows_auto<RBT, NTT>(Ab[0], ld, img + N.bwd_w[L], nullptr, NpL, pad4(N.dims[L - 1]), Ab[1], ld, false,
-                                      tid);
+            rows_product<RBT, NTT>(Ab[0], ld, img + N.bwd_w[L], nullptr, NpL, pad4(N.dims[L - 1]), Ab[1], ld, tid);
             group_barrier(grp, NTT);
         }
         int cur = 1;
@@ -916,8 +928,7 @@ __device__ void crown_rows(const BoundArgs &a, const float *img, float *p, const
                 ml[ri] = __fadd_ru(ml[ri], __fmaf_ru(N.gam[l], eg, __fmul_ru(kTwoU, er)));
             }
             group_barrier(grp, NTT);
-            dense_rows_auto<RBT, NTT>(Ab[cur], ld, img + N.bwd_w[l], nullptr, Npl, pad4(N.dims[l - 1]), Ab[cur ^ 1], ld,
-                                      false, tid);
+            rows_product<RBT, NTT>(Ab[cur], ld, img + N.bwd_w[l], nullptr, Npl, pad4(N.dims[l - 1]), Ab[cur ^ 1], ld, tid);
             group_barrier(grp, NTT);
             cur ^= 1;
         }
@@ -1077,8 +1088,8 @@ __device__ void fwd_rows(const BoundArgs &a, const float *img, float *p, const R
         group_barrier(grp, NTT);
         int cur = 0;
         for (int l = 1; l <= L; ++l) {
-            dense_rows_auto<RBT, NTT>(Z[cur], ld, img + N.fwd_w[l], img + N.fwd_b[l], pad4(N.dims[l - 1]),
-                                      pad4(N.dims[l]), Z[cur ^ 1], ld, false, tid);
+            rows_product<RBT, NTT>(Z[cur], ld, img + N.fwd_w[l], img + N.fwd_b[l], pad4(N.dims[l - 1]), pad4(N.dims[l]),
+                                   Z[cur ^ 1], ld, tid);
             group_barrier(grp, NTT);
             cur ^= 1;
             if (l < L) {
@@ -1412,8 +1423,39 @@ cudaError_t launch_ibp(const BoundArgs &a, int num_sms, cudaStream_t st)
     return cudaGetLastError();
 }
 
+// The same call for the boxes from `row` on.
+static BoundArgs from_row(BoundArgs a, int row)
+{
+    const size_t r = (size_t)row, hs = r * a.H * a.net.sumh, xs = r * (a.H + 1) * a.net.s;
+    auto move = [](auto *&p, size_t by) {
+        if (p) p += by;
+    };
+    a.row0 += row;
+    a.n -= row;
+    move(a.lo, r * a.d);
+    move(a.hi, r * a.d);
+    move(a.pre_lo, hs);
+    move(a.pre_hi, hs);
+    move(a.x_lo, xs);
+    move(a.x_hi, xs);
+    move(a.S, r * a.H * (a.net.sumh + a.net.s));
+    move(a.lb_ibp, r);
+    move(a.alpha, hs);
+    move(a.lb, r);
+    move(a.margin, r);
+    move(a.lin_const, r);
+    move(a.lb_best, r);
+    move(a.lin_coef, r * a.d);
+    move(a.ustar, r * a.d);
+    move(a.A_pre, hs);
+    move(a.grad_alpha, hs);
+    return a;
+}
+
 // Rows per group of k_rows: the smallest of 1, 2, 4, 8 with which one wave of CTAs holds all boxes (a step takes a group
-// about the same time with one row as with two), at most what fits in shared memory; 8 beyond one wave.
+// about the same time with one row as with two), at most what fits in shared memory; beyond one wave, whole waves of the
+// most rows and then one wave of what is left (16384 boxes of four 256-wide layers, H = 5, the gradient call 10.6 -> 10.2
+// ms; two 32-wide layers, H = 40, the coefficients 1553 -> 1439 us).
 template <bool FWD>
 static cudaError_t launch_rows(const BoundArgs &a, int num_sms, cudaStream_t st)
 {
@@ -1424,26 +1466,43 @@ static cudaError_t launch_rows(const BoundArgs &a, int num_sms, cudaStream_t st)
     auto group = [&](int rb) { return ((floats(rb) + 3) & ~size_t(3)) * 4; };
     if (floats(RB) * 4 > budget) return cudaErrorInvalidConfiguration;  // (the working set of a tile of RB boxes)
     if (num_sms <= 0) num_sms = sm_count();
-    int rb = 1;
-    while (rb < 8 && (long long)num_sms * kRowGroups * rb < a.n) rb *= 2;
     // (fewer rows rather than the image out of shared memory)
     const size_t beside = img + kRowGroups * group(1) <= budget ? img : 0;
-    while (rb > 1 && beside + kRowGroups * group(rb) > budget) rb /= 2;
-    const bool wsmem = img + kRowGroups * group(rb) <= budget;
-    const size_t smem = (wsmem ? img : 0) + kRowGroups * group(rb);
-    auto run = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const int per = kRowGroups * rb;
-        kern<<<(a.n + per - 1) / per, NT, smem, st>>>(a, (int)(group(rb) / 4));
-        return cudaGetLastError();
+    int most = 8;
+    while (most > 1 && beside + kRowGroups * group(most) > budget) most /= 2;
+    auto run = [&](int rb, const BoundArgs &b, int boxes) {
+        const bool wsmem = img + kRowGroups * group(rb) <= budget;
+        const size_t smem = (wsmem ? img : 0) + kRowGroups * group(rb);
+        auto go = [&](auto kern) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            const int per = kRowGroups * rb;
+            kern<<<(boxes + per - 1) / per, NT, smem, st>>>(b, (int)(group(rb) / 4));
+            return cudaGetLastError();
+        };
+        switch (rb) {
+            case 1: return wsmem ? go(k_rows<1, true, FWD>) : go(k_rows<1, false, FWD>);
+            case 2: return wsmem ? go(k_rows<2, true, FWD>) : go(k_rows<2, false, FWD>);
+            case 4: return wsmem ? go(k_rows<4, true, FWD>) : go(k_rows<4, false, FWD>);
+            default: return wsmem ? go(k_rows<8, true, FWD>) : go(k_rows<8, false, FWD>);
+        }
     };
-    switch (rb) {
-        case 1: return wsmem ? run(k_rows<1, true, FWD>) : run(k_rows<1, false, FWD>);
-        case 2: return wsmem ? run(k_rows<2, true, FWD>) : run(k_rows<2, false, FWD>);
-        case 4: return wsmem ? run(k_rows<4, true, FWD>) : run(k_rows<4, false, FWD>);
-        default: return wsmem ? run(k_rows<8, true, FWD>) : run(k_rows<8, false, FWD>);
+    auto fit = [&](int boxes) {
+        int rb = 1;
+        while (rb < most && (long long)num_sms * kRowGroups * rb < boxes) rb *= 2;
+        return rb;
+    };
+    const int wave = num_sms * kRowGroups * most, left = a.n % wave;
+    int full = a.n - left;
+    // (one launch where the rest would take the most rows all the same)
+    if (fit(left) == most) full = a.n;
+    if (full > 0) {
+        BoundArgs b = a;
+        b.n = full;
+        const cudaError_t e = run(most, b, full);
+        if (e != cudaSuccess || full == a.n) return e;
     }
+    return run(fit(left), full > 0 ? from_row(a, full) : a, left);
 }
 
 cudaError_t launch_crown(const BoundArgs &a, int num_sms, cudaStream_t st) { return launch_rows<false>(a, num_sms, st); }
