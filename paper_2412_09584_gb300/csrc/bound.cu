@@ -50,10 +50,6 @@ __device__ __forceinline__ unsigned long long ffma2_ru(unsigned long long a, uns
     asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
-__device__ __forceinline__ unsigned long long pack2f(float x, float y)
-{
-    return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
-}
 __device__ __forceinline__ float half2f(unsigned long long v, int e)
 {
     return __uint_as_float((uint32_t)(e ? v >> 32 : v));
@@ -181,14 +177,14 @@ __device__ __forceinline__ void ibp_input(const float *__restrict__ wr, const fl
     unsigned long long wp[TP], wn[TP], wa[TP];
 #pragma unroll
     for (int j = 0; j < TP; ++j) {
-        wp[j] = pack2f(fmaxf(w[2 * j], 0.f), fmaxf(w[2 * j + 1], 0.f));
-        wn[j] = pack2f(fminf(w[2 * j], 0.f), fminf(w[2 * j + 1], 0.f));
-        wa[j] = pack2f(fabsf(w[2 * j]), fabsf(w[2 * j + 1]));
+        wp[j] = pack_f32x2(fmaxf(w[2 * j], 0.f), fmaxf(w[2 * j + 1], 0.f));
+        wn[j] = pack_f32x2(fminf(w[2 * j], 0.f), fminf(w[2 * j + 1], 0.f));
+        wa[j] = pack_f32x2(fabsf(w[2 * j]), fabsf(w[2 * j + 1]));
     }
 #pragma unroll
     for (int i = 0; i < TR; ++i) {
         const float ah = kk == 0 ? h4[i].x : kk == 1 ? h4[i].y : kk == 2 ? h4[i].z : h4[i].w;
-        const unsigned long long ah2 = pack2f(ah, ah);
+        const unsigned long long ah2 = pack_f32x2(ah, ah);
         if (!LOWER) {
 #pragma unroll
             for (int j = 0; j < TP; ++j) {
@@ -198,7 +194,7 @@ __device__ __forceinline__ void ibp_input(const float *__restrict__ wr, const fl
         } else {
             const float al = kk == 0 ? l4[i].x : kk == 1 ? l4[i].y : kk == 2 ? l4[i].z : l4[i].w;
             const float am = FIRST ? fmaxf(fabsf(al), fabsf(ah)) : al;
-            const unsigned long long al2 = pack2f(al, al), am2 = pack2f(am, am);
+            const unsigned long long al2 = pack_f32x2(al, al), am2 = pack_f32x2(am, am);
 #pragma unroll
             for (int j = 0; j < TP; ++j) {
                 l2[i][j] = ffma2_rd(wn[j], ah2, ffma2_rd(wp[j], al2, l2[i][j]));
@@ -294,7 +290,7 @@ __device__ __forceinline__ bool ibp_dense(int tid, const float *__restrict__ alo
         for (int j = 0; j < TP; ++j)
 #pragma unroll
             for (int i = 0; i < TR; ++i) {
-                l2[i][j] = h2[i][j] = pack2f(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]);
+                l2[i][j] = h2[i][j] = pack_f32x2(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]);
                 v2[i][j] = 0ull;
             }
         for (int k = 0; k < Kp; k += 128) {
@@ -401,7 +397,7 @@ __device__ __forceinline__ bool ibp_dense_stream(const float *__restrict__ alo, 
     unsigned long long l2[TR][TP], h2[TR][TP], v2[TR][TP];
 #pragma unroll
     for (int j = 0; j < TP; ++j) {
-        const unsigned long long b2 = mine ? pack2f(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]) : 0ull;
+        const unsigned long long b2 = mine ? pack_f32x2(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]) : 0ull;
 #pragma unroll
         for (int i = 0; i < TR; ++i) {
             l2[i][j] = h2[i][j] = b2;

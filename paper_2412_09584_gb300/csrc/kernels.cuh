@@ -314,10 +314,6 @@ __device__ __forceinline__ void dense_rows(const float *__restrict__ in, int ldi
                         w[(j + 2) % (2 * TP)] = q.z;
                         w[(j + 3) % (2 * TP)] = q.w;
                     }
-                } else if (TN == 2) {
-                    const float2 q = *reinterpret_cast<const float2 *>(wr);
-                    w[0] = q.x;
-                    w[1] = q.y;
                 } else {
 #pragma unroll
                     for (int j = 0; j < 2 * TP; ++j) w[j] = (j < TN && c0 + j < Np) ? wr[j] : 0.f;

@@ -29,21 +29,10 @@ constexpr int kRows = 64;            // samples per tile
 constexpr int kThreads = 256;        // per CTA: groups x warps x 32
 constexpr int kSpan = 32, kStages = 2;  // inputs per span of the ring
 
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long pack2(float x, float y)
-{
-    return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
-}
 __device__ __forceinline__ float2 unpack2(unsigned long long v)
 {
     return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
 }
-__device__ __forceinline__ void group_sync(int g, int nt) { asm volatile("barrier.cta.sync %0, %1;" ::"r"(g + 1), "r"(nt) : "memory"); }
 __device__ __forceinline__ float lane4(const float4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 
 // Leading dimension of the activation rows: 4 mod 8 floats (16-byte loads of neighbouring rows on distinct banks).
@@ -72,19 +61,19 @@ __device__ __forceinline__ void product(const float *__restrict__ x, int ld, con
             const float *wr = w + (size_t)(k - k0 + kk) * Np;
             unsigned long long wv[TN / 2];
             const float4 a = *reinterpret_cast<const float4 *>(wr);
-            wv[0] = pack2(a.x, a.y);
-            wv[1] = pack2(a.z, a.w);
+            wv[0] = pack_f32x2(a.x, a.y);
+            wv[1] = pack_f32x2(a.z, a.w);
             if (TN == 8) {
                 const float4 b = hi ? *reinterpret_cast<const float4 *>(wr + 32) : make_float4(0.f, 0.f, 0.f, 0.f);
-                wv[2 % (TN / 2)] = pack2(b.x, b.y);
-                wv[3 % (TN / 2)] = pack2(b.z, b.w);
+                wv[2 % (TN / 2)] = pack_f32x2(b.x, b.y);
+                wv[3 % (TN / 2)] = pack_f32x2(b.z, b.w);
             }
 #pragma unroll
             for (int i = 0; i < TR; ++i) {
                 const float xs = lane4(xv[i], kk);
-                const unsigned long long x2 = pack2(xs, xs);
+                const unsigned long long x2 = pack_f32x2(xs, xs);
 #pragma unroll
-                for (int j = 0; j < TN / 2; ++j) acc[i][j] = ffma2(x2, wv[j], acc[i][j]);
+                for (int j = 0; j < TN / 2; ++j) acc[i][j] = ffma2_rn(x2, wv[j], acc[i][j]);
             }
         }
     }
@@ -114,11 +103,11 @@ __device__ __forceinline__ void layer(const LayerArgs &a, int grp, int tid, int 
         const float4 b1 = hi ? *reinterpret_cast<const float4 *>(a.bias + c0 + 32) : z;
 #pragma unroll
         for (int i = 0; i < TR; ++i) {
-            acc[i][0] = pack2(b0.x, b0.y);
-            acc[i][1] = pack2(b0.z, b0.w);
+            acc[i][0] = pack_f32x2(b0.x, b0.y);
+            acc[i][1] = pack_f32x2(b0.z, b0.w);
             if (TN == 8) {
-                acc[i][2 % (TN / 2)] = pack2(b1.x, b1.y);
-                acc[i][3 % (TN / 2)] = pack2(b1.z, b1.w);
+                acc[i][2 % (TN / 2)] = pack_f32x2(b1.x, b1.y);
+                acc[i][3 % (TN / 2)] = pack_f32x2(b1.z, b1.w);
             }
         }
     }
@@ -142,16 +131,16 @@ __device__ __forceinline__ void layer(const LayerArgs &a, int grp, int tid, int 
         for (int q = 0; q < nspan; ++q) {
             fetch(q + 1);  // its stage was last read before the barrier that closed the span before
             asm volatile("cp.async.wait_group 1;" ::: "memory");
-            group_sync(grp, nt);
+            group_barrier(grp, nt);
             const int k0 = q * kSpan;
             if (mine)
                 product<TR, TN>(x, ld, a.ring + (size_t)(q % kStages) * kSpan * kMaxWidth + c0, Np, k0,
                                 min(Kp, k0 + kSpan), hi, acc);
-            group_sync(grp, nt);
+            group_barrier(grp, nt);
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    if (!STREAM) group_sync(grp, nt);  // every input read
+    if (!STREAM) group_barrier(grp, nt);  // every input read
     if (mine) {
         float *o = a.act + (size_t)r0 * ld + c0;
 #pragma unroll
@@ -169,7 +158,7 @@ __device__ __forceinline__ void layer(const LayerArgs &a, int grp, int tid, int 
                 *reinterpret_cast<float4 *>(o + (size_t)4 * i * ld + 32 * h) = make_float4(p.x, p.y, q.x, q.y);
             }
     }
-    group_sync(grp, nt);
+    group_barrier(grp, nt);
 }
 
 // A layer of at most nt / 16 outputs (the network's last): one row and four columns per thread.
@@ -180,8 +169,8 @@ __device__ __forceinline__ void layer_narrow(const LayerArgs &a, int grp, int ti
     unsigned long long acc[2] = {0ull, 0ull};
     if (mine) {
         const float4 b = *reinterpret_cast<const float4 *>(a.bias + c0);
-        acc[0] = pack2(b.x, b.y);
-        acc[1] = pack2(b.z, b.w);
+        acc[0] = pack_f32x2(b.x, b.y);
+        acc[1] = pack_f32x2(b.z, b.w);
         const float *x = a.act + (size_t)r * a.ld;
 #pragma unroll 4
         for (int k = 0; k < a.Kp; k += 4) {
@@ -190,13 +179,13 @@ __device__ __forceinline__ void layer_narrow(const LayerArgs &a, int grp, int ti
             for (int kk = 0; kk < 4; ++kk) {
                 const float4 w = *reinterpret_cast<const float4 *>(a.W + (size_t)(k + kk) * Np + c0);
                 const float xs = lane4(xv, kk);
-                const unsigned long long x2 = pack2(xs, xs);
-                acc[0] = ffma2(x2, pack2(w.x, w.y), acc[0]);
-                acc[1] = ffma2(x2, pack2(w.z, w.w), acc[1]);
+                const unsigned long long x2 = pack_f32x2(xs, xs);
+                acc[0] = ffma2_rn(x2, pack_f32x2(w.x, w.y), acc[0]);
+                acc[1] = ffma2_rn(x2, pack_f32x2(w.z, w.w), acc[1]);
             }
         }
     }
-    group_sync(grp, nt);
+    group_barrier(grp, nt);
     if (mine) {
         float2 p = unpack2(acc[0]), q = unpack2(acc[1]);
         if (a.relu) {
@@ -207,7 +196,7 @@ __device__ __forceinline__ void layer_narrow(const LayerArgs &a, int grp, int ti
         }
         *reinterpret_cast<float4 *>(a.act + (size_t)r * a.ld + c0) = make_float4(p.x, p.y, q.x, q.y);
     }
-    group_sync(grp, nt);
+    group_barrier(grp, nt);
 }
 
 }  // namespace
@@ -244,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rollout_rows(RolloutArgs a)
     const float rho = a.rho;
     for (long long tile = blockIdx.x + (long long)gridDim.x * grp; tile < ntiles; tile += (long long)gridDim.x * G) {
         const long long g0 = tile * kRows;
-        group_sync(grp, TG);  // the last tile's rows are done with
+        group_barrier(grp, TG);  // the last tile's rows are done with
         for (int r = tid; r < kRows; r += TG) {
             const long long g = g0 + r;
             const int box = (int)((g < total ? g : total - 1) / M);  // (rows past the end repeat the last box)
@@ -255,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rollout_rows(RolloutArgs a)
             ps[2 * r + 1] = a.cost.p0y;
         }
         for (int i = tid; i < kRows * s; i += TG) xs[i] = a.x0[i / kRows];
-        group_sync(grp, TG);
+        group_barrier(grp, TG);
         for (int t = 0; t <= H; ++t) {
             // the first threads: state and cost of step t from the network's output, and the state part of the next
             // input row; the others: the actions u_t
@@ -311,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rollout_rows(RolloutArgs a)
                 }
             }
             if (t == H) break;
-            group_sync(grp, TG);
+            group_barrier(grp, TG);
             for (int l = 1; l <= L; ++l) {
                 LayerArgs la;
                 la.act = act;
