@@ -576,9 +576,34 @@ def run_ours(args):
            "fp32_peak_measured": fp32_peak_measured()}
     if not args.no_cpu_baseline and ws == 1:
         out["cpu_baseline"] = cpu_baseline(budget_s=args.cpu_budget)
-    print(json.dumps(out), flush=True)
+    line, details = split_line(out)
+    print(json.dumps(details), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
     if ws > 1:
         dist.destroy_process_group()
+
+
+SIDE_SECTIONS = ("time_to_gap", "time_to_gap_pushing", "batched", "manip_scale", "paper_bounding", "heuristics",
+                 "cem_search", "synthetic_objective", "obstacle_cost", "tiny_latency", "precision_lines")
+
+
+def split_line(out):
+    """(the JSON line, the side sections in full): the sections beside the headline are tens of kilobytes of curves and
+    per-variant times, more than a reader of one line takes; the line keeps each variant's time."""
+    times = ("ms_per_step", "ms_per_iteration", "us_per_iteration_graph", "bound_bf16x3_ms", "rollout_bf16_ms", "ibp_ms")
+
+    def brief(v):
+        if not isinstance(v, dict):
+            return None
+        found = {k: float("%.4g" % v[k]) for k in times if isinstance(v.get(k), (int, float))}
+        if len(found) == 1 and not any(isinstance(x, dict) and brief(x) for x in v.values()):
+            return next(iter(found.values()))
+        found.update({k: brief(x) for k, x in v.items() if isinstance(x, dict) and brief(x)})
+        return found or None
+
+    line = {k: v for k, v in out.items() if k not in SIDE_SECTIONS}
+    line["side_ms"] = {k: brief(out[k]) for k in SIDE_SECTIONS if brief(out.get(k))}
+    return line, {k: out[k] for k in SIDE_SECTIONS if k in out}
 
 
 def precision_lines(dev, seed, n_pick, headline, bound_precision, interval_precision="fp32", steps=3):
