@@ -1326,7 +1326,8 @@ static int ibp_tile(int rb, int Np, int &tile)
 }
 
 // Boxes per group of k_ibp over n boxes: the count up to `most` whose waves of tiles take the least time (per layer
-// its inputs' cycles plus about 700 for the barrier, the stores and the step's share of the rest).
+// its inputs' cycles plus about 700 for the barrier, the stores and the step's share of the rest, as measured on 128-wide
+// layers; networks of layers up to 64 wide go to k_ibp_warp).
 static int ibp_rows(const NetDesc &N, int n, int num_sms, int most, int &tiles)
 {
     int best = most;

@@ -185,7 +185,11 @@ extern "C" int bab_bound_crown_static(int n_layers, const int *dims, const float
     a.hi = hi;
     a.n = n;
     a.d_n = nullptr;
-    a.unchecked = 1;  // the caller's device parameters have not been seen
+    // The caller's device parameters have not been seen: layers wider than 64 take the loop of one output a thread, which
+    // minds products of 0 and infinity.  (Flags written while packing, read by the interval kernel, let a finite network
+    // take its tiles: 128-wide layers 1 box 76 -> 97 us, 16 to 300 boxes 6% more, 256-wide ones 20% less; the kernel
+    // itself 1 to 3% more in every call.)
+    a.unchecked = 1;
     a.H = horizon;
     a.batch.Hmax = horizon;
     a.d = N.k * horizon;
