@@ -628,10 +628,12 @@ cudaError_t launch_incumbent(const RolloutArgs &a, cudaStream_t st)
     const bool several = a.batch.P > 1;
     int ncta = macs > 4096 && (!several || (a.batch.P <= (a.H > 1 ? 64 : 32) && macs > 512LL * a.batch.P)) ? kIncCTAs : 1;
     if (ncta > 8 && !incumbent_wide()) ncta = 8;
-    // One CTA: the weights of a single step (of several problems: of one or two) are not worth their copy (512 problems
-    // of two 64-wide layers: one step 88 us with, 77 without; five steps 238 and 239).
+    // Few steps are not worth the copy of the weights: of one CTA a single step, of several problems' CTAs one or two (512
+    // problems of two 64-wide layers: one step 88 us with, 77 without; five steps 238 and 239), of several problems'
+    // clusters a single one (8 such problems: 45.4 and 43.3 us; two steps 59.7 both).
+    const int few = ncta == 1 ? (several ? 2 : 1) : (several ? 1 : 0);
     const size_t smem = incumbent_doubles(N, ncta) * sizeof(double);
-    if (smem <= kIncMaxSmem && (ncta > 1 || a.H > (several ? 2 : 1))) return incumbent_run<true>(a, ncta, smem, st);
+    if (smem <= kIncMaxSmem && a.H > few) return incumbent_run<true>(a, ncta, smem, st);
     return incumbent_run<false>(a, ncta, 0, st);
 }
 
